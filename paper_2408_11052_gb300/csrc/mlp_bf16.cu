@@ -514,7 +514,7 @@ void launch_gemm_cfg(const tc::GemmProblem* table, int nprob, int tiles, unsigne
     cudaFuncSetAttribute(tc::tc_gemm_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
     attr = true;
   }
-  launch_k(tc::tc_gemm_kernel<BN, STAGES>, dim3(tiles), dim3(128), S::kBytes, st, table, nprob, status);
+  launch_k(tc::tc_gemm_kernel<BN, STAGES>, dim3(tiles), dim3(tc::kTileThreads), S::kBytes, st, table, nprob, status);
 }
 
 int sm_count() {
@@ -534,12 +534,12 @@ void launch_gemm_persistent(const tc::GemmProblem* table, int nprob, int tiles, 
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(tc::tc_gemm_persistent_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         S::kBytes);
+                         S::kPersistentBytes);
     attr = true;
   }
   const int grid = std::min(tiles, sm_count());
-  launch_k(tc::tc_gemm_persistent_kernel<BN, STAGES>, dim3(grid), dim3(192), S::kBytes, st, table, nprob, tiles,
-           status);
+  launch_k(tc::tc_gemm_persistent_kernel<BN, STAGES>, dim3(grid), dim3(tc::kPersistentThreads), S::kPersistentBytes, st,
+           table, nprob, tiles, status);
 }
 
 // CTA-pair kernel: clusters of two CTAs, one cluster per pair of SMs at most
@@ -547,7 +547,7 @@ void launch_gemm_persistent(const tc::GemmProblem* table, int nprob, int tiles, 
 int pair_clusters_max(const void* kernel, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * 64);
-  cfg.blockDim = dim3(224);
+  cfg.blockDim = dim3(tc::kPairThreads);
   cfg.dynamicSmemBytes = smem;
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) {
@@ -566,7 +566,8 @@ void launch_gemm_pair(const tc::GemmProblem* table, int nprob, int tiles, unsign
     clusters = pair_clusters_max(reinterpret_cast<const void*>(tc::tc_gemm_pair_kernel<BN, STAGES>), S::kBytes);
   }
   const int grid = 2 * std::min(tiles, clusters);
-  launch_k(tc::tc_gemm_pair_kernel<BN, STAGES>, dim3(grid), dim3(224), S::kBytes, st, table, nprob, tiles, status);
+  launch_k(tc::tc_gemm_pair_kernel<BN, STAGES>, dim3(grid), dim3(tc::kPairThreads), S::kBytes, st, table, nprob, tiles,
+           status);
 }
 
 // A GEMM configuration: tile width, ring depth and kernel (0: one tile per CTA,
@@ -584,12 +585,12 @@ bool cfg_allowed(int cfg) {
 }
 constexpr int kGemmCfgs[10] = {gemm_cfg(64, 4),     gemm_cfg(64, 8),     gemm_cfg(128, 3),    gemm_cfg(128, 6),
                                gemm_cfg(256, 4),    gemm_cfg(64, 8, 1),  gemm_cfg(128, 6, 1), gemm_cfg(256, 4, 1),
-                               gemm_cfg(128, 8, 2), gemm_cfg(256, 6, 2)};
+                               gemm_cfg(128, 7, 2), gemm_cfg(256, 5, 2)};
 
 void launch_cfg(int cfg, const tc::GemmProblem* t, int nprob, int tiles, unsigned* status, cudaStream_t st) {
   switch (cfg) {
-    case gemm_cfg(128, 8, 2): launch_gemm_pair<128, 8>(t, nprob, tiles, status, st); break;
-    case gemm_cfg(256, 6, 2): launch_gemm_pair<256, 6>(t, nprob, tiles, status, st); break;
+    case gemm_cfg(128, 7, 2): launch_gemm_pair<128, 7>(t, nprob, tiles, status, st); break;
+    case gemm_cfg(256, 5, 2): launch_gemm_pair<256, 5>(t, nprob, tiles, status, st); break;
     case gemm_cfg(64, 8, 1): launch_gemm_persistent<64, 8>(t, nprob, tiles, status, st); break;
     case gemm_cfg(128, 6, 1): launch_gemm_persistent<128, 6>(t, nprob, tiles, status, st); break;
     case gemm_cfg(256, 4, 1): launch_gemm_persistent<256, 4>(t, nprob, tiles, status, st); break;
@@ -614,7 +615,7 @@ int heuristic_cfg(const std::vector<tc::GemmProblem>& probs, int min_bn) {
     // pair tiles want width: 256 columns wherever every problem has them
     int nmin = 1 << 30;
     for (const auto& p : probs) nmin = std::min(nmin, p.N);
-    return (bn == 256 || nmin >= 256) ? gemm_cfg(256, 6, 2) : gemm_cfg(128, 8, 2);
+    return (bn == 256 || nmin >= 256) ? gemm_cfg(256, 5, 2) : gemm_cfg(128, 7, 2);
   }
   return bn == 256 ? gemm_cfg(256, 4) : (bn == 128 ? gemm_cfg(128, 4) : gemm_cfg(64, 4));
 }

@@ -9,15 +9,15 @@
 // sizes, epilogue descriptor) lives in device memory and is never written
 // while kernels run.
 //
-// One CTA computes one 128 x BN tile (BN in {64, 128, 256}); 128 threads:
+// One CTA computes one 128 x BN tile (BN in {64, 128, 256}); 256 threads:
 //   warp 0 / lane 0 -- TMA producer: 64-wide K slices of A and B (as 64-row
 //                      boxes: every tensor map has box {64, 64}) into a
 //                      STAGES-deep shared-memory ring (128-byte swizzle);
 //   warp 1 / lane 0 -- MMA issuer: 4 x tcgen05.mma (K = 16 each) per slice
 //                      into the FP32 accumulator in TMEM (128 lanes x BN cols);
-//   all 4 warps     -- epilogue: warp w reads TMEM lanes 32w..32w+31 (rows)
-//                      in chunks of 32 columns and applies the problem's
-//                      epilogue (vectorised row stores).
+//   all 8 warps     -- epilogue: warp w reads TMEM lanes 32 (w % 4) .. (rows)
+//                      of every second 32-column step and applies the problem's
+//                      epilogue (whole row segments, through shared memory).
 // Either operand may be stored MN-major instead (the weight gradients read the
 // activations and output gradients as they are stored: the batch is K).
 // Out-of-range rows and columns of the operands are zero-filled by TMA; the
@@ -80,6 +80,9 @@ static_assert(alignof(GemmProblem) >= 64 && sizeof(GemmProblem) % 64 == 0, "prob
 // Ring depth STAGES: deep rings keep a whole 512-deep product in flight at
 // once (latency-bound small problems); shallow ones leave room for two CTAs
 // per SM, one's epilogue overlapping the other's main loop (large problems).
+constexpr int kTileThreads = 256;        // one-tile kernel: 8 warps
+constexpr int kPersistentThreads = 320;  // persistent kernel: producer, issuer, 8 epilogue warps
+constexpr int kPairThreads = 384;        // CTA-pair kernel: producer, issuer, relay, a spare, 8 epilogue warps
 template <int BN, int STAGES>
 struct GemmSmem {
   static constexpr uint32_t kABytes = kBM * kBK * 2;   // 16 KiB
@@ -88,28 +91,14 @@ struct GemmSmem {
   static constexpr int kStages = STAGES;
   // operand ring + barriers (full[S], empty[S], done) + TMEM slot, plus 1 KiB for alignment
   static constexpr uint32_t kBytes = kStages * kStageBytes + 1024 + 256;
+  // the persistent kernel's epilogue runs beside the ring and has staging blocks of its own
+  static constexpr uint32_t kPersistentBytes = kBytes + 8 * 4096;
   static constexpr uint32_t kTmemCols = BN;
   static_assert(BN % 64 == 0 && BN <= 256, "BN must be 64, 128 or 256");
   static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
+  static_assert(kStages * kStageBytes >= 8 * 4096, "the one-tile kernel stages its epilogue in the ring");
 };
 
-// 32 BF16 values -> four 16-byte stores (dst 16-byte aligned)
-__device__ __forceinline__ void store_bf16x32(__nv_bfloat16* dst, const float (&x)[32]) {
-  uint32_t w[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const __nv_bfloat162 p = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
-    w[i] = *reinterpret_cast<const uint32_t*>(&p);
-  }
-  uint4* d = reinterpret_cast<uint4*>(dst);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) d[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-}
-__device__ __forceinline__ void store_f32x32(float* dst, const float (&x)[32]) {
-  float4* d = reinterpret_cast<float4*>(dst);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) d[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-}
 __device__ __forceinline__ void load_bias32(const float* b, float (&x)[32]) {
   const float4* s = reinterpret_cast<const float4*>(b);
 #pragma unroll
@@ -121,21 +110,6 @@ __device__ __forceinline__ void load_bias32(const float* b, float (&x)[32]) {
     x[4 * q + 3] = t.w;
   }
 }
-__device__ __forceinline__ void load_mask32(const __nv_bfloat16* m, bool (&on)[32]) {
-  const uint4* s = reinterpret_cast<const uint4*>(m);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint4 t = s[q];
-    const uint32_t w[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&w[j]);
-      on[8 * q + 2 * j] = __low2float(p) > 0.f;
-      on[8 * q + 2 * j + 1] = __high2float(p) > 0.f;
-    }
-  }
-}
-
 // L2 prefetch of a tile's B operand (the weight side of every product here),
 // issued before pdl_wait so that its DRAM reads overlap the predecessor's
 // tail.  The predecessor never writes it: B holds weights (written by the
@@ -214,129 +188,284 @@ __device__ __forceinline__ uint32_t idesc_major(uint32_t idesc, const GemmProble
   return idesc | ((P->a_mn ? 1u : 0u) << 15) | ((P->b_mn ? 1u : 0u) << 16);
 }
 
-// Epilogue of one 32-column chunk (columns col0 .. col0 + 31) of row `row`.
-// The full-chunk paths use 16-byte accesses; they need 16-byte aligned rows:
-// leading dimensions a multiple of 8 BF16 / 4 FP32 elements (hidden widths
-// are multiples of 8; other widths are tested here) and 16-byte aligned base
-// pointers (library buffers come from cudaMalloc; crl_bind_params rejects
-// parameter and gradient arrays that are not 16-byte aligned).
-__device__ __forceinline__ void epilogue_chunk(const EpiDesc& e, int row, int col0, float (&v)[32], int M, int N) {
-  if (row >= M) return;
-  const bool full = col0 + 32 <= N;
-  using bf16 = __nv_bfloat16;
+// ---- epilogue -----------------------------------------------------------------
+// Eight warps: warp (eg, half) reads TMEM lanes (rows) 32 eg .. 32 eg + 31 and
+// every second column step of the tile.  A thread holds one row's columns, so
+// a direct 16-byte store per thread touches 32 rows: 32 L1 wavefronts and 32
+// half-used lines per instruction (measured 2.7 TB/s into L2 against 4.9-6.0
+// for whole rows).  Each warp therefore turns its block round in 4 KiB of shared
+// memory of its own and stores whole 64- or 128-byte row segments; the ReLU
+// masks of the input gradients are read in that layout too.
+constexpr int kEpiWarps = 8;
+constexpr uint32_t kStageWarpBytes = 4096;
+constexpr uint32_t kStageBytesAll = kEpiWarps * kStageWarpBytes;
+
+// Byte offset of the 16-byte chunk `ch` of row `row` in a warp's staging block:
+// rows of 128 bytes (8 chunks) or of 64 bytes (4 chunks), XOR-swizzled so that
+// both the row-per-thread writes and the segment reads are conflict-free.
+__device__ __forceinline__ uint32_t stage128(int row, int ch) { return row * 128 + ((ch ^ (row & 7)) << 4); }
+__device__ __forceinline__ uint32_t stage64(int row, int ch) { return row * 64 + ((ch ^ ((row >> 1) & 3)) << 4); }
+
+__device__ __forceinline__ uint4 pack_bf16x8(const float* x) {
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
+    w[i] = *reinterpret_cast<const uint32_t*>(&p);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// 32 FP32 columns of the warp's 32 rows through the staging block:
+// f(row, column, float4) for 4 rows of 128 bytes per instruction.
+template <class F>
+__device__ __forceinline__ void emit_f32x4(uint8_t* st, int lane, const float* v, F&& f) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    *reinterpret_cast<float4*>(st + stage128(lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  __syncwarp();
+  const int ch = lane & 7;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int row = 4 * j + (lane >> 3);
+    f(row, 4 * ch, *reinterpret_cast<const float4*>(st + stage128(row, ch)));
+  }
+  __syncwarp();
+}
+// The same, one row of 32 columns per instruction (rows without 16-byte alignment): f(row, column, float).
+template <class F>
+__device__ __forceinline__ void emit_f32(uint8_t* st, int lane, const float* v, F&& f) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    *reinterpret_cast<float4*>(st + stage128(lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  __syncwarp();
+#pragma unroll 8
+  for (int row = 0; row < 32; ++row)
+    f(row, lane, *reinterpret_cast<const float*>(st + stage128(row, lane >> 2) + 4 * (lane & 3)));
+  __syncwarp();
+}
+// NC (64 or 32) BF16 columns: f(j, row, column, uint4 of 8 columns), j = 0 .. NC / 8 - 1.
+template <int NC, class F>
+__device__ __forceinline__ void emit_bf16(uint8_t* st, int lane, const float* v, F&& f) {
+  constexpr int kCh = NC / 8;
+#pragma unroll
+  for (int q = 0; q < kCh; ++q)
+    *reinterpret_cast<uint4*>(st + (NC == 64 ? stage128(lane, q) : stage64(lane, q))) = pack_bf16x8(v + 8 * q);
+  __syncwarp();
+  const int ch = lane % kCh;
+#pragma unroll
+  for (int j = 0; j < kCh; ++j) {
+    const int row = (32 / kCh) * j + lane / kCh;
+    f(j, row, 8 * ch, *reinterpret_cast<const uint4*>(st + (NC == 64 ? stage128(row, ch) : stage64(row, ch))));
+  }
+  __syncwarp();
+}
+
+// Zero the BF16 halves of x whose unit is inactive (mask m <= 0: the post-ReLU
+// activations are never negative, so a live unit is one that is not +-0).
+__device__ __forceinline__ uint32_t mask_pair(uint32_t x, uint32_t m) {
+  const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&m);
+  const uint32_t lo = __low2float(p) > 0.f ? 0x0000FFFFu : 0u, hi = __high2float(p) > 0.f ? 0xFFFF0000u : 0u;
+  return x & (lo | hi);
+}
+
+// 32 columns of a gradient output (weights, split first-layer weights, first-layer inputs).
+__device__ __forceinline__ void epilogue_grad32(const EpiDesc& e, uint8_t* st, int row0, int lane, const float* v,
+                                                int col0, int M, int N) {
+  const int row = row0 + lane;   // v: this row's columns
   switch (e.kind) {
-    case kEpiFwdHidden: {
-      bf16* h = static_cast<bf16*>(e.out0);
-      if (full) {
-        float b[32];
-        load_bias32(e.bias + col0, b);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = fmaxf(v[i] + b[i], 0.f);
-        store_bf16x32(h + (size_t)row * e.ld0 + col0, v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] -= __bfloat162float(__float2bfloat16_rn(v[i]));
-        store_bf16x32(h + (size_t)row * e.ld0 + e.c0 + col0, v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (col0 + i >= N) break;
-          const float x = fmaxf(v[i] + e.bias[col0 + i], 0.f);
-          const bf16 o = __float2bfloat16_rn(x);
-          h[(size_t)row * e.ld0 + col0 + i] = o;
-          h[(size_t)row * e.ld0 + e.c0 + col0 + i] = __float2bfloat16_rn(x - __bfloat162float(o));
-        }
+    case kEpiBwdDW: {
+      float* dW = static_cast<float*>(e.out0);
+      if (col0 < e.kin) {
+        if ((e.kin & 3) == 0)
+          emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
+            if (row0 + r < M && col0 + k < e.kin)
+              *reinterpret_cast<float4*>(dW + (size_t)(row0 + r) * e.kin + col0 + k) = x;
+          });
+        else
+          emit_f32(st, lane, v, [&](int r, int k, float x) {
+            if (row0 + r < M && col0 + k < e.kin) dW[(size_t)(row0 + r) * e.kin + col0 + k] = x;
+          });
       }
-      break;
-    }
-    case kEpiFwdPreLN:
-    case kEpiFwdOut: {
-      float* z = static_cast<float*>(e.out0) + (size_t)row * e.ld0;
-      if (full && (e.ld0 & 3) == 0) {
-        float b[32];
-        load_bias32(e.bias + col0, b);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] += b[i];
-        store_f32x32(z + col0, v);
-      } else {
+      if (row < M && e.kin >= col0 && e.kin < col0 + 32) {
+        float* db = static_cast<float*>(e.out1);
 #pragma unroll
         for (int i = 0; i < 32; ++i)
-          if (col0 + i < N) z[col0 + i] = v[i] + e.bias[col0 + i];
-      }
-      break;
-    }
-    case kEpiBwdDX:
-    case kEpiBwdDXLN: {
-      const bf16* mrow = e.mask + (size_t)row * e.ldm;
-      if (full) {
-        bool on[32];
-        load_mask32(mrow + col0, on);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = on[i] ? v[i] : 0.f;
-        if (e.kind == kEpiBwdDXLN) store_f32x32(static_cast<float*>(e.out0) + (size_t)row * e.ld0 + col0, v);
-        else store_bf16x32(static_cast<bf16*>(e.out0) + (size_t)row * e.ld0 + col0, v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int c = col0 + i;
-          if (c >= N) break;
-          const float x = __bfloat162float(mrow[c]) > 0.f ? v[i] : 0.f;
-          if (e.kind == kEpiBwdDXLN) static_cast<float*>(e.out0)[(size_t)row * e.ld0 + c] = x;
-          else static_cast<bf16*>(e.out0)[(size_t)row * e.ld0 + c] = __float2bfloat16_rn(x);
-        }
-      }
-      break;
-    }
-    case kEpiBwdDW: {
-      float* dW = static_cast<float*>(e.out0) + (size_t)row * e.kin;
-      if (col0 + 32 <= e.kin && (e.kin & 3) == 0) {
-        store_f32x32(dW + col0, v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int c = col0 + i;
-          if (c >= N) break;
-          if (c < e.kin) dW[c] = v[i];
-          else static_cast<float*>(e.out1)[row] = v[i];
-        }
+          if (col0 + i == e.kin) db[row] = v[i];
       }
       break;
     }
     case kEpiBwdDW0: {
-      float* dW = static_cast<float*>(e.out0) + (size_t)row * e.kin;
+      float* dW = static_cast<float*>(e.out0);
+      // 16 summed columns per row, turned round so that 16 lanes store a row's segment
 #pragma unroll
-      for (int i = 0; i < 32; i += 2) {
-        const int c = col0 + i;
-        if (c < 2 * e.kin) dW[c / 2] = v[i] + v[i + 1];
-        else if (c == 2 * e.kin) static_cast<float*>(e.out1)[row] = v[i];
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(st + stage64(lane, q)) =
+            make_float4(v[8 * q] + v[8 * q + 1], v[8 * q + 2] + v[8 * q + 3], v[8 * q + 4] + v[8 * q + 5],
+                        v[8 * q + 6] + v[8 * q + 7]);
+      __syncwarp();
+      const int k = lane & 15, c = col0 / 2 + k;
+#pragma unroll 8
+      for (int j = 0; j < 16; ++j) {
+        const int r = 2 * j + (lane >> 4);
+        const float x = *reinterpret_cast<const float*>(st + stage64(r, k >> 2) + 4 * (k & 3));
+        if (row0 + r < M && c < e.kin) dW[(size_t)(row0 + r) * e.kin + c] = x;
+      }
+      __syncwarp();
+      if (row < M && 2 * e.kin >= col0 && 2 * e.kin < col0 + 32) {
+        float* db = static_cast<float*>(e.out1);
+#pragma unroll
+        for (int i = 0; i < 32; i += 2)
+          if (col0 + i == 2 * e.kin) db[row] = v[i];
       }
       break;
     }
     default: {  // kEpiDX0
-      float* dx = static_cast<float*>(e.out0) + (size_t)row * e.nc;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int c = col0 + i - e.c0;
-        if (col0 + i < N && c >= 0 && c < e.nc) dx[c] = v[i];
-      }
+      float* dx = static_cast<float*>(e.out0);
+      if (col0 + 32 <= e.c0 || col0 >= e.c0 + e.nc) break;
+      emit_f32(st, lane, v, [&](int r, int k, float x) {
+        const int c = col0 + k - e.c0;
+        if (row0 + r < M && col0 + k < N && c >= 0 && c < e.nc) dx[(size_t)(row0 + r) * e.nc + c] = x;
+      });
       break;
     }
   }
 }
 
-// The output layer feeding the fused energy (kEpiFwdOutEnergy): two passes over
-// this thread's row in TMEM (the tile holds all N columns): FP32 output and the
-// squared norm, then the scaled BF16 operand.
-__device__ __forceinline__ void epilogue_energy(const EpiDesc& e, int row, uint32_t lane_base, int N, int M) {
+// One step: NC (32 or 64) columns from col0 of the warp's rows row0 .. row0 + 31.
+// Hidden widths are multiples of 8 (their BF16 rows need 16-byte TMA strides),
+// so an 8-column chunk of a BF16 output lies wholly inside or outside the
+// problem; FP32 rows without 16-byte alignment (odd widths) take 4-byte stores.
+template <int NC>
+__device__ __forceinline__ void epilogue_step(const EpiDesc& e, uint8_t* st, int row0, int lane, uint32_t taddr,
+                                              int col0, int M, int N) {
   using bf16 = __nv_bfloat16;
-  const bool live = row < M;
+  float v[NC];
+  switch (e.kind) {
+    case kEpiFwdHidden: {
+      tmem_ldn(taddr, v);
+      bf16* h = static_cast<bf16*>(e.out0);
+#pragma unroll
+      for (int c = 0; c < NC; c += 32) {
+        float b[32];
+        if (col0 + c + 32 <= N) {
+          load_bias32(e.bias + col0 + c, b);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) b[i] = col0 + c + i < N ? __ldg(e.bias + col0 + c + i) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[c + i] = fmaxf(v[c + i] + b[i], 0.f);
+      }
+      auto put = [&](bf16* base) {
+        emit_bf16<NC>(st, lane, v, [&](int, int r, int c, uint4 x) {
+          if (row0 + r < M && col0 + c < N)
+            *reinterpret_cast<uint4*>(base + (size_t)(row0 + r) * e.ld0 + col0 + c) = x;
+        });
+      };
+      put(h);
+#pragma unroll
+      for (int i = 0; i < NC; ++i) v[i] -= __bfloat162float(__float2bfloat16_rn(v[i]));
+      put(h + e.c0);
+      break;
+    }
+    case kEpiFwdPreLN:
+    case kEpiFwdOut: {
+      tmem_ldn(taddr, v);
+      float* z = static_cast<float*>(e.out0);
+      const bool vec = (e.ld0 & 3) == 0 && (N & 3) == 0;
+#pragma unroll
+      for (int c = 0; c < NC; c += 32) {
+        if (col0 + c >= N) break;
+        float b[32];
+        if (col0 + c + 32 <= N) {
+          load_bias32(e.bias + col0 + c, b);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) b[i] = col0 + c + i < N ? __ldg(e.bias + col0 + c + i) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[c + i] += b[i];
+        if (vec)
+          emit_f32x4(st, lane, v + c, [&](int r, int k, float4 x) {
+            if (row0 + r < M && col0 + c + k < N)
+              *reinterpret_cast<float4*>(z + (size_t)(row0 + r) * e.ld0 + col0 + c + k) = x;
+          });
+        else
+          emit_f32(st, lane, v + c, [&](int r, int k, float x) {
+            if (row0 + r < M && col0 + c + k < N) z[(size_t)(row0 + r) * e.ld0 + col0 + c + k] = x;
+          });
+      }
+      break;
+    }
+    case kEpiBwdDX: {
+      // the masks of the segments this lane will store, in flight during the TMEM read
+      constexpr int kCh = NC / 8;
+      const int mc = col0 + 8 * (lane % kCh);
+      uint4 m[kCh];
+#pragma unroll
+      for (int j = 0; j < kCh; ++j) {
+        const int r = row0 + (32 / kCh) * j + lane / kCh;
+        m[j] = (r < M && mc < N) ? *reinterpret_cast<const uint4*>(e.mask + (size_t)r * e.ldm + mc)
+                                 : make_uint4(0u, 0u, 0u, 0u);
+      }
+      tmem_ldn(taddr, v);
+      bf16* dz = static_cast<bf16*>(e.out0);
+      emit_bf16<NC>(st, lane, v, [&](int j, int r, int c, uint4 x) {
+        if (row0 + r < M && col0 + c < N)
+          *reinterpret_cast<uint4*>(dz + (size_t)(row0 + r) * e.ld0 + col0 + c) =
+              make_uint4(mask_pair(x.x, m[j].x), mask_pair(x.y, m[j].y), mask_pair(x.z, m[j].z),
+                         mask_pair(x.w, m[j].w));
+      });
+      break;
+    }
+    case kEpiBwdDXLN: {
+      uint2 m[NC / 4];
+#pragma unroll
+      for (int j = 0; j < NC / 4; ++j) {
+        const int r = row0 + 4 * (j & 7) + (lane >> 3), c = col0 + 32 * (j >> 3) + 4 * (lane & 7);
+        m[j] = (r < M && c < N) ? *reinterpret_cast<const uint2*>(e.mask + (size_t)r * e.ldm + c) : make_uint2(0u, 0u);
+      }
+      tmem_ldn(taddr, v);
+      float* du = static_cast<float*>(e.out0);
+#pragma unroll
+      for (int c = 0; c < NC; c += 32) {
+        int j = c / 4;
+        emit_f32x4(st, lane, v + c, [&](int r, int k, float4 x) {
+          const uint2 mm = m[j++];
+          const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&mm.x);
+          const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&mm.y);
+          if (row0 + r < M && col0 + c + k < N)
+            *reinterpret_cast<float4*>(du + (size_t)(row0 + r) * e.ld0 + col0 + c + k) =
+                make_float4(__low2float(a) > 0.f ? x.x : 0.f, __high2float(a) > 0.f ? x.y : 0.f,
+                            __low2float(b) > 0.f ? x.z : 0.f, __high2float(b) > 0.f ? x.w : 0.f);
+        });
+      }
+      break;
+    }
+    default:
+      tmem_ldn(taddr, v);
+#pragma unroll
+      for (int c = 0; c < NC; c += 32)
+        if (col0 + c < N) epilogue_grad32(e, st, row0, lane, v + c, col0 + c, M, N);
+      break;
+  }
+}
+
+// The output layer feeding the fused energy (kEpiFwdOutEnergy): two passes over
+// this thread's row in TMEM (the tile holds all N columns, a multiple of 64):
+// the squared norm of the whole row (both half warps of a row block form it, in
+// column order), then the FP32 output and the scaled BF16 operand of this warp's
+// 32-column chunks.
+__device__ __forceinline__ void epilogue_energy(const EpiDesc& e, uint8_t* st, int row0, int lane, int half,
+                                                uint32_t lane_base, int N, int M) {
+  using bf16 = __nv_bfloat16;
   const bool cosine = e.energy == CRL_ENERGY_COS;
   float q = 0.f;
 #pragma unroll 1
   for (int c = 0; c < N; c += 32) {
-    float v[32];
-    tmem_ld32(lane_base + c, v);   // warp-collective: every lane, live or not
-    if (!live) continue;
-    float b[32];
+    float v[32], b[32];
+    tmem_ldn(lane_base + c, v);
     load_bias32(e.bias + c, b);
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
@@ -344,29 +473,52 @@ __device__ __forceinline__ void epilogue_energy(const EpiDesc& e, int row, uint3
       const float r = cosine ? v[i] : __bfloat162float(__float2bfloat16_rn(v[i]));
       q += r * r;
     }
-    store_f32x32(static_cast<float*>(e.out0) + (size_t)row * e.ld0 + c, v);
   }
   const float scale = cosine ? rsqrtf(q) : 1.f;
-  if (live) e.aux[row] = cosine ? scale : q;
+  if (half == 0 && row0 + lane < M) e.aux[row0 + lane] = cosine ? scale : q;
+  float* y = static_cast<float*>(e.out0);
   bf16* X = static_cast<bf16*>(e.out1);
 #pragma unroll 1
-  for (int c = 0; c < N; c += 32) {
-    float v[32];
-    tmem_ld32(lane_base + c, v);
-    if (!live) continue;
-    float b[32];
+  for (int c = 32 * half; c < N; c += 64) {
+    float v[32], b[32];
+    tmem_ldn(lane_base + c, v);
     load_bias32(e.bias + c, b);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = (v[i] + b[i]) * scale;
-    store_bf16x32(X + (size_t)row * N + c, v);
+    for (int i = 0; i < 32; ++i) v[i] += b[i];
+    emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
+      if (row0 + r < M) *reinterpret_cast<float4*>(y + (size_t)(row0 + r) * e.ld0 + c + k) = x;
+    });
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] *= scale;
+    emit_bf16<32>(st, lane, v, [&](int, int r, int k, uint4 x) {
+      if (row0 + r < M) *reinterpret_cast<uint4*>(X + (size_t)(row0 + r) * N + c + k) = x;
+    });
   }
+}
+
+// The warp's share of a 128 x BN tile at (m0, n0), accumulator at `acc`: rows
+// m0 + 32 eg .., every second step of NC columns.
+template <int BN, int NC>
+__device__ __forceinline__ void epilogue_tile(const EpiDesc& e, uint8_t* st, uint32_t acc, int eg, int half, int lane,
+                                              int m0, int n0, int M, int N) {
+  static_assert(BN % (2 * NC) == 0, "two half warps share the tile's steps");
+  const int row0 = m0 + 32 * eg;
+  if (row0 >= M) return;
+  const uint32_t lane_base = acc + ((uint32_t)(32 * eg) << 16);
+  if (e.kind == kEpiFwdOutEnergy) {
+    epilogue_energy(e, st, row0, lane, half, lane_base, N, M);
+    return;
+  }
+  const int ncol = (N - n0 < BN) ? N - n0 : BN;
+#pragma unroll 1
+  for (int c = NC * half; c < ncol; c += 2 * NC) epilogue_step<NC>(e, st, row0, lane, lane_base + c, n0 + c, M, N);
 }
 
 // nkA > 0: A has only nkA K-slices and slice kb of B multiplies slice kb % nkA of
 // A -- B holds the weight pair along K ([W_hi | W_lo], or [W_hi | W_hi | W_lo]
 // against A = [h_hi | h_lo]) and each A tile is used against several parts.
 template <int BN, int STAGES>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTileThreads, (GemmSmem<BN, STAGES>::kBytes <= 113 * 1024) ? 2 : 1)
     tc_gemm_kernel(const GemmProblem* __restrict__ probs, int nprob, unsigned* status) {
   using S = GemmSmem<BN, STAGES>;
   extern __shared__ uint8_t smem_raw[];
@@ -467,24 +619,34 @@ __global__ void __launch_bounds__(128, 1)
   }
   __syncwarp();
 
-  // epilogue (tcgen05.ld is warp-collective: keep the decision warp-uniform)
+  // epilogue (tcgen05.ld is warp-collective: keep the decision warp-uniform).
+  // Every MMA has completed, so the operand ring is free: it becomes the warps'
+  // staging blocks.
   const bool ok = __all_sync(0xffffffffu, mbar_wait(done, 0, lim) ? 1 : 0) != 0;
   fence_after_sync();
+  const int eg = warp & 3, half = warp >> 2;
+  uint8_t* stage = smem + warp * kStageWarpBytes;
   if (ok && ksplit > 1) {
     // split-K: store this split's FP32 partial tile; the last CTA of the tile to
-    // arrive adds the ksplit partials in split order (its own from TMEM) and
-    // runs the epilogue, so the result does not depend on which CTA is last
+    // arrive adds the ksplit partials in split order (its own included) and runs
+    // the epilogue, so the result does not depend on which CTA is last.  A
+    // partial is [BN / 4][128 rows] 16-byte pieces: a warp's accesses are
+    // contiguous (row-major partials cost 32 lines per instruction both ways).
     __shared__ int s_last;
     const EpiDesc e = P->epi;
-    const int r = warp * 32 + lane, row = m0 + r;
-    const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+    const int r = eg * 32 + lane;
+    const uint32_t lane_base = tmem + ((uint32_t)(eg * 32) << 16);
     const int ncol = (N - n0 < BN) ? N - n0 : BN;
-    float* part = P->part + (size_t)lt * ksplit * kBM * BN;
+    float4* part = reinterpret_cast<float4*>(P->part + (size_t)lt * ksplit * kBM * BN) + r;
+    constexpr size_t kPart = (size_t)kBM * BN / 4;   // 16-byte pieces per partial tile
 #pragma unroll 1
-    for (int c = 0; c < ncol; c += 32) {
+    for (int c = 32 * half; c < ncol; c += 64) {
       float v[32];
-      tmem_ld32(lane_base + c, v);
-      store_f32x32(part + ((size_t)split * kBM + r) * BN + c, v);
+      tmem_ldn(lane_base + c, v);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        __stcg(part + split * kPart + (size_t)(c / 4 + i) * kBM,
+               make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
     }
     __threadfence();
     __syncthreads();
@@ -493,40 +655,28 @@ __global__ void __launch_bounds__(128, 1)
     if (s_last) {
       __threadfence();
 #pragma unroll 1
-      for (int c = 0; c < ncol; c += 32) {
+      for (int c = 32 * half; c < ncol; c += 64) {
         float v[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = 0.f;
+#pragma unroll 2
         for (int q = 0; q < ksplit; ++q) {
-          const float4* src = reinterpret_cast<const float4*>(part + ((size_t)q * kBM + r) * BN + c);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const float4 x = __ldcg(src + i);
+            const float4 x = __ldcg(part + q * kPart + (size_t)(c / 4 + i) * kBM);
             v[4 * i] += x.x;
             v[4 * i + 1] += x.y;
             v[4 * i + 2] += x.z;
             v[4 * i + 3] += x.w;
           }
         }
-        epilogue_chunk(e, row, n0 + c, v, M, N);
+        if (m0 + 32 * eg < M) epilogue_grad32(e, stage, m0 + 32 * eg, lane, v, n0 + c, M, N);
       }
       if (threadIdx.x == 0) P->tickets[lt] = 0u;
     }
   } else if (ok) {
     const EpiDesc e = P->epi;
-    const int row = m0 + warp * 32 + lane;
-    const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-    const int ncol = (N - n0 < BN) ? N - n0 : BN;
-    if (e.kind == kEpiFwdOutEnergy) {
-      epilogue_energy(e, row, lane_base, ncol, M);
-    } else {
-#pragma unroll 1
-      for (int c = 0; c < ncol; c += 32) {
-        float v[32];
-        tmem_ld32(lane_base + c, v);
-        epilogue_chunk(e, row, n0 + c, v, M, N);
-      }
-    }
+    epilogue_tile<BN, 32>(e, stage, tmem, eg, half, lane, m0, n0, M, N);
   } else if (threadIdx.x == 0) {
     atomicOr(status, CRL_STATUS_TIMEOUT);
   }
@@ -550,28 +700,29 @@ __device__ __forceinline__ const GemmProblem* find_problem(const GemmProblem* __
 
 // Persistent variant: gridDim.x CTAs (one per SM at most) walk the tiles
 // t = blockIdx.x, blockIdx.x + gridDim.x, ... of the whole problem list.
-// 192 threads:
+// 320 threads:
 //   warp 0 / lane 0 -- TMA producer over all of the CTA's tiles: the operand
 //                      ring runs on across tile boundaries;
 //   warp 1 / lane 0 -- MMA issuer: tile i accumulates into TMEM buffer i % 2
 //                      (2 x BN columns), once the epilogue has released it;
-//   warps 2..5      -- epilogue of tile i from buffer i % 2 while the MMAs of
+//   warps 2..9      -- epilogue of tile i from buffer i % 2 while the MMAs of
 //                      tile i + 1 fill the other one (warp w reads TMEM lanes
-//                      32 (w % 4) ..).
+//                      32 (w % 4) .., every second column step).
 // The epilogue is the same as the one-tile kernel's, so both give identical
 // outputs.
 template <int BN, int STAGES>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kPersistentThreads, 1)
     tc_gemm_persistent_kernel(const GemmProblem* __restrict__ probs, int nprob, int total, unsigned* status) {
   using S = GemmSmem<BN, STAGES>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   uint8_t* sA = smem;
   uint8_t* sB = smem + S::kStages * S::kABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kStages * S::kStageBytes);
+  uint8_t* sE = smem + S::kStages * S::kStageBytes;   // epilogue staging, 4 KiB per warp
+  uint64_t* full = reinterpret_cast<uint64_t*>(sE + kStageBytesAll);
   uint64_t* empty = full + S::kStages;
   uint64_t* accf = empty + S::kStages;  // [2] accumulator buffer ready (MMA -> epilogue)
-  uint64_t* acce = accf + 2;            // [2] accumulator buffer free (epilogue -> MMA), 4 arrivals
+  uint64_t* acce = accf + 2;            // [2] accumulator buffer free (epilogue -> MMA), 8 arrivals
   uint64_t* drain = acce + 2;           // every MMA of this CTA has completed (teardown)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
@@ -588,7 +739,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 4);
+      mbar_init(&acce[b], kEpiWarps);
     }
     mbar_init(drain, 1);
     fence_mbar_init();
@@ -670,7 +821,8 @@ __global__ void __launch_bounds__(192, 1)
     }
   } else {
     // epilogue warps (tcgen05.ld is warp-collective: decisions stay warp-uniform)
-    const int eg = warp & 3;
+    constexpr int NC = BN >= 128 ? 64 : 32;
+    const int eg = warp & 3, ew = warp - 2, half = ew >> 2;
     int i = 0;
     for (int t = blockIdx.x; t < total; t += gridDim.x, ++i) {
       const int buf = i & 1, use = i >> 1;
@@ -685,19 +837,7 @@ __global__ void __launch_bounds__(192, 1)
       const int m0 = (lt / P->tiles_n) * kBM, n0 = (lt % P->tiles_n) * BN;
       const int M = P->M, N = P->N;
       const EpiDesc e = P->epi;
-      const int row = m0 + eg * 32 + lane;
-      const uint32_t lane_base = tmem + (uint32_t)(buf * BN) + ((uint32_t)(eg * 32) << 16);
-      const int ncol = (N - n0 < BN) ? N - n0 : BN;
-      if (e.kind == kEpiFwdOutEnergy) {
-        epilogue_energy(e, row, lane_base, ncol, M);
-      } else {
-#pragma unroll 1
-        for (int c = 0; c < ncol; c += 32) {
-          float v[32];
-          tmem_ld32(lane_base + c, v);
-          epilogue_chunk(e, row, n0 + c, v, M, N);
-        }
-      }
+      epilogue_tile<BN, NC>(e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
       // release the buffer to the MMA issuer
       fence_before_sync();
       __syncwarp();
@@ -723,10 +863,10 @@ __global__ void __launch_bounds__(192, 1)
 //   warp 1 / lane 0 -- even CTA: MMA issuer (waits for its own slot and the
 //                      odd CTA's `pfull` arrival); odd CTA: reports each
 //                      landed slot to the even CTA's `pfull`;
-//   warps 2..5      -- epilogue of this CTA's 128 rows from TMEM buffer i % 2;
-//                      all eight warps release the buffer on the even CTA's `acce`;
-//   warp 6 / lane 0 -- even CTA: passes each freed slot (`empty`) and each
-//                      finished accumulator (`accf`) on to the odd CTA.
+//   warp 2 / lane 0 -- even CTA: passes each freed slot (`empty`) and each
+//                      finished accumulator (`accf`) on to the odd CTA;
+//   warps 4..11     -- epilogue of this CTA's 128 rows from TMEM buffer i % 2;
+//                      the pair's sixteen warps release it on the even CTA's `acce`.
 // The epilogue is the one-tile kernel's, so every kernel gives identical outputs
 // where the MMA sums each K = 16 slice the same way.
 template <int BN, int STAGES>
@@ -737,8 +877,8 @@ struct GemmPairSmem {
   static constexpr int kStages = STAGES;
   // ring + barriers (full, empty, pfull [S]; accf, acce [2]; drain) + TMEM slot, plus 1 KiB for
   // alignment and one more B half behind the ring, so that the last slot's B rows plus BN / 2
-  // rows stay inside this CTA's shared memory
-  static constexpr uint32_t kBytes = kStages * kStageBytes + kBBytes + 1024 + 512;
+  // rows stay inside this CTA's shared memory; then the epilogue's staging blocks
+  static constexpr uint32_t kBytes = kStages * kStageBytes + kBBytes + 8 * 4096 + 1024 + 512;
   static constexpr uint32_t kTmemCols = 2 * BN;   // two accumulator buffers
   static_assert(BN == 128 || BN == 256, "pair tiles are 256 x 128 or 256 x 256");
   static_assert(kTmemCols <= 512, "TMEM columns");
@@ -746,7 +886,7 @@ struct GemmPairSmem {
 };
 
 template <int BN, int STAGES>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     tc_gemm_pair_kernel(const GemmProblem* __restrict__ probs, int nprob, int total, unsigned* status) {
   using S = GemmPairSmem<BN, STAGES>;
   constexpr int kPairM = 2 * kBM;
@@ -754,11 +894,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
   uint8_t* smem = align1024(smem_raw);
   uint8_t* sA = smem;
   uint8_t* sB = smem + S::kStages * S::kABytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kStages * S::kStageBytes + S::kBBytes);
+  uint8_t* sE = smem + S::kStages * S::kStageBytes + S::kBBytes;   // epilogue staging, 4 KiB per warp
+  uint64_t* full = reinterpret_cast<uint64_t*>(sE + kStageBytesAll);
   uint64_t* empty = full + S::kStages;
   uint64_t* pfull = empty + S::kStages;  // even CTA: the odd CTA's slot has landed
   uint64_t* accf = pfull + S::kStages;   // [2] accumulator buffer ready
-  uint64_t* acce = accf + 2;             // [2] even CTA: buffer read out by all 8 epilogue warps
+  uint64_t* acce = accf + 2;             // [2] even CTA: buffer read out by all 16 epilogue warps
   uint64_t* drain = acce + 2;            // every MMA of the pair has completed (teardown)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
@@ -779,7 +920,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accf[b], 1);
-      mbar_init(&acce[b], 8);
+      mbar_init(&acce[b], 2 * kEpiWarps);
     }
     mbar_init(drain, 1);
     fence_mbar_init();
@@ -839,7 +980,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
         const bool amn = P->a_mn != 0, bmn = P->b_mn != 0;
         const uint32_t sa = slice_step(amn), sb = slice_step(bmn);
         const int buf = i & 1, use = i >> 1;
-        // all eight epilogue warps must have read out this buffer (tile i - 2)
+        // all sixteen epilogue warps must have read out this buffer (tile i - 2)
         if (use > 0 && !mbar_wait_cluster(&acce[buf], (use - 1) & 1, lim)) {
           atomicOr(status, CRL_STATUS_TIMEOUT);
           break;
@@ -882,7 +1023,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
         }
       }
     }
-  } else if (warp == 6) {
+  } else if (warp == 2) {
     if (lane == 0 && even) {
       // relay of the even CTA: every completed MMA slice frees the odd CTA's
       // slot too, and every completed tile its accumulator rows (a thread of
@@ -911,9 +1052,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
         mbar_arrive_remote(mapa_shared(&accf[buf], 1));
       }
     }
-  } else {
+  } else if (warp >= 4) {
     // epilogue warps: this CTA's 128 rows of the pair's tile
-    const int eg = warp & 3;
+    constexpr int NC = 64;
+    const int eg = warp & 3, ew = warp - 4, half = ew >> 2;
     int i = 0;
     for (int t = cl; t < total; t += ncl, ++i) {
       const int buf = i & 1, use = i >> 1;
@@ -929,19 +1071,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(224, 1)
       const int m0 = (lt / P->tiles_n) * kPairM + kBM * (int)rank, n0 = (lt % P->tiles_n) * BN;
       const int M = P->M, N = P->N;
       const EpiDesc e = P->epi;
-      const int row = m0 + eg * 32 + lane;
-      const uint32_t lane_base = tmem + (uint32_t)(buf * BN) + ((uint32_t)(eg * 32) << 16);
-      const int ncol = (N - n0 < BN) ? N - n0 : BN;
-      if (e.kind == kEpiFwdOutEnergy) {
-        epilogue_energy(e, row, lane_base, ncol, M);
-      } else {
-#pragma unroll 1
-        for (int c = 0; c < ncol; c += 32) {
-          float v[32];
-          tmem_ld32(lane_base + c, v);
-          epilogue_chunk(e, row, n0 + c, v, M, N);
-        }
-      }
+      epilogue_tile<BN, NC>(e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
       // release the buffer to the MMA issuer
       fence_before_sync();
       __syncwarp();
