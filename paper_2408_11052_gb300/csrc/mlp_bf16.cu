@@ -585,39 +585,50 @@ bool cfg_allowed(int cfg) {
 }
 constexpr int kGemmCfgs[10] = {gemm_cfg(64, 4),     gemm_cfg(64, 8),     gemm_cfg(128, 3),    gemm_cfg(128, 6),
                                gemm_cfg(256, 4),    gemm_cfg(64, 8, 1),  gemm_cfg(128, 6, 1), gemm_cfg(256, 4, 1),
-                               gemm_cfg(128, 7, 2), gemm_cfg(256, 5, 2)};
+                               gemm_cfg(128, 8, 2), gemm_cfg(256, 6, 2)};
 
 void launch_cfg(int cfg, const tc::GemmProblem* t, int nprob, int tiles, unsigned* status, cudaStream_t st) {
   switch (cfg) {
-    case gemm_cfg(128, 7, 2): launch_gemm_pair<128, 7>(t, nprob, tiles, status, st); break;
-    case gemm_cfg(256, 5, 2): launch_gemm_pair<256, 5>(t, nprob, tiles, status, st); break;
+    case gemm_cfg(128, 8, 2): launch_gemm_pair<128, 8>(t, nprob, tiles, status, st); break;
+    case gemm_cfg(256, 6, 2): launch_gemm_pair<256, 6>(t, nprob, tiles, status, st); break;
     case gemm_cfg(64, 8, 1): launch_gemm_persistent<64, 8>(t, nprob, tiles, status, st); break;
     case gemm_cfg(128, 6, 1): launch_gemm_persistent<128, 6>(t, nprob, tiles, status, st); break;
     case gemm_cfg(256, 4, 1): launch_gemm_persistent<256, 4>(t, nprob, tiles, status, st); break;
     case gemm_cfg(64, 8): launch_gemm_cfg<64, 8>(t, nprob, tiles, status, st); break;
     case gemm_cfg(128, 3): launch_gemm_cfg<128, 3>(t, nprob, tiles, status, st); break;
-    case gemm_cfg(128, 4): launch_gemm_cfg<128, 4>(t, nprob, tiles, status, st); break;
     case gemm_cfg(128, 6): launch_gemm_cfg<128, 6>(t, nprob, tiles, status, st); break;
     case gemm_cfg(256, 4): launch_gemm_cfg<256, 4>(t, nprob, tiles, status, st); break;
     default: launch_gemm_cfg<64, 4>(t, nprob, tiles, status, st); break;
   }
 }
 
-// Configuration without measurement: 128 x 64 tiles unless 128 x 128 tiles
-// already fill the 152 SMs; 4-deep rings.
-int heuristic_cfg(const std::vector<tc::GemmProblem>& probs, int min_bn) {
-  long long ctas128 = 0;
-  for (const auto& p : probs) ctas128 += (long long)ceil_div(p.M, 128) * ceil_div(p.N, 128);
+// Configuration without measurement (op-level calls, and contexts with the tuner
+// off).  Wide problems (every N >= 256) whose 128 x 256 tiles come near to filling
+// the SMs take those: one tile per CTA for a single wave, else the persistent
+// kernel, whose epilogue runs beside the next tile's products (us, 128 x 128
+// tiles with a 3-deep ring first: 3 x [8192 x 512 x 1536] 58 -> 42, 2 x [8192 x
+// 512 x 512] 20.7 -> 16.6, 1 x [8192 x 512 x 512] 11.8 -> 11.1).  Fewer tiles than
+// that leave SMs idle: 128 x 128 tiles, two CTAs per SM, where they fill the SMs,
+// else 128 x 64, with the deep ring where every CTA has an SM to itself.
+int heuristic_cfg(const std::vector<tc::GemmProblem>& probs, int min_bn, bool one_tile_only) {
+  long long ctas64 = 0, ctas128 = 0, ctas256 = 0;
+  int nmin = 1 << 30;
+  for (const auto& p : probs) {
+    ctas64 += (long long)ceil_div(p.M, 128) * ceil_div(p.N, 64);
+    ctas128 += (long long)ceil_div(p.M, 128) * ceil_div(p.N, 128);
+    ctas256 += (long long)ceil_div(p.M, 128) * ceil_div(p.N, 256);
+    nmin = std::min(nmin, p.N);
+  }
   const int bn = std::max(ctas128 >= 148 ? 128 : 64, min_bn <= 64 ? 64 : (min_bn <= 128 ? 128 : 256));
   if (g_gemm_kernel == CRL_GEMM_PERSISTENT)
     return bn == 256 ? gemm_cfg(256, 4, 1) : (bn == 128 ? gemm_cfg(128, 6, 1) : gemm_cfg(64, 8, 1));
-  if (g_gemm_kernel == CRL_GEMM_CTA_PAIR) {
-    // pair tiles want width: 256 columns wherever every problem has them
-    int nmin = 1 << 30;
-    for (const auto& p : probs) nmin = std::min(nmin, p.N);
-    return (bn == 256 || nmin >= 256) ? gemm_cfg(256, 5, 2) : gemm_cfg(128, 7, 2);
-  }
-  return bn == 256 ? gemm_cfg(256, 4) : (bn == 128 ? gemm_cfg(128, 4) : gemm_cfg(64, 4));
+  if (g_gemm_kernel == CRL_GEMM_CTA_PAIR)   // pair tiles want width: 256 columns wherever every problem has them
+    return (bn == 256 || nmin >= 256) ? gemm_cfg(256, 6, 2) : gemm_cfg(128, 8, 2);
+  if (nmin >= 256 && ctas256 >= 96 && ctas256 <= sm_count()) return gemm_cfg(256, 4);
+  if (nmin >= 256 && ctas256 > sm_count() && g_gemm_kernel == CRL_GEMM_ANY && !one_tile_only) return gemm_cfg(256, 4, 1);
+  if (bn == 256) return gemm_cfg(256, 4);
+  if (bn == 128) return gemm_cfg(128, 3);
+  return ctas64 <= sm_count() ? gemm_cfg(64, 8) : gemm_cfg(64, 4);
 }
 
 // Autotuner: time each candidate configuration (tile width, ring depth) on
@@ -688,8 +699,10 @@ const char* launch_group(GemmGroups& gg, std::vector<tc::GemmProblem>& probs, do
   const uint64_t key = fnv1a(probs.data(), probs.size() * sizeof(tc::GemmProblem));
   // an energy-operand epilogue needs the whole row in one tile
   int min_bn = 0;
-  for (const auto& p : probs)
+  for (const auto& p : probs) {
     if (p.epi.kind == tc::kEpiFwdOutEnergy) min_bn = std::max(min_bn, p.N);
+    if (p.epi.kind == tc::kEpiFwdHidden && !p.tma_out) return "no output map for a hidden layer (16-byte alignment)";
+  }
   if (min_bn > 256) return "an energy-operand output layer wider than 256 columns";
   // a list that splits over K stays on the one-tile kernel whatever the timings
   // say, so its outputs never depend on the pick (all one-tile widths give the
@@ -705,7 +718,7 @@ const char* launch_group(GemmGroups& gg, std::vector<tc::GemmProblem>& probs, do
       cfg = tune_cfg(gg, probs, min_bn, one_tile_only, status, st, flops);
       if (cfg) gg.set_tuned_bn(key, cfg);
     }
-    if (cfg == 0) cfg = heuristic_cfg(probs, min_bn);
+    if (cfg == 0) cfg = heuristic_cfg(probs, min_bn, one_tile_only);
   }
   int tiles = 0;
   const char* err = nullptr;
@@ -1026,6 +1039,12 @@ tc::GemmProblem forward_problem(const BfPass& bp, int l, bool ln) {
   if (l > 0) {   // h_lo sits two 64-column blocks after h_hi's last slice
     p.a_gap = L.kp / 64;
     p.a_skip = L.kp / 64;
+  }
+  if (e.kind == tc::kEpiFwdHidden) {
+    p.tma_out = tc::make_tmap_store(&p.o0, n.h[l], H, bp.M, n.ldh, false) &&
+                tc::make_tmap_store(&p.o1, n.h[l] + n.hlo, H, bp.M, n.ldh, false);
+  } else if (e.kind != tc::kEpiFwdOutEnergy) {
+    p.tma_out = tc::make_tmap_store(&p.o0, e.out0, L.out, bp.M, e.ld0, true);
   }
   return p;
 }

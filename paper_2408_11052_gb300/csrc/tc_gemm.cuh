@@ -64,6 +64,7 @@ struct EpiDesc {
 
 struct GemmProblem {   // 128-byte aligned by its tensor maps
   CUtensorMap a, b;
+  CUtensorMap o0, o1;   // tma_out: output maps, boxes of 32 rows x 128 bytes (o1: the lo part of a hidden layer)
   int M, N, K, nkA;   // nkA > 0: split-weight product (see tc_gemm_kernel)
   int a_mn, b_mn;     // operand stored MN-major ([K][M] / [K][N], the M / N index contiguous): its
                       // tensor map's inner dimension is M / N, boxes {64 MN, 64 K}
@@ -71,6 +72,7 @@ struct GemmProblem {   // 128-byte aligned by its tensor maps
   int tiles_n, tile_begin;
   int ksplit;         // > 1: K is split over ksplit CTAs per output tile (one-tile kernel only)
   int ksplit_cap;     // the most splits the problem's buffers hold (the launch picks ksplit <= it)
+  int tma_out, pad_;
   EpiDesc epi;
   float* part;        // split-K partial tiles [tile][ksplit][128][BN] (FP32)
   unsigned* tickets;  // split-K arrival count per output tile (zero between launches)
@@ -82,7 +84,7 @@ static_assert(alignof(GemmProblem) >= 64 && sizeof(GemmProblem) % 64 == 0, "prob
 // per SM, one's epilogue overlapping the other's main loop (large problems).
 constexpr int kTileThreads = 256;        // one-tile kernel: 8 warps
 constexpr int kPersistentThreads = 320;  // persistent kernel: producer, issuer, 8 epilogue warps
-constexpr int kPairThreads = 384;        // CTA-pair kernel: producer, issuer, relay, a spare, 8 epilogue warps
+constexpr int kPairThreads = 320;        // CTA-pair kernel: producer, issuer, 8 epilogue warps
 template <int BN, int STAGES>
 struct GemmSmem {
   static constexpr uint32_t kABytes = kBM * kBK * 2;   // 16 KiB
@@ -110,6 +112,7 @@ __device__ __forceinline__ void load_bias32(const float* b, float (&x)[32]) {
     x[4 * q + 3] = t.w;
   }
 }
+
 // L2 prefetch of a tile's B operand (the weight side of every product here),
 // issued before pdl_wait so that its DRAM reads overlap the predecessor's
 // tail.  The predecessor never writes it: B holds weights (written by the
@@ -199,6 +202,12 @@ __device__ __forceinline__ uint32_t idesc_major(uint32_t idesc, const GemmProble
 constexpr int kEpiWarps = 8;
 constexpr uint32_t kStageWarpBytes = 4096;
 constexpr uint32_t kStageBytesAll = kEpiWarps * kStageWarpBytes;
+// Columns per step: 64 with the 256-wide tiles (whole 128-byte BF16 lines that
+// leave as TMA stores), 32 with the narrower ones, whose segments the warps store
+// themselves.  Measured at 3 x [8192 x 512] hidden outputs, K = 384 (persistent
+// kernel): 256-wide 25.6 -> 18.9 us with TMA stores, 128-wide 28.6 -> 34.
+template <int BN>
+constexpr int kStepCols = BN == 256 ? 64 : 32;
 
 // Byte offset of the 16-byte chunk `ch` of row `row` in a warp's staging block:
 // rows of 128 bytes (8 chunks) or of 64 bytes (4 chunks), XOR-swizzled so that
@@ -332,69 +341,167 @@ __device__ __forceinline__ void epilogue_grad32(const EpiDesc& e, uint8_t* st, i
   }
 }
 
+// The bias of 32 columns (every lane reads the same 16 bytes; the lines were touched ahead, see touch_bias).
+__device__ __forceinline__ void bias_cols32(const EpiDesc& e, int col0, int N, float (&x)[32]) {
+  if (col0 + 32 <= N) {
+    load_bias32(e.bias + col0, x);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = col0 + i < N ? __ldg(e.bias + col0 + i) : 0.f;
+  }
+}
+
+// ---- TMA stores of staged blocks
+// A staged block (32 rows of 128 bytes, stage128) leaves as one box of the
+// problem's output map: one instruction, no address arithmetic, and the warp
+// goes on while the copy engine writes whole lines.  The map clips rows >= M and
+// columns >= N.
+__device__ __forceinline__ void stage_publish(const CUtensorMap* map, const uint8_t* st, int lane, int x, int y) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // this lane's writes, before the copy reads them
+  __syncwarp();
+  if (lane == 0) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(smem_u32(st)), "r"(x), "r"(y)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  }
+}
+// The warp's earlier stores have read the staging block: it may be written again.
+__device__ __forceinline__ void stage_reclaim(int lane) {
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  __syncwarp();
+}
+
+// 32 columns of an FP32 output.
+__device__ __forceinline__ void epilogue_f32x32(const GemmProblem* P, const EpiDesc& e, uint8_t* st, bool tma, int row0,
+                                                int lane, uint32_t taddr, int col0, int M, int N) {
+  float v[32];
+  switch (e.kind) {
+    case kEpiFwdPreLN:
+    case kEpiFwdOut: {
+      tmem_ldn(taddr, v);
+      float* z = static_cast<float*>(e.out0);
+      float b[32];
+      bias_cols32(e, col0, N, b);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] += b[i];
+      if (tma) {
+        stage_reclaim(lane);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(st + stage128(lane, q)) =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        stage_publish(&P->o0, st, lane, col0, row0);
+      } else if ((e.ld0 & 3) == 0 && (N & 3) == 0) {
+        emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
+          if (row0 + r < M && col0 + k < N) *reinterpret_cast<float4*>(z + (size_t)(row0 + r) * e.ld0 + col0 + k) = x;
+        });
+      } else {
+        emit_f32(st, lane, v, [&](int r, int k, float x) {
+          if (row0 + r < M && col0 + k < N) z[(size_t)(row0 + r) * e.ld0 + col0 + k] = x;
+        });
+      }
+      break;
+    }
+    case kEpiBwdDXLN: {
+      // the masks of the segments this lane will store, in flight during the TMEM read
+      uint2 m[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = row0 + 4 * j + (lane >> 3), c = col0 + 4 * (lane & 7);
+        m[j] = (r < M && c < N) ? *reinterpret_cast<const uint2*>(e.mask + (size_t)r * e.ldm + c) : make_uint2(0u, 0u);
+      }
+      tmem_ldn(taddr, v);
+      float* du = static_cast<float*>(e.out0);
+      emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
+        const uint2 mm = m[(r - (lane >> 3)) / 4];
+        const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&mm.x);
+        const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&mm.y);
+        if (row0 + r < M && col0 + k < N)
+          *reinterpret_cast<float4*>(du + (size_t)(row0 + r) * e.ld0 + col0 + k) =
+              make_float4(__low2float(a) > 0.f ? x.x : 0.f, __high2float(a) > 0.f ? x.y : 0.f,
+                          __low2float(b) > 0.f ? x.z : 0.f, __high2float(b) > 0.f ? x.w : 0.f);
+      });
+      break;
+    }
+    default:
+      tmem_ldn(taddr, v);
+      epilogue_grad32(e, st, row0, lane, v, col0, M, N);
+      break;
+  }
+}
+
+// Eight BF16 hi parts of v (returned), v left as the remainders v - hi.
+__device__ __forceinline__ uint4 split_bf16x8(float* v) {
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    w[i] = *reinterpret_cast<const uint32_t*>(&p);
+    // v - hi, one rounding (two columns per instruction)
+    const float2 r = fma_x2(make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u)),
+                            make_float2(-1.f, -1.f), make_float2(v[2 * i], v[2 * i + 1]));
+    v[2 * i] = r.x;
+    v[2 * i + 1] = r.y;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // One step: NC (32 or 64) columns from col0 of the warp's rows row0 .. row0 + 31.
 // Hidden widths are multiples of 8 (their BF16 rows need 16-byte TMA strides),
 // so an 8-column chunk of a BF16 output lies wholly inside or outside the
 // problem; FP32 rows without 16-byte alignment (odd widths) take 4-byte stores.
 template <int NC>
-__device__ __forceinline__ void epilogue_step(const EpiDesc& e, uint8_t* st, int row0, int lane, uint32_t taddr,
-                                              int col0, int M, int N) {
+__device__ __forceinline__ void epilogue_step(const GemmProblem* P, const EpiDesc& e, uint8_t* st, bool tma, int row0,
+                                              int lane, uint32_t taddr, int col0, int M, int N) {
   using bf16 = __nv_bfloat16;
-  float v[NC];
   switch (e.kind) {
     case kEpiFwdHidden: {
+      float v[NC];
       tmem_ldn(taddr, v);
-      bf16* h = static_cast<bf16*>(e.out0);
 #pragma unroll
       for (int c = 0; c < NC; c += 32) {
         float b[32];
-        if (col0 + c + 32 <= N) {
-          load_bias32(e.bias + col0 + c, b);
-        } else {
+        bias_cols32(e, col0 + c, N, b);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) b[i] = col0 + c + i < N ? __ldg(e.bias + col0 + c + i) : 0.f;
+        for (int i = 0; i < 32; i += 2) {
+          const float2 t = add_x2(make_float2(v[c + i], v[c + i + 1]), make_float2(b[i], b[i + 1]));
+          v[c + i] = fmaxf(t.x, 0.f);
+          v[c + i + 1] = fmaxf(t.y, 0.f);
         }
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[c + i] = fmaxf(v[c + i] + b[i], 0.f);
       }
-      auto put = [&](bf16* base) {
-        emit_bf16<NC>(st, lane, v, [&](int, int r, int c, uint4 x) {
-          if (row0 + r < M && col0 + c < N)
-            *reinterpret_cast<uint4*>(base + (size_t)(row0 + r) * e.ld0 + col0 + c) = x;
-        });
-      };
-      put(h);
+      if constexpr (NC == 64) {
+        // hi block, then lo block, each leaving as one TMA store
+        stage_reclaim(lane);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) v[i] -= __bfloat162float(__float2bfloat16_rn(v[i]));
-      put(h + e.c0);
-      break;
-    }
-    case kEpiFwdPreLN:
-    case kEpiFwdOut: {
-      tmem_ldn(taddr, v);
-      float* z = static_cast<float*>(e.out0);
-      const bool vec = (e.ld0 & 3) == 0 && (N & 3) == 0;
+        for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4*>(st + stage128(lane, q)) = split_bf16x8(v + 8 * q);
+        stage_publish(&P->o0, st, lane, col0, row0);
+        uint4 w[8];
 #pragma unroll
-      for (int c = 0; c < NC; c += 32) {
-        if (col0 + c >= N) break;
-        float b[32];
-        if (col0 + c + 32 <= N) {
-          load_bias32(e.bias + col0 + c, b);
-        } else {
+        for (int q = 0; q < 8; ++q) w[q] = pack_bf16x8(v + 8 * q);
+        stage_reclaim(lane);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) b[i] = col0 + c + i < N ? __ldg(e.bias + col0 + c + i) : 0.f;
+        for (int q = 0; q < 8; ++q) *reinterpret_cast<uint4*>(st + stage128(lane, q)) = w[q];
+        stage_publish(&P->o1, st, lane, col0, row0);
+      } else {
+        // narrow tiles: hi and lo halves of a row side by side in the staging block, 64-byte segments
+        bf16* h = static_cast<bf16*>(e.out0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          *reinterpret_cast<uint4*>(st + stage128(lane, q)) = split_bf16x8(v + 8 * q);
+          *reinterpret_cast<uint4*>(st + stage128(lane, 4 + q)) = pack_bf16x8(v + 8 * q);
         }
+        __syncwarp();
+        const int ch = lane & 7, c = 8 * (ch & 3);
+        bf16* base = h + (ch < 4 ? 0 : e.c0) + col0 + c;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[c + i] += b[i];
-        if (vec)
-          emit_f32x4(st, lane, v + c, [&](int r, int k, float4 x) {
-            if (row0 + r < M && col0 + c + k < N)
-              *reinterpret_cast<float4*>(z + (size_t)(row0 + r) * e.ld0 + col0 + c + k) = x;
-          });
-        else
-          emit_f32(st, lane, v + c, [&](int r, int k, float x) {
-            if (row0 + r < M && col0 + c + k < N) z[(size_t)(row0 + r) * e.ld0 + col0 + c + k] = x;
-          });
+        for (int j = 0; j < 8; ++j) {
+          const int r = 4 * j + (lane >> 3);
+          const uint4 x = *reinterpret_cast<const uint4*>(st + stage128(r, ch));
+          if (row0 + r < M && col0 + c < N) *reinterpret_cast<uint4*>(base + (size_t)(row0 + r) * e.ld0) = x;
+        }
+        __syncwarp();
       }
       break;
     }
@@ -409,6 +516,7 @@ __device__ __forceinline__ void epilogue_step(const EpiDesc& e, uint8_t* st, int
         m[j] = (r < M && mc < N) ? *reinterpret_cast<const uint4*>(e.mask + (size_t)r * e.ldm + mc)
                                  : make_uint4(0u, 0u, 0u, 0u);
       }
+      float v[NC];
       tmem_ldn(taddr, v);
       bf16* dz = static_cast<bf16*>(e.out0);
       emit_bf16<NC>(st, lane, v, [&](int j, int r, int c, uint4 x) {
@@ -419,36 +527,13 @@ __device__ __forceinline__ void epilogue_step(const EpiDesc& e, uint8_t* st, int
       });
       break;
     }
-    case kEpiBwdDXLN: {
-      uint2 m[NC / 4];
-#pragma unroll
-      for (int j = 0; j < NC / 4; ++j) {
-        const int r = row0 + 4 * (j & 7) + (lane >> 3), c = col0 + 32 * (j >> 3) + 4 * (lane & 7);
-        m[j] = (r < M && c < N) ? *reinterpret_cast<const uint2*>(e.mask + (size_t)r * e.ldm + c) : make_uint2(0u, 0u);
-      }
-      tmem_ldn(taddr, v);
-      float* du = static_cast<float*>(e.out0);
-#pragma unroll
-      for (int c = 0; c < NC; c += 32) {
-        int j = c / 4;
-        emit_f32x4(st, lane, v + c, [&](int r, int k, float4 x) {
-          const uint2 mm = m[j++];
-          const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&mm.x);
-          const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&mm.y);
-          if (row0 + r < M && col0 + c + k < N)
-            *reinterpret_cast<float4*>(du + (size_t)(row0 + r) * e.ld0 + col0 + c + k) =
-                make_float4(__low2float(a) > 0.f ? x.x : 0.f, __high2float(a) > 0.f ? x.y : 0.f,
-                            __low2float(b) > 0.f ? x.z : 0.f, __high2float(b) > 0.f ? x.w : 0.f);
-        });
-      }
+    default: {
+      // FP32 outputs, 32 columns at a time
+#pragma unroll 1
+      for (int c = 0; c < NC && col0 + c < N; c += 32)
+        epilogue_f32x32(P, e, st, tma, row0, lane, taddr + c, col0 + c, M, N);
       break;
     }
-    default:
-      tmem_ldn(taddr, v);
-#pragma unroll
-      for (int c = 0; c < NC; c += 32)
-        if (col0 + c < N) epilogue_grad32(e, st, row0, lane, v + c, col0 + c, M, N);
-      break;
   }
 }
 
@@ -499,8 +584,8 @@ __device__ __forceinline__ void epilogue_energy(const EpiDesc& e, uint8_t* st, i
 // The warp's share of a 128 x BN tile at (m0, n0), accumulator at `acc`: rows
 // m0 + 32 eg .., every second step of NC columns.
 template <int BN, int NC>
-__device__ __forceinline__ void epilogue_tile(const EpiDesc& e, uint8_t* st, uint32_t acc, int eg, int half, int lane,
-                                              int m0, int n0, int M, int N) {
+__device__ __forceinline__ void epilogue_tile(const GemmProblem* P, const EpiDesc& e, uint8_t* st, uint32_t acc, int eg,
+                                              int half, int lane, int m0, int n0, int M, int N) {
   static_assert(BN % (2 * NC) == 0, "two half warps share the tile's steps");
   const int row0 = m0 + 32 * eg;
   if (row0 >= M) return;
@@ -510,8 +595,32 @@ __device__ __forceinline__ void epilogue_tile(const EpiDesc& e, uint8_t* st, uin
     return;
   }
   const int ncol = (N - n0 < BN) ? N - n0 : BN;
+  const bool tma = NC == 64 && P->tma_out != 0;
 #pragma unroll 1
-  for (int c = NC * half; c < ncol; c += 2 * NC) epilogue_step<NC>(e, st, row0, lane, lane_base + c, n0 + c, M, N);
+  for (int c = NC * half; c < ncol; c += 2 * NC)
+    epilogue_step<NC>(P, e, st, tma, row0, lane, lane_base + c, n0 + c, M, N);
+}
+
+// Before the accumulator is ready: the bias lines of the warp's columns into L1
+// (a first touch costs an L2 round trip that would otherwise stand in every
+// tile's epilogue), and the tensor-map proxy's view of the output maps.
+template <int BN, int NC>
+__device__ __forceinline__ void epilogue_ahead(const GemmProblem* P, int half, int lane, int n0) {
+  if (P->epi.bias != nullptr && 4 * lane < BN / 2) {
+    const int k = 4 * lane, c = n0 + NC * half + 2 * NC * (k / NC) + k % NC;   // the warp's k-th column
+    if (c < P->N) {
+      float x;
+      asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(P->epi.bias + c));
+    }
+  }
+  if (NC == 64 && lane == 0 && P->tma_out) {
+    tmap_acquire(&P->o0);
+    if (P->epi.kind == kEpiFwdHidden) tmap_acquire(&P->o1);
+  }
+}
+// After the warp's last tile: its stores have read the staging block.
+__device__ __forceinline__ void epilogue_end(int lane) {
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // nkA > 0: A has only nkA K-slices and slice kb of B multiplies slice kb % nkA of
@@ -546,6 +655,7 @@ __global__ void __launch_bounds__(kTileThreads, (GemmSmem<BN, STAGES>::kBytes <=
   const int m0 = (lt / P->tiles_n) * kBM, n0 = (lt % P->tiles_n) * BN;
   const CUtensorMap* tmA = &P->a;
   const CUtensorMap* tmB = &P->b;
+  const EpiDesc e = P->epi;   // (immutable: read ahead of the predecessor's end, not at the epilogue's start)
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nk_all = (K + kBK - 1) / kBK;
@@ -622,9 +732,11 @@ __global__ void __launch_bounds__(kTileThreads, (GemmSmem<BN, STAGES>::kBytes <=
   // epilogue (tcgen05.ld is warp-collective: keep the decision warp-uniform).
   // Every MMA has completed, so the operand ring is free: it becomes the warps'
   // staging blocks.
+  const int eg = warp & 3, half = warp >> 2;
+  constexpr int NC = kStepCols<BN>;
+  epilogue_ahead<BN, NC>(P, half, lane, n0);
   const bool ok = __all_sync(0xffffffffu, mbar_wait(done, 0, lim) ? 1 : 0) != 0;
   fence_after_sync();
-  const int eg = warp & 3, half = warp >> 2;
   uint8_t* stage = smem + warp * kStageWarpBytes;
   if (ok && ksplit > 1) {
     // split-K: store this split's FP32 partial tile; the last CTA of the tile to
@@ -633,7 +745,6 @@ __global__ void __launch_bounds__(kTileThreads, (GemmSmem<BN, STAGES>::kBytes <=
     // partial is [BN / 4][128 rows] 16-byte pieces: a warp's accesses are
     // contiguous (row-major partials cost 32 lines per instruction both ways).
     __shared__ int s_last;
-    const EpiDesc e = P->epi;
     const int r = eg * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(eg * 32) << 16);
     const int ncol = (N - n0 < BN) ? N - n0 : BN;
@@ -675,8 +786,8 @@ __global__ void __launch_bounds__(kTileThreads, (GemmSmem<BN, STAGES>::kBytes <=
       if (threadIdx.x == 0) P->tickets[lt] = 0u;
     }
   } else if (ok) {
-    const EpiDesc e = P->epi;
-    epilogue_tile<BN, 32>(e, stage, tmem, eg, half, lane, m0, n0, M, N);
+    epilogue_tile<BN, NC>(P, e, stage, tmem, eg, half, lane, m0, n0, M, N);
+    if (NC == 64) epilogue_end(lane);
   } else if (threadIdx.x == 0) {
     atomicOr(status, CRL_STATUS_TIMEOUT);
   }
@@ -821,28 +932,31 @@ __global__ void __launch_bounds__(kPersistentThreads, 1)
     }
   } else {
     // epilogue warps (tcgen05.ld is warp-collective: decisions stay warp-uniform)
-    constexpr int NC = BN >= 128 ? 64 : 32;
+    constexpr int NC = kStepCols<BN>;
     const int eg = warp & 3, ew = warp - 2, half = ew >> 2;
     int i = 0;
     for (int t = blockIdx.x; t < total; t += gridDim.x, ++i) {
       const int buf = i & 1, use = i >> 1;
+      // everything the epilogue reads of its problem, before the accumulator is ready
+      const GemmProblem* P = find_problem(probs, nprob, t);
+      const int lt = t - P->tile_begin;
+      const int m0 = (lt / P->tiles_n) * kBM, n0 = (lt % P->tiles_n) * BN;
+      const int M = P->M, N = P->N;
+      const EpiDesc& e = P->epi;   // fields read where used (L1): the steps need the registers
+      epilogue_ahead<BN, NC>(P, half, lane, n0);
       const bool ok = __all_sync(0xffffffffu, mbar_wait(&accf[buf], use & 1, lim) ? 1 : 0) != 0;
       if (!ok) {
         if (lane == 0) atomicOr(status, CRL_STATUS_TIMEOUT);
         break;
       }
       fence_after_sync();
-      const GemmProblem* P = find_problem(probs, nprob, t);
-      const int lt = t - P->tile_begin;
-      const int m0 = (lt / P->tiles_n) * kBM, n0 = (lt % P->tiles_n) * BN;
-      const int M = P->M, N = P->N;
-      const EpiDesc e = P->epi;
-      epilogue_tile<BN, NC>(e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
+      epilogue_tile<BN, NC>(P, e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
       // release the buffer to the MMA issuer
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce[buf]);
     }
+    if (NC == 64) epilogue_end(lane);
   }
   // no MMA may still write the accumulators when they are freed
   if (threadIdx.x == 0) mbar_wait(drain, 0, kDrainLimitNs);
@@ -863,9 +977,11 @@ __global__ void __launch_bounds__(kPersistentThreads, 1)
 //   warp 1 / lane 0 -- even CTA: MMA issuer (waits for its own slot and the
 //                      odd CTA's `pfull` arrival); odd CTA: reports each
 //                      landed slot to the even CTA's `pfull`;
-//   warp 2 / lane 0 -- even CTA: passes each freed slot (`empty`) and each
-//                      finished accumulator (`accf`) on to the odd CTA;
-//   warps 4..11     -- epilogue of this CTA's 128 rows from TMEM buffer i % 2;
+//                      its commits free each slot (`empty`) and announce each
+//                      finished accumulator (`accf`) in both CTAs at once (a
+//                      relay warp cost about 0.5 us per slot: more than one
+//                      slot's MMA time);
+//   warps 2..9      -- epilogue of this CTA's 128 rows from TMEM buffer i % 2;
 //                      the pair's sixteen warps release it on the even CTA's `acce`.
 // The epilogue is the one-tile kernel's, so every kernel gives identical outputs
 // where the MMA sums each K = 16 slice the same way.
@@ -875,10 +991,11 @@ struct GemmPairSmem {
   static constexpr uint32_t kBBytes = (BN / 2) * kBK * 2;    // this CTA's BN / 2 rows of B
   static constexpr uint32_t kStageBytes = kABytes + kBBytes;
   static constexpr int kStages = STAGES;
-  // ring + barriers (full, empty, pfull [S]; accf, acce [2]; drain) + TMEM slot, plus 1 KiB for
-  // alignment and one more B half behind the ring, so that the last slot's B rows plus BN / 2
-  // rows stay inside this CTA's shared memory; then the epilogue's staging blocks
-  static constexpr uint32_t kBytes = kStages * kStageBytes + kBBytes + 8 * 4096 + 1024 + 512;
+  // ring, the epilogue's staging blocks, barriers (full, empty, pfull [S]; accf, acce [2]; drain) +
+  // TMEM slot, plus 1 KiB for alignment (the last slot's B rows plus BN / 2 rows stay inside this
+  // CTA's shared memory)
+  static constexpr uint32_t kBytes = kStages * kStageBytes + 8 * 4096 + 1024 + 512;
+  static_assert(kBBytes <= 8 * 4096, "the staging blocks cover one more B half behind the ring");
   static constexpr uint32_t kTmemCols = 2 * BN;   // two accumulator buffers
   static_assert(BN == 128 || BN == 256, "pair tiles are 256 x 128 or 256 x 256");
   static_assert(kTmemCols <= 512, "TMEM columns");
@@ -894,7 +1011,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   uint8_t* sA = smem;
   uint8_t* sB = smem + S::kStages * S::kABytes;
-  uint8_t* sE = smem + S::kStages * S::kStageBytes + S::kBBytes;   // epilogue staging, 4 KiB per warp
+  uint8_t* sE = smem + S::kStages * S::kStageBytes;   // epilogue staging, 4 KiB per warp
   uint64_t* full = reinterpret_cast<uint64_t*>(sE + kStageBytesAll);
   uint64_t* empty = full + S::kStages;
   uint64_t* pfull = empty + S::kStages;  // even CTA: the odd CTA's slot has landed
@@ -1000,9 +1117,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
             mma_bf16_pair(d, da + sa * k, db + sb * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          mma_commit_pair(&empty[s]);
+          mma_commit_both(&empty[s]);
         }
-        if (ok) mma_commit_pair(&accf[buf]);
+        if (ok) mma_commit_both(&accf[buf]);
       }
       mma_commit_pair(drain);   // completes once every MMA issued above has
     } else if (lane == 0) {
@@ -1023,42 +1140,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         }
       }
     }
-  } else if (warp == 2) {
-    if (lane == 0 && even) {
-      // relay of the even CTA: every completed MMA slice frees the odd CTA's
-      // slot too, and every completed tile its accumulator rows (a thread of
-      // its own, so that no cluster-scope release waits behind the producer's
-      // copies or the epilogue's stores)
-      int it = 0, i = 0;
-      bool ok = true;
-      for (int t = cl; t < total && ok; t += ncl, ++i) {
-        const GemmProblem* P = find_problem(probs, nprob, t);
-        const int nk = (P->K + kBK - 1) / kBK;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const int s = it % S::kStages;
-          if (!mbar_wait(&empty[s], (it / S::kStages) & 1, lim)) {
-            atomicOr(status, CRL_STATUS_TIMEOUT);
-            ok = false;
-            break;
-          }
-          mbar_arrive_remote(mapa_shared(&empty[s], 1));
-        }
-        if (!ok) break;
-        const int buf = i & 1, use = i >> 1;
-        if (!mbar_wait(&accf[buf], use & 1, lim)) {
-          atomicOr(status, CRL_STATUS_TIMEOUT);
-          break;
-        }
-        mbar_arrive_remote(mapa_shared(&accf[buf], 1));
-      }
-    }
-  } else if (warp >= 4) {
+  } else {
     // epilogue warps: this CTA's 128 rows of the pair's tile
-    constexpr int NC = 64;
-    const int eg = warp & 3, ew = warp - 4, half = ew >> 2;
+    constexpr int NC = kStepCols<BN>;
+    const int eg = warp & 3, ew = warp - 2, half = ew >> 2;
     int i = 0;
     for (int t = cl; t < total; t += ncl, ++i) {
       const int buf = i & 1, use = i >> 1;
+      // everything the epilogue reads of its problem, before the accumulator is ready
+      const GemmProblem* P = find_problem(probs, nprob, t);
+      const int lt = t - P->tile_begin;
+      const int m0 = (lt / P->tiles_n) * kPairM + kBM * (int)rank, n0 = (lt % P->tiles_n) * BN;
+      const int M = P->M, N = P->N;
+      const EpiDesc& e = P->epi;   // fields read where used (L1): the steps need the registers
+      epilogue_ahead<BN, NC>(P, half, lane, n0);
       const bool got = even ? mbar_wait(&accf[buf], use & 1, lim) : mbar_wait_cluster(&accf[buf], use & 1, lim);
       const bool ok = __all_sync(0xffffffffu, got ? 1 : 0) != 0;
       if (!ok) {
@@ -1066,12 +1161,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         break;
       }
       fence_after_sync();
-      const GemmProblem* P = find_problem(probs, nprob, t);
-      const int lt = t - P->tile_begin;
-      const int m0 = (lt / P->tiles_n) * kPairM + kBM * (int)rank, n0 = (lt % P->tiles_n) * BN;
-      const int M = P->M, N = P->N;
-      const EpiDesc e = P->epi;
-      epilogue_tile<BN, NC>(e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
+      epilogue_tile<BN, NC>(P, e, sE + ew * kStageWarpBytes, tmem + (uint32_t)(buf * BN), eg, half, lane, m0, n0, M, N);
       // release the buffer to the MMA issuer
       fence_before_sync();
       __syncwarp();
@@ -1080,6 +1170,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         else mbar_arrive_remote(mapa_shared(&acce[buf], 0));
       }
     }
+    if (NC == 64) epilogue_end(lane);
   }
   // teardown: no MMA may still write either CTA's accumulators when they are
   // freed, and no remote arrival may reach a CTA that has left

@@ -50,5 +50,21 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t inner, uint64_t
   return true;
 }
 
+bool make_tmap_store(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint64_t row_stride_elems,
+                     bool fp32) {
+  std::call_once(g_once, load_entry_point);
+  const uint64_t es = fp32 ? 4 : 2;
+  memset(map, 0, sizeof(*map));   // the map's bytes key the grouped-GEMM table cache
+  if (!g_encode || (reinterpret_cast<uintptr_t>(base) & 15) != 0 || (row_stride_elems * es) % 16 != 0) return false;
+  const cuuint64_t dims[2] = {inner, rows};
+  const cuuint64_t strides[1] = {row_stride_elems * es};
+  const cuuint32_t box[2] = {fp32 ? 32u : 64u, 32u};
+  const cuuint32_t estride[2] = {1, 1};
+  return g_encode(map, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                  const_cast<void*>(base), dims, strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tc
 }  // namespace crl
