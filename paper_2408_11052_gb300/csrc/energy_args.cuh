@@ -94,7 +94,8 @@ struct BwdArgs {
 
 struct HCoef {
   float a_own;    // own auxiliary (|x|^2 for the L2 energies)
-  float l_own2;   // own logsumexp x log2(e)
+  float l_own;    // own logsumexp
+  float l_own2;   // the same x log2(e)
   float k_own;    // scale (w_own + 2 beta p_own l_own)
   float k_own_tau;  // k_own / tau
   float k_diag;   // scale (w_f + w_b): the positive pair's -1 terms

@@ -570,6 +570,7 @@ __device__ __forceinline__ void fwd_body(const CUtensorMap* tmX, const CUtensorM
     const float dpair = anchored ? s_d[r] : 0.f;
     float row_m = -INFINITY, row_s = 0.f;   // this row's running (max, sum) over the chunk, log2 units
     float vp = 0.f, kp = 0.f;               // objective partials of this row
+    float ay_next = t0 * kTile + q * 32 + lane < a.B ? __ldg(a.auxY + t0 * kTile + q * 32 + lane) : 0.f;
     bool good = true;
     for (int t = 0; t < nt; ++t) {
       const int b = t & 1;
@@ -593,15 +594,21 @@ __device__ __forceinline__ void fwd_body(const CUtensorMap* tmX, const CUtensorM
       const int jn = row_ok ? min(32, a.B - jb) : 0;
       float ay[32];
       {
-        const float4* a4 = reinterpret_cast<const float4*>(a.auxY + jb);
+        // the columns' auxiliaries, loaded a tile ahead (one per lane) and handed
+        // round through this warp's block (free between tiles)
+        blk[lane] = ay_next;
+        const int jn1 = jb + kTile + lane;
+        ay_next = (t + 1 < nt && jn1 < a.B) ? __ldg(a.auxY + jn1) : 0.f;
+        __syncwarp();
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const float4 x = (jb + 4 * k < a.B) ? __ldg(a4 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 x = reinterpret_cast<const float4*>(blk)[k];
           ay[4 * k] = x.x;
           ay[4 * k + 1] = x.y;
           ay[4 * k + 2] = x.z;
           ay[4 * k + 3] = x.w;
         }
+        __syncwarp();
       }
       float m, mn;
       const bool full = i0 + kTile <= a.B && j0 + kTile <= a.B;
@@ -819,146 +826,276 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   return y;
 }
 
-// NC consecutive columns cb .. cb + NC - 1 of the tile (NC = 16 or 32).  The
-// other side's per-column inputs come from global memory (every lane reads the
-// same 16 bytes: L1 broadcasts): aux_o = its auxiliaries, lse_o = its
-// logsumexps (LIVE != 1), with k_oth = kb_oth + k2_oth * lse.
-template <int EK, int OBJ, int LIVE, bool EDGE, int NC>
-__device__ __forceinline__ void build_h(const float (&sv)[NC], const HCoef& hc, const float* __restrict__ aux_o,
-                                        const float* __restrict__ lse_o, float kb_oth, float k2_oth, int cb, int u,
-                                        int v0, int B, float& rowsum, uint32_t (&packed)[NC / 2]) {
-  // the per-column inputs of four columns at a time, the next group's loads
-  // issued before this group's arithmetic
-  float cax[4], clse[4], ckoth[4], nax[4] = {0.f, 0.f, 0.f, 0.f}, nlse[4] = {0.f, 0.f, 0.f, 0.f};
-  auto load4 = [&](int k, float (&ax)[4], float (&ls)[4]) {
-    const int c4 = v0 + cb + k;
-    if (EDGE) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const bool in = c4 + e < B;
-        if (EK != 2) ax[e] = in ? __ldg(aux_o + c4 + e) : 0.f;
-        if (LIVE != 1) ls[e] = in ? __ldg(lse_o + c4 + e) : 0.f;
-      }
-    } else {
-      if (EK != 2) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(aux_o + c4));
-        ax[0] = t.x, ax[1] = t.y, ax[2] = t.z, ax[3] = t.w;
-      }
-      if (LIVE != 1) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(lse_o + c4));
-        ls[0] = t.x, ls[1] = t.y, ls[2] = t.z, ls[3] = t.w;
-      }
-    }
-  };
-  load4(0, nax, nlse);
-#pragma unroll
-  for (int k = 0; k < NC; k += 2) {
-    if ((k & 3) == 0) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        cax[e] = nax[e];
-        clse[e] = nlse[e];
-      }
-      if (k + 4 < NC) load4(k + 4, nax, nlse);
-      if (LIVE != 1) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          ckoth[e] = fmaf(k2_oth, clse[e], kb_oth);
-          clse[e] *= kLog2e;
-        }
-      }
-    }
-    float h2[2];
-    if constexpr (EK == 0 && LIVE != 0 && !EDGE && OBJ == kObjInfo) {
-      // the common case (-L2, one live softmax term, interior tile, InfoNCE),
-      // both columns of the pair at once: h = 2^(-k1 d - l2) k / (tau d), with
-      // k / tau per row or per column
-      const int c = k & 3;
-      const float2 t2 = fma_x2(make_float2(-2.f, -2.f), make_float2(sv[k], sv[k + 1]),
-                               make_float2(hc.a_own + cax[c], hc.a_own + cax[c + 1]));
-      const float t0 = fmaxf(t2.x, 0.f), t1 = fmaxf(t2.y, 0.f);
-      const float2 rs = make_float2(t0 >= 1e-24f ? rsqrt_approx(t0) : 0.f, t1 >= 1e-24f ? rsqrt_approx(t1) : 0.f);
-      const float2 d = mul_x2(make_float2(t0, t1), rs);
-      float2 arg, fac;
-      if (LIVE == 1) {
-        arg = fma_x2(make_float2(-hc.k1, -hc.k1), d, make_float2(-hc.l_own2, -hc.l_own2));
-        fac = mul_x2(make_float2(hc.k_own_tau, hc.k_own_tau), rs);
-      } else {
-        arg = fma_x2(make_float2(-hc.k1, -hc.k1), d, make_float2(-clse[c], -clse[c + 1]));
-        fac = mul_x2(make_float2(ckoth[c] * hc.inv_tau, ckoth[c + 1] * hc.inv_tau), rs);
-      }
-      const float2 hv = mul_x2(make_float2(ex2(arg.x), ex2(arg.y)), fac);
-      h2[0] = hv.x;
-      h2[1] = hv.y;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int cl = cb + k + e;
-        const int v = v0 + cl;
-        const int c = (k & 3) + e;
-        const float sval = sv[k + e];
-        float f2, fac;
-        if (EK == 0) {
-          const float t = fmaxf(fmaf(-2.f, sval, hc.a_own + cax[c]), 0.f);
-          const float rs = t >= 1e-24f ? rsqrt_approx(t) : 0.f;
-          f2 = -(t * rs) * hc.k1;
-          fac = hc.inv_tau * rs;
-        } else if (EK == 1) {
-          const float t = fmaxf(fmaf(-2.f, sval, hc.a_own + cax[c]), 0.f);
-          f2 = -t * hc.k1;
-          fac = 2.f * hc.inv_tau;
-        } else {
-          f2 = sval * hc.k1;
-          fac = hc.inv_tau;
-        }
-        float g;
-        if (LIVE == 1) g = ex2(f2 - hc.l_own2) * hc.k_own;
-        else if (LIVE == 2) g = ex2(f2 - clse[c]) * ckoth[c];
-        else g = fmaf(ex2(f2 - hc.l_own2), hc.k_own, ex2(f2 - clse[c]) * ckoth[c]);
-        if (EDGE && u == v) g -= hc.k_diag;
-        if (OBJ != kObjInfo) {
-          const float d_row = hc.transposed ? (v < B ? __ldg(hc.dpre + v) : 0.f) : hc.d_own;
-          const float k_row = hc.transposed ? (v < B ? __ldg(hc.kd + v) : 0.f) : hc.kd_own;
-          g += objective_coef<OBJ>(f2, EDGE && u == v, d_row, k_row, hc);
-        }
-        h2[e] = (!EDGE || (u < B && v < B)) ? g * fac : 0.f;
-      }
-    }
-    const __nv_bfloat162 p2 = __floats2bfloat162_rn(h2[0], h2[1]);
-    // the row sum takes the BF16-rounded coefficients the MMA multiplies, so
-    // acc - rowsum * own stays a sum of H (other - own) terms
+// Per-column inputs of 16 columns, staged in shared memory (every lane reads the
+// same 16 bytes): [0, 16) the other side's auxiliaries, [16, 32) minus its
+// logsumexps (x log2(e) for kFoldTau), [32, 48) k_oth = kb_oth + k2_oth lse (x 1 / tau for kFoldTau).
+constexpr int kCinFloats = 48;
+// The interior -L2 tile with only the other side's term folds 1 / tau into k_oth.
+template <int EK, int OBJ, int LIVE, bool EDGE>
+constexpr bool kFoldTau = EK == 0 && OBJ == kObjInfo && LIVE == 2 && !EDGE;
+
+// Whether F log2(e) is rounded before the other side's logsumexp is taken from it
+// (else the product and the subtraction are one fused operation).
+template <int EK, int OBJ, int LIVE>
+constexpr bool kRoundOther = LIVE == 0 || OBJ != kObjInfo || (EK == 0 && LIVE == 2);
+
+// The smallest of 16 values, NaN if any is NaN (three-input minimum).
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+// Columns k, k + 1 of a staged array, read 16 bytes at a time (the compiler shares the load of a group of four).
+__device__ __forceinline__ float2 half_of(const float* p, int k) {
+  const float4 t = *reinterpret_cast<const float4*>(p + (k & ~3));
+  return (k & 2) ? make_float2(t.z, t.w) : make_float2(t.x, t.y);
+}
+
+// 16 consecutive columns cb .. cb + 15 of the tile.
+template <int EK, int OBJ, int LIVE, bool EDGE>
+__device__ __forceinline__ void build_h(const float (&sv)[16], const HCoef& hc, const float* __restrict__ cin, int cb,
+                                        int u, int v0, int B, float& rowsum, uint32_t (&packed)[8]) {
+  // the row sum takes the BF16-rounded coefficients the MMA multiplies, so
+  // acc - rowsum * own stays a sum of H (other - own) terms
+  auto put = [&](int k, float2 h) {
+    const __nv_bfloat162 p2 = __floats2bfloat162_rn(h.x, h.y);
     rowsum += __low2float(p2) + __high2float(p2);
     packed[k / 2] = *reinterpret_cast<const uint32_t*>(&p2);
+  };
+  if constexpr (EK == 0 && !EDGE && OBJ == kObjInfo) {
+    // interior -L2 tile of the InfoNCE family: t = d^2 of both columns of a pair
+    // per instruction
+    float t[16];
+    float mn = INFINITY;
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      const float2 ax = half_of(cin, k);
+      const float2 t2 = fma_x2(make_float2(-2.f, -2.f), make_float2(sv[k], sv[k + 1]),
+                               add_x2(make_float2(hc.a_own, hc.a_own), ax));
+      t[k] = t2.x;
+      t[k + 1] = t2.y;
+      mn = min3_nan(mn, t2.x, t2.y);
+    }
+    // No pair coincides (d^2 >= 1e-24, the rule): neither the clamp at 0 nor the
+    // zero coefficient of coincident pairs applies, and the loop drops both tests
+    // (3 of about 10 operations per element).  Warp-uniform.
+    float r[16];
+    if (__all_sync(0xffffffffu, mn >= 1e-24f)) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) r[k] = rsqrt_approx(t[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        t[k] = fmaxf(t[k], 0.f);
+        const float q = rsqrt_approx(t[k]);
+        r[k] = t[k] >= 1e-24f ? q : 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      const float2 rs = make_float2(r[k], r[k + 1]);
+      const float2 d = mul_x2(make_float2(t[k], t[k + 1]), rs);
+      const float2 nk1 = make_float2(-hc.k1, -hc.k1);
+      float2 e_own, e_oth;
+      if (LIVE == 1) {
+        const float2 arg = fma_x2(nk1, d, make_float2(-hc.l_own2, -hc.l_own2));
+        e_own = make_float2(ex2(arg.x), ex2(arg.y));
+      } else if (LIVE == 2) {
+        const float2 arg = fma_x2(nk1, d, half_of(cin + 16, k));
+        e_oth = make_float2(ex2(arg.x), ex2(arg.y));
+      } else {
+        const float2 f2 = mul_x2(nk1, d);   // rounded once for both terms
+        const float2 a = add_x2(f2, make_float2(-hc.l_own2, -hc.l_own2));
+        const float2 b = fma_x2(half_of(cin + 16, k), make_float2(kLog2e, kLog2e), f2);
+        e_own = make_float2(ex2(a.x), ex2(a.y));
+        e_oth = make_float2(ex2(b.x), ex2(b.y));
+      }
+      float2 h;
+      if (LIVE == 1) {
+        h = mul_x2(e_own, mul_x2(make_float2(hc.k_own_tau, hc.k_own_tau), rs));
+      } else if (LIVE == 2) {
+        h = mul_x2(e_oth, mul_x2(half_of(cin + 32, k), rs));
+      } else {
+        const float2 g = fma_x2(e_own, make_float2(hc.k_own, hc.k_own), mul_x2(e_oth, half_of(cin + 32, k)));
+        h = mul_x2(g, mul_x2(make_float2(hc.inv_tau, hc.inv_tau), rs));
+      }
+      put(k, h);
+    }
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) {
+    float h2[2];
+    const float2 cax = EK != 2 ? half_of(cin, k) : make_float2(0.f, 0.f);
+    const float2 cl2 = LIVE != 1 ? half_of(cin + 16, k) : make_float2(0.f, 0.f);
+    const float2 cko = LIVE != 1 ? half_of(cin + 32, k) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int v = v0 + cb + k + e;
+      const float sval = sv[k + e];
+      float fa, fac;   // F log2(e) = fa k1
+      if (EK == 0) {
+        const float t = fmaxf(fmaf(-2.f, sval, hc.a_own + (e ? cax.y : cax.x)), 0.f);
+        const float q = rsqrt_approx(t);
+        const float rs = t >= 1e-24f ? q : 0.f;
+        fa = -(t * rs);
+        fac = hc.inv_tau * rs;
+      } else if (EK == 1) {
+        const float t = fmaxf(fmaf(-2.f, sval, hc.a_own + (e ? cax.y : cax.x)), 0.f);
+        fa = -t;
+        fac = 2.f * hc.inv_tau;
+      } else {
+        fa = sval;
+        fac = hc.inv_tau;
+      }
+      const float nl = e ? cl2.y : cl2.x, ko = e ? cko.y : cko.x;
+      float g;
+      // F log2(e) - l log2(e), with the roundings spelled out (one fused operation where F is
+      // used once, else F rounded first; a contraction left to the compiler changes with the code around it)
+      const float f2 = __fmul_rn(fa, hc.k1);
+      const float xo = OBJ != kObjInfo ? fmaf(-hc.l_own, kLog2e, f2)
+                       : LIVE == 0     ? __fadd_rn(f2, -hc.l_own2)
+                                       : fmaf(fa, hc.k1, -hc.l_own2);
+      const float xt = kRoundOther<EK, OBJ, LIVE> ? fmaf(nl, kLog2e, f2) : fmaf(fa, hc.k1, -__fmul_rn(-nl, kLog2e));
+      if (LIVE == 1) g = ex2(xo) * hc.k_own;
+      else if (LIVE == 2) g = ex2(xt) * ko;
+      else g = fmaf(ex2(xo), hc.k_own, ex2(xt) * ko);
+      if (EDGE && u == v) g -= hc.k_diag;
+      if (OBJ != kObjInfo) {
+        const float d_row = hc.transposed ? (v < B ? __ldg(hc.dpre + v) : 0.f) : hc.d_own;
+        const float k_row = hc.transposed ? (v < B ? __ldg(hc.kd + v) : 0.f) : hc.kd_own;
+        g += objective_coef<OBJ>(f2, EDGE && u == v, d_row, k_row, hc);
+      }
+      h2[e] = (!EDGE || (u < B && v < B)) ? g * fac : 0.f;
+    }
+    put(k, make_float2(h2[0], h2[1]));
   }
 }
 
 // lb in [0, 2 nrow): the row pass for lb < nrow, else the column pass.
 //
-// 18 warps.  Warp 16 lane 0 loads the own tile once and the other side's tiles
+// 19 warps.  Warp 16 lane 0 loads the own tile once and the other side's tiles
 // into two buffers (tile v into buffer v % 2 once the MMAs of tile v - 2 are
-// done with it).  Warp 17 lane 0 issues the MMAs in whatever order their inputs
-// allow (polling): S(v) = own . other(v)^T into TMEM accumulator v % 2 once
-// tile v has landed and the builders have read S(v - 2), and the two halves of
-// acc += H(v) other(v) (K = 64 rows of the other tile each) as the builders
-// publish them.  The 16 builder warps turn S(v) into the BF16 coefficient tile
-// H one 64-column half at a time (warp w: rows 32 (w % 4) .., 16 columns of each
-// half): the accumulation of one half runs while the next half (or the next
-// tile's first half) is built, and S(v + 1) is ready before H(v) is done.
+// done with it).  Warp 17 lane 0 issues S(v) = own . other(v)^T into TMEM
+// accumulator v % 2 once tile v has landed and the builders have read S(v - 2);
+// warp 18 lane 0 issues the two halves of acc += H(v) other(v) (K = 64 rows of the
+// other tile each) as the builders publish them.  (One issuer that polled both
+// kinds of input had to sleep between polls to leave the builders their issue
+// slots; the sleep stood in the loop acc(v) -> buffer free -> tile v + 2 -> S(v + 2).)
+// The 16 builder warps turn S(v) into the BF16 coefficient tile H one 64-column
+// half at a time (warp w: rows 32 (w % 4) .., 16 columns of each half): the
+// accumulation of one half runs while the next half (or the next tile's first
+// half) is built, and S(v + 1) is ready before H(v) is done.
+//
+// The other side's per-column inputs (auxiliary, logsumexp) come through shared
+// memory too: a warp loads the values of its next 16 columns one half tile ahead
+// (one per lane) and writes them, with what only depends on the column, into slot
+// h of its column group when it begins half tile (v, h).  Read from global memory
+// as they were used, their first touch of every tile was an L2 round trip in each
+// builder's serial chain, and every row's thread formed the column's factors
+// again.  The four warps of a column group write the same values to the same slot;
+// a warp beginning (v, h) has seen the accumulation of (v - 1, h) complete, so
+// every builder is past that half tile and the slot is free.
 constexpr int kBwdWarps = 16;
-constexpr int kBwdThreads = 32 * (kBwdWarps + 2);
+constexpr int kBwdCinBytes = 2 * 4 * kCinFloats * 4;
+constexpr int kBwdThreads = 32 * (kBwdWarps + 3);
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
+// 16 columns at taddr and 16 at taddr + 64, both reads in flight together.
+__device__ __forceinline__ void tmem_ld16x2(uint32_t taddr, float (&v)[16], float (&w)[16]) {
+  uint32_t r[32];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr), "r"(taddr + 64)
       : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) {
+    v[i] = __uint_as_float(r[i]);
+    w[i] = __uint_as_float(r[16 + i]);
+  }
+}
+
+// What a builder warp needs of its CTA, in registers (the argument blocks of the
+// two passes are selected at run time: a field read in the loop would be a
+// memory access each time).
+struct BuildCtx {
+  const float* cin_src;   // this lane's per-column input (null-free; read only where cin_live)
+  float* cin_all;
+  uint64_t *sfull, *sfree, *hready, *hdone;
+  uint8_t* Hs;
+  unsigned long long lim;
+  uint32_t tmem;          // S accumulators at this warp's lanes
+  int q, lane, r, u, u0, nV, B;
+  bool cin_live;
+  float kb_oth, k2_oth;
+};
+
+// The builder loop of one warp.  No block-wide barrier per tile: the warp waits
+// for what it reads (S(vt), a free H region) and arrives on what it produces (S
+// read, half written).  Both halves' columns of S come in one TMEM read.
+template <int EK, int OBJ, int LIVE>
+__device__ __forceinline__ bool build_tiles(const BuildCtx& bc, const HCoef& hc, float& rowsum) {
+  const int q = bc.q, lane = bc.lane, r = bc.r, B = bc.B;
+  auto cin_load = [&](int vt, int h) {
+    const int v = vt * kTile + 64 * h + 16 * q + (lane & 15);
+    return (bc.cin_live && v < B) ? __ldg(bc.cin_src + v) : 0.f;
+  };
+  float cin_next = cin_load(0, 0);
+  for (int vt = 0; vt < bc.nV; ++vt) {
+    const int v0 = vt * kTile, b = vt & 1;
+    if (!__all_sync(0xffffffffu, tc::mbar_wait(&bc.sfull[b], (vt >> 1) & 1, bc.lim) ? 1 : 0)) return false;
+    tc::fence_after_sync();
+    // (the objectives outside InfoNCE always take the tested form: fewer instantiations)
+    const bool edge = OBJ != kObjInfo || bc.u0 == v0 || bc.u0 + kTile > B || v0 + kTile > B;
+    float sv[2][16];
+    tmem_ld16x2(bc.tmem + (uint32_t)(b * 128) + 16 * q, sv[0], sv[1]);
+    // this warp is done with S(vt): the accumulator may take S(vt + 2)
+    tc::fence_before_sync();
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&bc.sfree[b]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      // half h's region (and input slot) is free once the accumulation of tile vt - 1's half h is done
+      if (vt >= 1 && !__all_sync(0xffffffffu, tc::mbar_wait(&bc.hdone[h], (vt - 1) & 1, bc.lim) ? 1 : 0)) return false;
+      const int cb = 64 * h + 16 * q;   // this warp's 16 columns of half h
+      float* cin = bc.cin_all + (4 * h + q) * kCinFloats;
+      if (lane < 16) {
+        cin[lane] = cin_next;
+      } else if (LIVE != 1) {
+        float ko = fmaf(bc.k2_oth, cin_next, bc.kb_oth);
+        if (kFoldTau<EK, OBJ, LIVE, false> && !edge) ko *= hc.inv_tau;
+        cin[lane] = kFoldTau<EK, OBJ, LIVE, false> && !edge ? -__fmul_rn(cin_next, kLog2e) : -cin_next;
+        cin[16 + lane] = ko;
+      }
+      if (h == 0) cin_next = cin_load(vt, 1);
+      else if (vt + 1 < bc.nV) cin_next = cin_load(vt + 1, 0);
+      __syncwarp();
+      uint32_t packed[8];
+      if (edge) build_h<EK, OBJ, LIVE, true>(sv[h], hc, cin, cb, bc.u, v0, B, rowsum, packed);
+      else build_h<EK, OBJ, LIVE, OBJ != kObjInfo>(sv[h], hc, cin, cb, bc.u, v0, B, rowsum, packed);
+      // columns 16 q .. 16 q + 15 of half h: 16-byte chunks 2 q, 2 q + 1 of the
+      // half's 128-byte-swizzled K-major tile
+      uint8_t* hb = bc.Hs + h * 16384;
+#pragma unroll
+      for (int c2 = 0; c2 < 2; ++c2) {
+        const uint4 val = make_uint4(packed[4 * c2], packed[4 * c2 + 1], packed[4 * c2 + 2], packed[4 * c2 + 3]);
+        *reinterpret_cast<uint4*>(hb + sw128_offset(r, 2 * q + c2)) = val;
+      }
+      // make the generic-proxy H writes visible to the tensor core, then publish
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&bc.hready[h]);
+    }
+  }
+  return true;
 }
 
 template <int OBJ>
@@ -976,7 +1113,8 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
   uint8_t* Ys = Xs + tbytes;                              // other tiles, 2 buffers    2 x nk x 16 KiB
   uint8_t* Hs = Ys + 2 * tbytes;                          // H halves                  2 x 16 KiB
   float* s_red = reinterpret_cast<float*>(Hs);              // [4][128] partial sums (H is free by then)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(Hs + 2 * 16384);
+  float* cin_all = reinterpret_cast<float*>(Hs + 2 * 16384);  // [2][4][48] staged per-column inputs
+  uint64_t* bars = reinterpret_cast<uint64_t*>(Hs + 2 * 16384 + kBwdCinBytes);
   uint64_t* xload = bars;
   uint64_t* yfull = bars + 1;   // [2] other tile v landed in buffer v % 2
   uint64_t* sfull = bars + 3;   // [2] S(v) in accumulator v % 2
@@ -1006,7 +1144,7 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
       tc::mbar_init(&hready[b], kBwdWarps);
       tc::mbar_init(&hdone[b], 1);
     }
-    tc::mbar_init(drain, 1);
+    tc::mbar_init(drain, 2);   // both issuers
     tc::fence_mbar_init();
   }
   if (warp == kBwdWarps + 1) {
@@ -1051,66 +1189,54 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
     }
   } else if (warp == kBwdWarps + 1) {
     if (lane == 0) {
-      // MMA issuer: S(v) and the halves of acc(v), each as soon as its inputs are ready
+      // S issuer: S(v) = own . other(v)^T as soon as tile v has landed and the builders have read S(v - 2)
       constexpr uint32_t idesc_s = tc::idesc_bf16_f32(128, 128);
-      const uint32_t idesc_acc = tc::idesc_bf16_f32_bmn(128, a.R);
       bool ok = tc::mbar_wait(xload, 0, lim);
-      if (!ok) atomicOr(a.status, CRL_STATUS_TIMEOUT);
-      tc::fence_after_sync();
-      int next_s = 0, next_h = 0;   // next S(v) to issue; next accumulation half (2 v + h)
-      unsigned long long t_idle = tc::globaltimer();
-      while (ok && (next_s < nV || next_h < 2 * nV)) {
-        bool progress = false;
-        if (next_s < nV && next_s <= next_h / 2 + 1) {
-          const int v = next_s, b = v & 1;
-          if (tc::mbar_test_wait(&yfull[b], (v >> 1) & 1) &&
-              (v < 2 || tc::mbar_test_wait(&sfree[b], ((v >> 1) - 1) & 1))) {
-            tc::fence_after_sync();
-            const uint8_t* ys = Ys + b * tbytes;
-            for (int kb = 0; kb < nk; ++kb) {
-              const uint64_t dx = tc::sdesc_kmajor_sw128(Xs + kb * 16384);
-              const uint64_t dy = tc::sdesc_kmajor_sw128(ys + kb * 16384);
+      for (int v = 0; v < nV && ok; ++v) {
+        const int b = v & 1;
+        ok = tc::mbar_wait(&yfull[b], (v >> 1) & 1, lim) && (v < 2 || tc::mbar_wait(&sfree[b], ((v >> 1) - 1) & 1, lim));
+        if (!ok) break;
+        tc::fence_after_sync();
+        const uint8_t* ys = Ys + b * tbytes;
+        for (int kb = 0; kb < nk; ++kb) {
+          const uint64_t dx = tc::sdesc_kmajor_sw128(Xs + kb * 16384);
+          const uint64_t dy = tc::sdesc_kmajor_sw128(ys + kb * 16384);
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                tc::mma_bf16(tmem + (uint32_t)(b * 128), dx + 2 * k, dy + 2 * k, idesc_s, (kb | k) ? 1u : 0u);
-            }
-            tc::mma_commit(&sfull[b]);
-            ++next_s;
-            progress = true;
-          }
+          for (int k = 0; k < 4; ++k)
+            tc::mma_bf16(tmem + (uint32_t)(b * 128), dx + 2 * k, dy + 2 * k, idesc_s, (kb | k) ? 1u : 0u);
         }
-        if (next_h < 2 * nV && next_h / 2 < next_s) {
-          const int v = next_h / 2, h = next_h % 2;
-          if (tc::mbar_test_wait(&hready[h], v & 1)) {
-            tc::fence_after_sync();
-            // half h of H (K = other rows 64 h .. 64 h + 63) times the other tile as the MN-major
-            // B operand: K steps of 16 rows are 2048 bytes, R chunks of 64 columns 16 KiB apart
-            const uint8_t* ys = Ys + (v & 1) * tbytes;
-            const uint64_t dh = tc::sdesc_kmajor_sw128(Hs + h * 16384);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const uint64_t dt = tc::sdesc_mnmajor_sw128(ys + h * 8192 + k * 2048, 16384);
-              tc::mma_bf16(tAcc, dh + 2 * k, dt, idesc_acc, (v | h | k) ? 1u : 0u);
-            }
-            tc::mma_commit(&hdone[h]);
-            ++next_h;
-            progress = true;
-          }
-        }
-        if (progress) {
-          t_idle = tc::globaltimer();
-        } else if (tc::globaltimer() - t_idle > lim) {
-          atomicOr(a.status, CRL_STATUS_TIMEOUT);
-          ok = false;
-        } else {
-          __nanosleep(128);   // leave the issue slots to the builder warps
-        }
+        tc::mma_commit(&sfull[b]);
       }
+      if (!ok) atomicOr(a.status, CRL_STATUS_TIMEOUT);
       tc::mma_commit(drain);   // completes once every MMA issued above has
+    }
+  } else if (warp == kBwdWarps + 2) {
+    if (lane == 0) {
+      // accumulation issuer: half h of H(v) (K = other rows 64 h .. 64 h + 63) times the other tile
+      // as the MN-major B operand: K steps of 16 rows are 2048 bytes, R chunks of 64 columns 16 KiB apart
+      const uint32_t idesc_acc = tc::idesc_bf16_f32_bmn(128, a.R);
+      bool ok = true;
+      for (int n = 0; n < 2 * nV && ok; ++n) {
+        const int v = n >> 1, h = n & 1;
+        ok = tc::mbar_wait(&yfull[v & 1], (v >> 1) & 1, lim) && tc::mbar_wait(&hready[h], v & 1, lim);
+        if (!ok) break;
+        tc::fence_after_sync();
+        const uint8_t* ys = Ys + (v & 1) * tbytes;
+        const uint64_t dh = tc::sdesc_kmajor_sw128(Hs + h * 16384);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint64_t dt = tc::sdesc_mnmajor_sw128(ys + h * 8192 + k * 2048, 16384);
+          tc::mma_bf16(tAcc, dh + 2 * k, dt, idesc_acc, (n | k) ? 1u : 0u);
+        }
+        tc::mma_commit(&hdone[h]);
+      }
+      if (!ok) atomicOr(a.status, CRL_STATUS_TIMEOUT);
+      tc::mma_commit(drain);
     }
   } else {
     // ---- builder warps
     const int lg = warp % 4, q = warp / 4;
+    const int B = row.B;           // (both passes')
     const int r = lg * 32 + lane;  // row of this thread within the tile
     const uint32_t lane_off = (uint32_t)(lg * 32) << 16;
     const int u = u0 + r;
@@ -1122,6 +1248,7 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
     const float w_oth = a.transposed ? a.w.wf : a.w.wb, p_oth = a.transposed ? a.w.pr : a.w.pc;
     HCoef hc;
     hc.a_own = a_own;
+    hc.l_own = l_own;
     hc.l_own2 = l_own * kLog2e;
     hc.k_own = a.scale * (w_own + 2.f * a.beta * p_own * l_own);
     hc.k_own_tau = hc.k_own * a.inv_tau;
@@ -1143,72 +1270,25 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
     hc.transposed = a.transposed;
     const int ek = a.energy == CRL_ENERGY_L2 ? 0 : (a.energy == CRL_ENERGY_L2SQ ? 1 : 2);
     const float kb_oth = a.scale * w_oth, k2_oth = 2.f * a.scale * a.beta * p_oth;
+    // this lane's share of the inputs of columns v0 + 64 h + 16 q ..: the auxiliary
+    // of column lane (lanes 0 .. 15) or the logsumexp of column lane - 16
+    const float* cin_src = lane < 16 ? a.aux_other : a.lse_other;
+    const bool cin_live = lane < 16 ? ek != 2 : live != 1;
     float rowsum = 0.f;
     bool ok = true;
-    // No block-wide barrier per tile: each warp waits for what it reads (S(vt),
-    // a free H region) and arrives on what it produces (S read, half written).
-    for (int vt = 0; vt < nV && ok; ++vt) {
-      const int v0 = vt * kTile, b = vt & 1;
-      ok = __all_sync(0xffffffffu, tc::mbar_wait(&sfull[b], (vt >> 1) & 1, lim) ? 1 : 0) != 0;
-      if (!ok) break;
-      tc::fence_after_sync();
-      // (the objectives outside InfoNCE always take the tested form: fewer instantiations)
-      const bool edge = OBJ != kObjInfo || u0 == v0 || u0 + kTile > a.B || v0 + kTile > a.B;
-#pragma unroll 1
-      for (int h = 0; h < 2 && ok; ++h) {
-        const int cb = 64 * h + 16 * q;   // this warp's 16 columns of half h
-        float sv[16];
-        tmem_ld16(tmem + (uint32_t)(b * 128) + lane_off + cb, sv);
-        if (h == 1) {
-          // this warp is done with S(vt): the accumulator may take S(vt + 2)
-          tc::fence_before_sync();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&sfree[b]);
-        }
-        uint32_t packed[8];
-#define CRL_BUILD_H(EK, LV, ED)                                                                              \
-  build_h<EK, OBJ, LV, (ED) || OBJ != kObjInfo, 16>(sv, hc, a.aux_other, a.lse_other, kb_oth, k2_oth, cb, u, v0, \
-                                                    a.B, rowsum, packed)
-        switch (2 * (3 * ek + live) + (edge ? 1 : 0)) {
-          case 0: CRL_BUILD_H(0, 0, false); break;
-          case 1: CRL_BUILD_H(0, 0, true); break;
-          case 2: CRL_BUILD_H(0, 1, false); break;
-          case 3: CRL_BUILD_H(0, 1, true); break;
-          case 4: CRL_BUILD_H(0, 2, false); break;
-          case 5: CRL_BUILD_H(0, 2, true); break;
-          case 6: CRL_BUILD_H(1, 0, false); break;
-          case 7: CRL_BUILD_H(1, 0, true); break;
-          case 8: CRL_BUILD_H(1, 1, false); break;
-          case 9: CRL_BUILD_H(1, 1, true); break;
-          case 10: CRL_BUILD_H(1, 2, false); break;
-          case 11: CRL_BUILD_H(1, 2, true); break;
-          case 12: CRL_BUILD_H(2, 0, false); break;
-          case 13: CRL_BUILD_H(2, 0, true); break;
-          case 14: CRL_BUILD_H(2, 1, false); break;
-          case 15: CRL_BUILD_H(2, 1, true); break;
-          case 16: CRL_BUILD_H(2, 2, false); break;
-          default: CRL_BUILD_H(2, 2, true); break;
-        }
-#undef CRL_BUILD_H
-        // half h's region is free once the accumulation of tile vt - 1's half h is done
-        if (vt >= 1) {
-          ok = __all_sync(0xffffffffu, tc::mbar_wait(&hdone[h], (vt - 1) & 1, lim) ? 1 : 0) != 0;
-          if (!ok) break;
-        }
-        // columns 16 q .. 16 q + 15 of half h: 16-byte chunks 2 q, 2 q + 1 of the
-        // half's 128-byte-swizzled K-major tile
-        uint8_t* hb = Hs + h * 16384;
-#pragma unroll
-        for (int c2 = 0; c2 < 2; ++c2) {
-          const uint4 val = make_uint4(packed[4 * c2], packed[4 * c2 + 1], packed[4 * c2 + 2], packed[4 * c2 + 3]);
-          *reinterpret_cast<uint4*>(hb + sw128_offset(r, 2 * q + c2)) = val;
-        }
-        // make the generic-proxy H writes visible to the tensor core, then publish
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&hready[h]);
-      }
+    const BuildCtx bc{cin_src, cin_all, sfull, sfree, hready, hdone, Hs, lim, tmem + lane_off, q, lane, r, u, u0,
+                      nV, B, cin_live, kb_oth, k2_oth};
+    // one loop per energy and set of live softmax terms: no dispatch per half tile
+    switch (3 * ek + live) {
+      case 0: ok = build_tiles<0, OBJ, 0>(bc, hc, rowsum); break;
+      case 1: ok = build_tiles<0, OBJ, 1>(bc, hc, rowsum); break;
+      case 2: ok = build_tiles<0, OBJ, 2>(bc, hc, rowsum); break;
+      case 3: ok = build_tiles<1, OBJ, 0>(bc, hc, rowsum); break;
+      case 4: ok = build_tiles<1, OBJ, 1>(bc, hc, rowsum); break;
+      case 5: ok = build_tiles<1, OBJ, 2>(bc, hc, rowsum); break;
+      case 6: ok = build_tiles<2, OBJ, 0>(bc, hc, rowsum); break;
+      case 7: ok = build_tiles<2, OBJ, 1>(bc, hc, rowsum); break;
+      default: ok = build_tiles<2, OBJ, 2>(bc, hc, rowsum); break;
     }
     if (!ok && lane == 0) atomicOr(a.status, CRL_STATUS_TIMEOUT);
     // every accumulation done: the H regions become the row-sum partials
@@ -1358,9 +1438,8 @@ int fwd_chunk_tiles(int n) {
   return best;
 }
 size_t bwd_smem(int R) {
-  // own tile, two other tiles, H (then the row-sum partials), three per-tile arrays, barriers, alignment
-  // own tile, two other tiles, the two H halves (then the row-sum partials), barriers, alignment
-  return (size_t)3 * (R / 64) * 16384 + 2 * 16384 + 128 + 1024;
+  // own tile, two other tiles, the two H halves (then the row-sum partials), staged inputs, barriers, alignment
+  return (size_t)3 * (R / 64) * 16384 + 2 * 16384 + kBwdCinBytes + 128 + 1024;
 }
 
 FwdArgs fwd_args(const EnergyTc& e, const LossSpec& ls, int B, void* ws, float* loss4, float* r, float* c,
