@@ -21,11 +21,17 @@ __global__ void __launch_bounds__(256) adam_kernel(T* __restrict__ p, const T* _
   pdl_enter();
   // Bias corrections in double (1 - b^t loses most of its digits in float for
   // small t), computed once per block.
+  // b^t by repeated squaring (at most 31 double products; pow() took several us of
+  // the FP64 pipe before every block's first load), one thread per power.
   __shared__ double s_corr[2];
-  if (threadIdx.x == 0) {
-    const int t = t_dev ? *t_dev : t_host;
-    s_corr[0] = (double)lr / (1.0 - pow((double)b1, (double)t));
-    s_corr[1] = 1.0 / (1.0 - pow((double)b2, (double)t));
+  if (threadIdx.x == 0 || threadIdx.x == kWarp) {
+    double x = threadIdx.x == 0 ? (double)b1 : (double)b2, bt = 1.0;
+    for (int t = t_dev ? *t_dev : t_host; t > 0; t >>= 1) {
+      if (t & 1) bt *= x;
+      x *= x;
+    }
+    if (threadIdx.x == 0) s_corr[0] = (double)lr / (1.0 - bt);
+    else s_corr[1] = 1.0 / (1.0 - bt);
   }
   __syncthreads();
   const T step = T(s_corr[0]);

@@ -138,24 +138,37 @@ __global__ void __launch_bounds__(256) row_lse_kernel(int B, const T* __restrict
   if (lane == 0) r[row] = m + dev_log(s);
 }
 
-// c_j = LSE_i F_ij.  Block = 32 columns x 8 row groups; each thread keeps a
-// running (max, sum) over its rows, then the 8 partials of a column are merged.
+// Column kernels: block = 32 columns x 32 row groups (1024 threads), eight rows
+// per step of a thread, loaded together.  (Eight row groups of single rows left a
+// chain of B / 8 dependent loads and exponentials per thread: 24 us at B = 1001
+// against 5 now; a thread per column for the sums, 26 against 4.)
+constexpr int kColRows = 32, kColBatch = 8;
+
+// c_j = LSE_i F_ij: a running (max, sum) per thread over its rows, eight at a
+// time (one rescaling per step), then the 32 partials of a column are merged.
 template <typename T>
-__global__ void __launch_bounds__(256) col_lse_kernel(int B, const T* __restrict__ F, T* __restrict__ c) {
+__global__ void __launch_bounds__(32 * kColRows) col_lse_kernel(int B, const T* __restrict__ F, T* __restrict__ c) {
   pdl_enter();
-  __shared__ T sm_m[8][33], sm_s[8][33];
+  __shared__ T sm_m[kColRows][33], sm_s[kColRows][33];
   const int cx = threadIdx.x % 32, ry = threadIdx.x / 32;
   const int j = blockIdx.x * 32 + cx;
   T m = -INFINITY, s = 0;
   if (j < B) {
-    for (int i = ry; i < B; i += 8) {
-      const T x = F[(size_t)i * B + j];
-      if (x > m) {
-        s = s * dev_exp(m - x) + T(1);
-        m = x;
-      } else {
-        s += dev_exp(x - m);
+    for (int i = ry; i < B; i += kColRows * kColBatch) {
+      T x[kColBatch], mb = m;
+#pragma unroll
+      for (int q = 0; q < kColBatch; ++q) {
+        const int r = i + kColRows * q;
+        x[q] = r < B ? F[(size_t)r * B + j] : T(-INFINITY);
+        mb = fmax(mb, x[q]);
       }
+      // (the maximum's own term is 1 whatever it is: no inf - inf)
+      T t = m == mb ? s : s * dev_exp(m - mb);
+#pragma unroll
+      for (int q = 0; q < kColBatch; ++q)
+        if (i + kColRows * q < B) t += x[q] == mb ? T(1) : dev_exp(x[q] - mb);
+      s = t;
+      m = mb;
     }
   }
   sm_m[ry][cx] = m;
@@ -163,34 +176,35 @@ __global__ void __launch_bounds__(256) col_lse_kernel(int B, const T* __restrict
   __syncthreads();
   if (ry == 0 && j < B) {
     T mm = sm_m[0][cx];
-    for (int r = 1; r < 8; ++r) mm = fmax(mm, sm_m[r][cx]);
+    for (int r = 1; r < kColRows; ++r) mm = fmax(mm, sm_m[r][cx]);
     T ss = 0;
-    for (int r = 0; r < 8; ++r)
+#pragma unroll 8
+    for (int r = 0; r < kColRows; ++r)
       if (sm_s[r][cx] > T(0)) ss += sm_s[r][cx] * dev_exp(sm_m[r][cx] - mm);
     c[j] = mm + dev_log(ss);
   }
 }
 
-// Row sums (warp per row) and column sums (thread per column) of H.
+// Column sums of H.
 template <typename T>
-__global__ void __launch_bounds__(256) row_sum_kernel(int B, const T* __restrict__ H, T* __restrict__ out) {
+__global__ void __launch_bounds__(32 * kColRows) col_sum_kernel(int B, const T* __restrict__ H, T* __restrict__ out) {
   pdl_enter();
-  const int lane = threadIdx.x % kWarp;
-  const int row = blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp;
-  if (row >= B) return;
+  __shared__ T sm[kColRows][33];
+  const int cx = threadIdx.x % 32, ry = threadIdx.x / 32;
+  const int j = blockIdx.x * 32 + cx;
   T s = 0;
-  for (int c = lane; c < B; c += kWarp) s += H[(size_t)row * B + c];
-  s = warp_sum(s);
-  if (lane == 0) out[row] = s;
-}
-template <typename T>
-__global__ void __launch_bounds__(256) col_sum_kernel(int B, const T* __restrict__ H, T* __restrict__ out) {
-  pdl_enter();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= B) return;
-  T s = 0;
-  for (int i = 0; i < B; ++i) s += H[(size_t)i * B + j];
-  out[j] = s;
+  if (j < B) {
+#pragma unroll 8
+    for (int i = ry; i < B; i += kColRows) s += H[(size_t)i * B + j];
+  }
+  sm[ry][cx] = s;
+  __syncthreads();
+  if (ry == 0 && j < B) {
+    T t = 0;
+#pragma unroll
+    for (int r = 0; r < kColRows; ++r) t += sm[r][cx];
+    out[j] = t;
+  }
 }
 
 // wf, wb: weights of the InfoNCE directions in the loss and its gradient (FlatNCE
@@ -283,7 +297,7 @@ __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__
                                                    double beta, T* __restrict__ loss4, unsigned* status,
                                                    int* t_bump) {
   pdl_enter();
-  __shared__ T sm[32];
+  __shared__ T sm[5][32];   // 1024 threads: 32 warps
   T a_f = 0, a_b = 0, a_r2 = 0, a_c2 = 0, a_o = 0;
   for (int i = threadIdx.x; i < B; i += blockDim.x) {
     const T d = F[(size_t)i * ldf + i];
@@ -293,11 +307,22 @@ __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__
     a_c2 += c[i] * c[i];
     if (ov) a_o += ov[i];
   }
-  a_f = block_sum(a_f, sm);
-  a_b = block_sum(a_b, sm);
-  a_r2 = block_sum(a_r2, sm);
-  a_c2 = block_sum(a_c2, sm);
-  a_o = block_sum(a_o, sm);
+  // the five block sums in one round: warp sums, then warp 0 adds the warps' parts
+  {
+    const int lane = threadIdx.x % kWarp, wid = threadIdx.x / kWarp;
+    T part[5] = {a_f, a_b, a_r2, a_c2, a_o};
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      part[q] = warp_sum(part[q]);
+      if (lane == 0) sm[q][wid] = part[q];
+    }
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int q = 0; q < 5; ++q) part[q] = warp_sum(sm[q][lane]);
+    }
+    a_f = part[0], a_b = part[1], a_r2 = part[2], a_c2 = part[3], a_o = part[4];
+  }
   if (threadIdx.x == 0) {
     const T inv = T(1) / T(B);
     const T lf = a_f * inv, lb = a_b * inv;
@@ -315,22 +340,27 @@ __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__
 
 // F -> H in place (see the header comment).
 // dg, kd: F_ii and k_i from objective_rows_kernel (objectives outside InfoNCE).
+// One block per row: the row's constants are read once, no index division, and the
+// row sums of H (rsum, may be null) cost no further pass over the matrix.
 template <typename T>
 __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ F, const T* __restrict__ r,
                                                         const T* __restrict__ c, const T* __restrict__ dg,
                                                         const T* __restrict__ kd, DirWeights w, double beta,
-                                                        double dtotal, int energy, double tau) {
+                                                        double dtotal, int energy, double tau, T* __restrict__ rsum) {
   pdl_enter();
-  const size_t n = (size_t)B * B;
+  __shared__ T sm[32];
+  const int i = blockIdx.x;
+  T* __restrict__ row = F + (size_t)i * B;
+  const T ri = r[i];
+  T sum = 0;
   const T scale = T(dtotal / B);
   const T bb = T(B) * T(B);
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / B), j = (int)(e % B);
-    const T f = F[e];
-    const T P = dev_exp(f - r[i]);
+  for (int j = threadIdx.x; j < B; j += blockDim.x) {
+    const T f = row[j];
+    const T P = dev_exp(f - ri);
     const T Q = dev_exp(f - c[j]);
     const T dlt = (i == j) ? T(1) : T(0);
-    T g = T(w.wf) * (P - dlt) + T(w.wb) * (Q - dlt) + T(2.0 * beta) * (T(w.pr) * r[i] * P + T(w.pc) * c[j] * Q);
+    T g = T(w.wf) * (P - dlt) + T(w.wb) * (Q - dlt) + T(2.0 * beta) * (T(w.pr) * ri * P + T(w.pc) * c[j] * Q);
     g *= scale;
     if (w.obj >= CRL_LOSS_FB) {
       T o = 0;
@@ -353,8 +383,12 @@ __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ 
       case CRL_ENERGY_L2SQ: h = T(2) * g / T(tau); break;
       default: h = g / T(tau); break;  // dot, cos
     }
-    F[e] = h;
+    row[j] = h;
+    sum += h;
   }
+  if (rsum == nullptr) return;
+  sum = block_sum(sum, sm);
+  if (threadIdx.x == 0) rsum[i] = sum;
 }
 
 // dphi_i = (dx_i - x_i <x_i, dx_i>) * inv_i, in place on dx.  One warp per row.
@@ -456,7 +490,7 @@ void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int 
     default: gemm<T, InnerOp::kMul>(B, B, R, la, lb, ep, st, CRL_TRACE_ENERGY); break;
   }
   { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(row_lse_kernel<T>, dim3(nb), dim3(256), 0, st, B, w.F, row_lse); }
-  { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(col_lse_kernel<T>, dim3(ceil_div(B, 32)), dim3(256), 0, st, B, w.F, col_lse); }
+  { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(col_lse_kernel<T>, dim3(ceil_div(B, 32)), dim3(32 * kColRows), 0, st, B, w.F, col_lse); }
   const bool rows = has_rows_pass(ls.loss);
   if (rows) {
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
@@ -495,16 +529,15 @@ void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
     launch_k(objective_rows_kernel<T>, dim3(nb), dim3(256), 0, st, B, (const T*)w.F, ls.loss, w.dg, w.ov, w.kd);
   }
-  const int ge = (int)std::min<int64_t>(ceil_div((int64_t)B * B, 256), 152 * 16);
+  const bool diff = ls.energy == CRL_ENERGY_L2 || ls.energy == CRL_ENERGY_L2SQ;
   {
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
-    launch_k(grad_coeff_kernel<T>, dim3(ge), dim3(256), 0, st, B, w.F, row_lse, col_lse, (const T*)w.dg,
-             (const T*)w.kd, weights(ls), ls.beta, dtotal, ls.energy, ls.tau);
+    launch_k(grad_coeff_kernel<T>, dim3(B), dim3(256), 0, st, B, w.F, row_lse, col_lse, (const T*)w.dg,
+             (const T*)w.kd, weights(ls), ls.beta, dtotal, ls.energy, ls.tau, diff ? w.rsum : (T*)nullptr);
   }
   const T* H = w.F;
-  if (ls.energy == CRL_ENERGY_L2 || ls.energy == CRL_ENERGY_L2SQ) {
-    { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(row_sum_kernel<T>, dim3(nb), dim3(256), 0, st, B, H, w.rsum); }
-    { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(col_sum_kernel<T>, dim3(ceil_div(B, 256)), dim3(256), 0, st, B, H, w.csum); }
+  if (diff) {
+    { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(col_sum_kernel<T>, dim3(ceil_div(B, 32)), dim3(32 * kColRows), 0, st, B, H, w.csum); }
     gemm<T>(B, R, B, LoadMK<T>{H, B}, LoadKN<T>{psi, R}, EpiSubRowScaled<T>{dphi, R, T(1), w.rsum, phi, R}, st,
             CRL_TRACE_ENERGY);
     gemm<T>(B, R, B, LoadTrans<T>{H, B}, LoadKN<T>{phi, R}, EpiSubRowScaled<T>{dpsi, R, T(1), w.csum, psi, R},
