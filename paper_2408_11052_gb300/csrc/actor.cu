@@ -321,10 +321,9 @@ const char* multi_tables(BlobCache& cache, const std::vector<Task>& tasks, int i
 template <typename T>
 void actor_head_forward(const ActorSpec& as, const T* pi_out, const float* eps, const unsigned long long* step_dev,
                         uint64_t seed, uint64_t agent, int B, T* a_new, T* logpi, T* eps_used, cudaStream_t st,
-                        __nv_bfloat16* x0, int x0_ld, int x0_col, int noise_extra) {
+                        __nv_bfloat16* x0, int x0_ld, int x0_col) {
   TraceLaunch tr(CRL_TRACE_AUX, st, (double)B * as.A * sizeof(T) * 5);
-  const HeadFwdArgs<T> p{B,        as.A, pi_out, eps,   step_dev, seed,  agent,      a_new,
-                         logpi,    eps_used, x0, x0_ld, x0_col,   noise_extra};
+  const HeadFwdArgs<T> p{B, as.A, pi_out, eps, step_dev, seed, agent, a_new, logpi, eps_used, x0, x0_ld, x0_col};
   launch_k(head_forward_kernel<T>, dim3(ceil_div(B, 8)), dim3(256), 0, st, p);
 }
 
@@ -381,7 +380,7 @@ void actor_head_backward(const ActorSpec& as, const T* pi_out, const T* eps_used
 #define CRL_INST_ACTOR(T)                                                                                        \
   template void actor_head_forward<T>(const ActorSpec&, const T*, const float*, const unsigned long long*,       \
                                       uint64_t, uint64_t, int, T*, T*, T*, cudaStream_t, __nv_bfloat16*, int,    \
-                                      int, int);                                                                 \
+                                      int);                                                                      \
   template void actor_energy_and_loss<T>(const ActorSpec&, const T*, const T*, const T*, int, int, T*, T*, T*,   \
                                          void*, unsigned*, unsigned*, int*, unsigned long long*,                 \
                                          const unsigned long long*, cudaStream_t, __nv_bfloat16*, int);          \

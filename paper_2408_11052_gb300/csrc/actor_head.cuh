@@ -39,7 +39,7 @@ __device__ __forceinline__ void head_forward_body(const HeadFwdArgs<T>& p, int l
     const T mu = out[(size_t)b * 2 * A + d];
     const T lraw = out[(size_t)b * 2 * A + A + d];
     const T l = fmin(fmax(lraw, T(kLogStdMin)), T(kLogStdMax));
-    const T e = eps ? T(eps[(size_t)b * A + d]) : philox_normal<T>(step, b, 1ull + p.noise_extra, d, seed, agent);
+    const T e = eps ? T(eps[(size_t)b * A + d]) : philox_normal<T>(step, b, 1ull, d, seed, agent);
     const T u = mu + dev_exp(l) * e;
     const T act = dev_tanh(u);
     a_new[(size_t)b * A + d] = act;

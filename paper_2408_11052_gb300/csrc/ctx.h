@@ -106,9 +106,7 @@ struct crl_ctx {
     float* g = nullptr;                   // [E][G] current commanded goals
     int32_t* t = nullptr;                 // [E] step within the episode
     unsigned long long* step = nullptr;   // next collection step (Philox counter)
-    void *pi_out = nullptr, *a = nullptr, *logpi = nullptr, *eps = nullptr, *saved = nullptr;
-    float *obs = nullptr, *act = nullptr;  // one time slice for the insert
-    uint8_t* done = nullptr;
+    void *pi_out = nullptr, *a = nullptr, *saved = nullptr;
   } env;
   // logit statistics of the critic steps (crl_set_logit_stats): [2] floats and per-tile FP64 sums
   bool stats_on = false;

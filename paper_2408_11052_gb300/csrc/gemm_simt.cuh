@@ -120,124 +120,152 @@ __global__ void __launch_bounds__(256) gemm_tile_kernel(int M, int N, int K, LA 
 }
 
 // ---- FP32 kernel ---------------------------------------------------------------
-// The same product for FP32 operands.  The 2 x 2 and 4 x 4 outputs per thread of
-// the kernel above take one 4-byte shared read per operand value: at 32 x 32 tiles
-// the shared-memory pipe, not the FMA pipe, set the pace (1024 x 256 x 256: 10 us
-// against 1.7 us of FMAs).  Here a thread owns TM x TN neighbouring outputs, reads
-// its operands 8 or 16 bytes at a time and multiplies two columns per instruction;
-// slices of 16 k arrive through a four-deep ring of asynchronous copies.  Every
-// output is the same chain of fused multiply-adds over k in order, so it has the
-// bits of the kernel above, whatever the tile.
+// The same product for FP32 operands.  The kernel above takes one 4-byte shared
+// read per operand value: at 32 x 32 tiles the shared-memory pipe, not the FMA pipe,
+// set the pace (1024 x 256 x 256: 10 us against 1.7 us of FMAs).  Here every shared
+// read is 8 or 16 bytes, and slices of 16 k arrive through a four-deep ring of
+// asynchronous copies (16 bytes each where the rows allow it).  An operand stays in
+// the order it has in memory: k along rows ([m][16 + 4]: the pitch and the strided
+// rows of a thread, ty, ty + BM / TM, ..., make the reads conflict-free), or m / n
+// along rows ([k][BM + 4], a thread's neighbouring columns, two per instruction).
+// Every output is the same chain of fused multiply-adds over k in order, so it has
+// the bits of the kernel above, whatever the tile and the orders.
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool live) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(live ? 4 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool live) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(live ? 16 : 0) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(live ? 16 : 0) : "memory");
 }
 
-template <int N>
-__device__ __forceinline__ void lds_row(const float* p, float (&v)[N]) {
-  if constexpr (N == 4) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-  } else {
-    const float2 t = *reinterpret_cast<const float2*>(p);
-    v[0] = t.x, v[1] = t.y;
+constexpr int kF32K = 16, kF32Stages = 4;
+
+// One operand's ring: R rows or columns of the tile, T of them per thread.
+// KC: k is contiguous in memory (and in the ring).
+template <bool KC, int R, int T>
+struct F32Ring {
+  static constexpr int kPitch = KC ? kF32K + 4 : R + 4;
+  static constexpr int kRows = KC ? R : kF32K;
+  float v[kF32Stages][kRows][kPitch];
+  // copy slice k0 .. k0 + 15; at(i, k): element address; rows [r0, n) and k < K live
+  template <int THREADS, class AT>
+  __device__ __forceinline__ void load(int buf, int k0, int r0, int n, int K, bool vec, const AT& at) {
+    const int tid = threadIdx.x;
+    if (vec) {   // 4 consecutive elements of a row per copy, wholly inside or outside
+#pragma unroll
+      for (int e0 = 0; e0 < R * kF32K / 4; e0 += THREADS) {
+        const int e = e0 + tid;
+        if (R * kF32K / 4 % THREADS != 0 && e >= R * kF32K / 4) break;
+        const int r = KC ? e / (kF32K / 4) : 4 * (e % (R / 4)), kk = KC ? 4 * (e % (kF32K / 4)) : e / (R / 4);
+        const bool live = r0 + r < n && k0 + kk < K;
+        cp_async16(KC ? &v[buf][r][kk] : &v[buf][kk][r], at(live ? r0 + r : 0, live ? k0 + kk : 0), live);
+      }
+    } else {
+#pragma unroll
+      for (int e0 = 0; e0 < R * kF32K; e0 += THREADS) {
+        const int e = e0 + tid;
+        const int r = KC ? e / kF32K : e % R, kk = KC ? e % kF32K : e / R;
+        const bool live = r0 + r < n && k0 + kk < K;
+        cp_async4(KC ? &v[buf][r][kk] : &v[buf][kk][r], at(live ? r0 + r : 0, live ? k0 + kk : 0), live);
+      }
+    }
   }
-}
+  // this thread's i-th row / column of the tile
+  static __device__ __forceinline__ int index(int t, int i) { return KC ? t + (R / T) * i : T * t + i; }
+  // its T values at k = k4 .. k4 + 3
+  __device__ __forceinline__ void read(int buf, int t, int k4, float (&x)[4][T]) const {
+    if constexpr (KC) {
+#pragma unroll
+      for (int i = 0; i < T; ++i) {
+        const float4 f = *reinterpret_cast<const float4*>(&v[buf][index(t, i)][k4]);
+        x[0][i] = f.x, x[1][i] = f.y, x[2][i] = f.z, x[3][i] = f.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if constexpr (T == 4) {
+          const float4 f = *reinterpret_cast<const float4*>(&v[buf][k4 + q][T * t]);
+          x[q][0] = f.x, x[q][1] = f.y, x[q][2] = f.z, x[q][3] = f.w;
+        } else {
+          const float2 f = *reinterpret_cast<const float2*>(&v[buf][k4 + q][T * t]);
+          x[q][0] = f.x, x[q][1] = f.y;
+        }
+      }
+    }
+  }
+};
 
 template <InnerOp OP, int BM, int BN, int TM, int TN, class LA, class LB, class EP>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
     gemm_f32_kernel(int M, int N, int K, LA la, LB lb, EP ep, int vec_a, int vec_b) {
-  constexpr int BK = 16, kStages = 4, kThreads = (BM / TM) * (BN / TN);
-  constexpr int LDA = BM + 4, LDB = BN + 4;   // rows stay 16-byte aligned
-  static_assert((BM * BK) % (4 * kThreads) == 0 || BM * BK / 4 < kThreads, "A copies per thread");
-  __shared__ __align__(16) float As[kStages][BK][LDA];
-  __shared__ __align__(16) float Bs[kStages][BK][LDB];
+  constexpr int kThreads = (BM / TM) * (BN / TN);
+  static_assert(BM * kF32K % kThreads == 0 && BN * kF32K % kThreads == 0, "copies per thread");
+  using RA = F32Ring<LA::kContigK, BM, TM>;
+  using RB = F32Ring<LB::kContigK, BN, TN>;
+  __shared__ __align__(16) RA As;
+  __shared__ __align__(16) RB Bs;
   pdl_enter();
   const int tid = threadIdx.x;
   const int tx = tid % (BN / TN), ty = tid / (BN / TN);
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   auto load = [&](int buf, int k0) {
-    if (!LA::kContigK && vec_a) {   // 4 m of one k per copy
-      for (int e = tid; e < BM * BK / 4; e += kThreads) {
-        const int mm = 4 * (e % (BM / 4)), kk = e / (BM / 4), m = m0 + mm, k = k0 + kk;
-        const bool live = m < M && k < K;
-        cp_async16(&As[buf][kk][mm], la.addr(live ? m : 0, live ? k : 0), live);
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < (BM * BK + kThreads - 1) / kThreads; ++r) {
-        const int e = tid + r * kThreads;
-        const int mm = LA::kContigK ? e / BK : e % BM, kk = LA::kContigK ? e % BK : e / BM;
-        const int m = m0 + mm, k = k0 + kk;
-        const bool live = m < M && k < K;
-        cp_async4(&As[buf][kk][mm], la.addr(live ? m : 0, live ? k : 0), live);
-      }
-    }
-    if (!LB::kContigK && vec_b) {
-      for (int e = tid; e < BN * BK / 4; e += kThreads) {
-        const int nn = 4 * (e % (BN / 4)), kk = e / (BN / 4), n = n0 + nn, k = k0 + kk;
-        const bool live = n < N && k < K;
-        cp_async16(&Bs[buf][kk][nn], lb.addr(live ? k : 0, live ? n : 0), live);
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < (BN * BK + kThreads - 1) / kThreads; ++r) {
-        const int e = tid + r * kThreads;
-        const int nn = LB::kContigK ? e / BK : e % BN, kk = LB::kContigK ? e % BK : e / BN;
-        const int n = n0 + nn, k = k0 + kk;
-        const bool live = n < N && k < K;
-        cp_async4(&Bs[buf][kk][nn], lb.addr(live ? k : 0, live ? n : 0), live);
-      }
-    }
+    As.template load<kThreads>(buf, k0, m0, M, K, vec_a != 0, [&](int m, int k) { return la.addr(m, k); });
+    Bs.template load<kThreads>(buf, k0, n0, N, K, vec_b != 0, [&](int n, int k) { return lb.addr(k, n); });
   };
   float2 acc[TM][TN / 2];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  const int nk = (K + BK - 1) / BK;
+  const int nk = (K + kF32K - 1) / kF32K;
 #pragma unroll
-  for (int s = 0; s < kStages - 1; ++s) {
-    if (s < nk) load(s, s * BK);
+  for (int s = 0; s < kF32Stages - 1; ++s) {
+    if (s < nk) load(s, s * kF32K);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   for (int t = 0; t < nk; ++t) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(kF32Stages - 2) : "memory");
     __syncthreads();   // slice t has landed for every thread, and slice t - 1 has been read
-    if (t + kStages - 1 < nk) load((t + kStages - 1) % kStages, (t + kStages - 1) * BK);
+    if (t + kF32Stages - 1 < nk) load((t + kF32Stages - 1) % kF32Stages, (t + kF32Stages - 1) * kF32K);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const float* as = &As[t % kStages][0][TM * ty];
-    const float* bs = &Bs[t % kStages][0][TN * tx];
+    const int buf = t % kF32Stages;
     // (padded k are zero on both sides: they add 0 for every inner op)
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[TM], b[TN];
-      lds_row<TM>(as + kk * LDA, a);
-      lds_row<TN>(bs + kk * LDB, b);
+    for (int k4 = 0; k4 < kF32K; k4 += 4) {
+      float a[4][TM], b[4][TN];
+      As.read(buf, ty, k4, a);
+      Bs.read(buf, tx, k4, b);
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+      for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int j = 0; j < TN / 2; ++j) {
-          const float2 aa = make_float2(a[i], a[i]), bb = make_float2(b[2 * j], b[2 * j + 1]);
-          if constexpr (OP == InnerOp::kMul) {
-            acc[i][j] = fma_x2(aa, bb, acc[i][j]);
-          } else {
-            const float2 d = fma_x2(bb, make_float2(-1.f, -1.f), aa);   // a - b
-            if constexpr (OP == InnerOp::kSqDiff) acc[i][j] = fma_x2(d, d, acc[i][j]);
-            else acc[i][j] = add_x2(acc[i][j], make_float2(fabsf(d.x), fabsf(d.y)));
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN / 2; ++j) {
+            const float x = a[q][i], y0 = b[q][2 * j], y1 = b[q][2 * j + 1];
+            if constexpr (!LB::kContigK && OP == InnerOp::kMul) {   // neighbouring columns: two per instruction
+              acc[i][j] = fma_x2(make_float2(x, x), make_float2(y0, y1), acc[i][j]);
+            } else if constexpr (OP == InnerOp::kMul) {
+              acc[i][j].x = fmaf(x, y0, acc[i][j].x);
+              acc[i][j].y = fmaf(x, y1, acc[i][j].y);
+            } else {
+              const float d0 = x - y0, d1 = x - y1;
+              if constexpr (OP == InnerOp::kSqDiff) {
+                acc[i][j].x = fmaf(d0, d0, acc[i][j].x);
+                acc[i][j].y = fmaf(d1, d1, acc[i][j].y);
+              } else {
+                acc[i][j].x += fabsf(d0);
+                acc[i][j].y += fabsf(d1);
+              }
+            }
           }
-        }
     }
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int m = m0 + TM * ty + i, n = n0 + TN * tx + j;
+      const int m = m0 + RA::index(ty, i), n = n0 + RB::index(tx, j);
       if (m < M && n < N) ep(m, n, (j & 1) ? acc[i][j / 2].y : acc[i][j / 2].x);
     }
 }
@@ -245,7 +273,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 template <InnerOp OP, int BM, int BN, int TM, int TN, class LA, class LB, class EP>
 void launch_gemm_f32(int M, int N, int K, const LA& la, const LB& lb, const EP& ep, cudaStream_t st) {
   launch_k(gemm_f32_kernel<OP, BM, BN, TM, TN, LA, LB, EP>, dim3(ceil_div(N, BN), ceil_div(M, BM)),
-           dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, la, lb, ep, la.vec4(M) ? 1 : 0, lb.vec4(N) ? 1 : 0);
+           dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, la, lb, ep, la.vec4(M, K) ? 1 : 0, lb.vec4(N, K) ? 1 : 0);
 }
 
 // Launch; traced as class `cls` (CRL_TRACE_*) with 2 M N K flops of work.  FP32
@@ -289,7 +317,10 @@ struct LoadRowsSplit {
   __device__ const T* addr(int m, int k) const {
     return k < split ? p0 + (size_t)m * ld0 + k : p1 + (size_t)m * ld1 + (k - split);
   }
-  bool vec4(int) const { return false; }
+  // 16-byte pieces along k: one source, aligned rows, whole pieces
+  bool vec4(int, int K) const {
+    return K == split && (reinterpret_cast<uintptr_t>(p0) & 15) == 0 && (ld0 & 3) == 0 && (K & 3) == 0;
+  }
 };
 // B(k, n) = X[k][n] split by columns (row-major X, n contiguous): weight gradient dY^T X.
 template <typename T, typename T0, typename T1>
@@ -304,8 +335,8 @@ struct LoadColsSplit {
   __device__ const T* addr(int k, int n) const {
     return n < split ? p0 + (size_t)k * ld0 + n : p1 + (size_t)k * ld1 + (n - split);
   }
-  // 16-byte pieces: one source, aligned rows, whole pieces
-  bool vec4(int n) const {
+  // the same along n
+  bool vec4(int n, int) const {
     return n == split && (reinterpret_cast<uintptr_t>(p0) & 15) == 0 && (ld0 & 3) == 0 && (n & 3) == 0;
   }
 };
@@ -317,7 +348,7 @@ struct LoadNK {
   int ld;
   __device__ T operator()(int k, int n) const { return p[(size_t)n * ld + k]; }
   __device__ const T* addr(int k, int n) const { return p + (size_t)n * ld + k; }
-  bool vec4(int) const { return false; }
+  bool vec4(int, int K) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (K & 3) == 0; }
 };
 // B(k, n) = W[k][n] (n contiguous).
 template <typename T>
@@ -327,7 +358,7 @@ struct LoadKN {
   int ld;
   __device__ T operator()(int k, int n) const { return p[(size_t)k * ld + n]; }
   __device__ const T* addr(int k, int n) const { return p + (size_t)k * ld + n; }
-  bool vec4(int n) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (n & 3) == 0; }
+  bool vec4(int n, int) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (n & 3) == 0; }
 };
 // A(m, k) = X[k][m]: the transposed operand of dY^T X (m contiguous).
 template <typename T>
@@ -337,7 +368,7 @@ struct LoadTrans {
   int ld;
   __device__ T operator()(int m, int k) const { return p[(size_t)k * ld + m]; }
   __device__ const T* addr(int m, int k) const { return p + (size_t)k * ld + m; }
-  bool vec4(int m) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (m & 3) == 0; }
+  bool vec4(int m, int) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (m & 3) == 0; }
 };
 // A(m, k) = X[m][k] (k contiguous).
 template <typename T>
@@ -347,7 +378,7 @@ struct LoadMK {
   int ld;
   __device__ T operator()(int m, int k) const { return p[(size_t)m * ld + k]; }
   __device__ const T* addr(int m, int k) const { return p + (size_t)m * ld + k; }
-  bool vec4(int) const { return false; }
+  bool vec4(int, int K) const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0 && (K & 3) == 0; }
 };
 
 // ---- epilogues -------------------------------------------------------------
