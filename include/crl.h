@@ -506,7 +506,9 @@ int crl_mlp_saved_bytes(const crl_mlp_desc* d, int32_t M, size_t* bytes);
 int crl_mlp_forward(const crl_mlp_desc* d, const void* params, const float* x0, const float* x1,
                     int32_t M, void* y, void* saved, void* stream);
 /* Given dy [M][out]: writes dparams (flat layout; overwritten) and, if not
- * NULL, dx0 [M][in0] / dx1 [M][in1].  dparams may be NULL (input gradient only). */
+ * NULL, dx0 [M][in0] / dx1 [M][in1].  dparams may be NULL (input gradient only).
+ * The padding between the layout's tensors is set to 0 for CRL_PREC_BF16 and left
+ * as it was for the other dtypes. */
 int crl_mlp_backward(const crl_mlp_desc* d, const void* params, const float* x0, const float* x1,
                      int32_t M, const void* saved, const void* dy, void* dparams, void* dx0,
                      void* dx1, void* stream);
@@ -525,11 +527,22 @@ int crl_infonce_workspace_bytes(const crl_loss_desc* d, int32_t B, int32_t R, si
 int crl_infonce_forward(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
                         void* loss4, void* row_lse, void* col_lse, void* ws, size_t ws_bytes,
                         void* stream);
+/* The same, and a second copy of the total in `total` (device, dtype, one value). */
+int crl_infonce_forward_total(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
+                              void* loss4, void* total, void* row_lse, void* col_lse, void* ws,
+                              size_t ws_bytes, void* stream);
 /* dphi, dpsi [B][R] = dtotal * d loss4[0] / d(phi, psi), using the row/col
  * logsumexp of the forward call.  dtotal: scalar multiplier. */
 int crl_infonce_backward(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
                          const void* row_lse, const void* col_lse, double dtotal, void* dphi,
                          void* dpsi, void* ws, size_t ws_bytes, void* stream);
+/* The same with the multiplier in device memory: dtotal points to one value of
+ * the call's dtype (float for CRL_PREC_BF16), read when the kernels run, so a
+ * caller whose multiplier comes from earlier work on the stream need not wait
+ * for it. */
+int crl_infonce_backward_device_scale(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B,
+                                      int32_t R, const void* row_lse, const void* col_lse, const void* dtotal,
+                                      void* dphi, void* dpsi, void* ws, size_t ws_bytes, void* stream);
 
 /* Allocation-free variant of crl_infonce_forward (the paper has no
  * counterpart; this is a library service).  For callers that must not

@@ -181,10 +181,10 @@ void critic_impl(crl_ctx* c, const float* s, const float* a, const float* g, int
   mlp_forward<T, float>(c->shapes[CRL_NET_PHI], pphi, s, a, B, phi, c->saved[CRL_NET_PHI], st);
   mlp_forward<T, float>(c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, psi, c->saved[CRL_NET_PSI], st);
   const LossSpec ls = loss_spec(cf);
-  infonce_forward<T>(ls, phi, psi, B, cf.repr, loss, rl, cl, c->ws, cf.path, &c->ctr->status,
+  infonce_forward<T>(ls, phi, psi, B, cf.repr, loss, nullptr, rl, cl, c->ws, cf.path, &c->ctr->status,
                      apply ? &c->ctr->t_critic : nullptr, st);
   logit_stats_launch(c, phi, psi, B, sizeof(T) == 8, st);
-  infonce_backward<T>(ls, phi, psi, B, cf.repr, rl, cl, 1.0, dphi, dpsi, c->ws, cf.path, st);
+  infonce_backward<T>(ls, phi, psi, B, cf.repr, rl, cl, 1.0, nullptr, dphi, dpsi, c->ws, cf.path, st);
   mlp_backward<T, float>(c->shapes[CRL_NET_PHI], pphi, s, a, B, c->saved[CRL_NET_PHI], dphi,
                          static_cast<T*>(c->nets[CRL_NET_PHI].grads), nullptr, nullptr, st);
   mlp_backward<T, float>(c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, c->saved[CRL_NET_PSI], dpsi,
@@ -367,16 +367,16 @@ void critic_impl_bf16(crl_ctx* c, const float* s, const float* a, const float* g
     // fused tcgen05 energy stage: no B x B matrix; the gradients land in the encoders' dy buffers
     const char* e = energy_tc_maps(c->etc, B);
     if (e) throw Failure(CRL_E_CUDA, std::string("tensor map: ") + e);
-    energy_tc_forward(c->etc, ls, B, P.y, Q.y, loss, rl, cl, c->etc_ws, status, apply ? &c->ctr->t_critic : nullptr,
+    energy_tc_forward(c->etc, ls, B, P.y, Q.y, loss, nullptr, rl, cl, c->etc_ws, status, apply ? &c->ctr->t_critic : nullptr,
                       st);
     energy_tc_backward(c->etc, ls, B, P.y, Q.y, rl, cl, 1.0, P.dz[P.layers], Q.dz[Q.layers], c->etc_ws, status,
                        st);
   } else {
-    infonce_forward<float>(ls, P.y, Q.y, B, cf.repr, loss, rl, cl, c->ws, CRL_PATH_PLAIN, status,
+    infonce_forward<float>(ls, P.y, Q.y, B, cf.repr, loss, nullptr, rl, cl, c->ws, CRL_PATH_PLAIN, status,
                            apply ? &c->ctr->t_critic : nullptr, st);
-    infonce_backward<float>(ls, P.y, Q.y, B, cf.repr, rl, cl, 1.0, dphi, dpsi, c->ws, CRL_PATH_PLAIN, st);
-    bf_net_load_dy(P, dphi, B, st);
-    bf_net_load_dy(Q, dpsi, B, st);
+    infonce_backward<float>(ls, P.y, Q.y, B, cf.repr, rl, cl, 1.0, nullptr, dphi, dpsi, c->ws, CRL_PATH_PLAIN, st);
+    bf_net_load_dy(P, dphi, B, nullptr, st);
+    bf_net_load_dy(Q, dpsi, B, nullptr, st);
   }
   bf_check(bf_backward(c->groups, pass, 2, status, st));
   if (apply) {
@@ -708,7 +708,6 @@ int crl_create(const crl_config* cfg, crl_ctx** out) {
       EnergyTc& e = c->etc;
       e.R = R;
       e.Bmax = B;
-      e.ldt = B;
       e.X = static_cast<__nv_bfloat16*>(c->dalloc((size_t)B * R * 2));
       e.Y = static_cast<__nv_bfloat16*>(c->dalloc((size_t)B * R * 2));
       e.auxX = static_cast<float*>(c->dalloc((size_t)B * 4));
@@ -1151,30 +1150,81 @@ int crl_infonce_workspace_bytes(const crl_loss_desc* d, int32_t B, int32_t R, si
   });
 }
 
+}  // extern "C"
+
+namespace {
+// total: a second copy of the total, or null.
+void infonce_forward_call(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R, void* loss4,
+                          void* total, void* row_lse, void* col_lse, void* ws, size_t ws_bytes, void* stream) {
+  const LossSpec ls = checked_loss(d);
+  CRL_REQUIRE(phi && psi && loss4 && row_lse && col_lse && ws && B >= 1 && R >= 1, CRL_E_INVALID_ARG,
+              "bad argument");
+  CRL_REQUIRE(ws_bytes >= (d->dtype == CRL_PREC_BF16 ? infonce_bf16_ws_bytes(ls, B, R)
+                                                     : infonce_ws_bytes(ls, B, R, dtype_size(d->dtype), d->path)),
+              CRL_E_SHAPE, "workspace too small");
+  CRL_REQUIRE(ls.loss != CRL_LOSS_FB || B >= 2, CRL_E_SHAPE, "the forward-backward objective needs B >= 2");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (d->dtype == CRL_PREC_BF16)
+    infonce_bf16_forward(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
+                         static_cast<float*>(loss4), static_cast<float*>(total), static_cast<float*>(row_lse),
+                         static_cast<float*>(col_lse), ws, st);
+  else if (d->dtype == CRL_PREC_FP64)
+    infonce_forward<double>(ls, static_cast<const double*>(phi), static_cast<const double*>(psi), B, R,
+                            static_cast<double*>(loss4), static_cast<double*>(total), static_cast<double*>(row_lse),
+                            static_cast<double*>(col_lse), ws, d->path, nullptr, nullptr, st);
+  else
+    infonce_forward<float>(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
+                           static_cast<float*>(loss4), static_cast<float*>(total), static_cast<float*>(row_lse),
+                           static_cast<float*>(col_lse), ws, d->path, nullptr, nullptr, st);
+  check_launch("infonce forward");
+}
+
+// dtotal_dev: the multiplier as a device scalar of the call's dtype (float for BF16), or null: dtotal.
+void infonce_backward_call(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
+                           const void* row_lse, const void* col_lse, double dtotal, const void* dtotal_dev, void* dphi,
+                           void* dpsi, void* ws, size_t ws_bytes, void* stream) {
+  const LossSpec ls = checked_loss(d);
+  CRL_REQUIRE(phi && psi && row_lse && col_lse && dphi && dpsi && ws && B >= 1 && R >= 1, CRL_E_INVALID_ARG,
+              "bad argument");
+  CRL_REQUIRE(ws_bytes >= (d->dtype == CRL_PREC_BF16 ? infonce_bf16_ws_bytes(ls, B, R)
+                                                     : infonce_ws_bytes(ls, B, R, dtype_size(d->dtype), d->path)),
+              CRL_E_SHAPE, "workspace too small");
+  CRL_REQUIRE(ls.loss != CRL_LOSS_FB || B >= 2, CRL_E_SHAPE, "the forward-backward objective needs B >= 2");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (d->dtype == CRL_PREC_BF16)
+    infonce_bf16_backward(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
+                          static_cast<const float*>(row_lse), static_cast<const float*>(col_lse), dtotal,
+                          static_cast<const float*>(dtotal_dev), static_cast<float*>(dphi),
+                          static_cast<float*>(dpsi), ws, st);
+  else if (d->dtype == CRL_PREC_FP64)
+    infonce_backward<double>(ls, static_cast<const double*>(phi), static_cast<const double*>(psi), B, R,
+                             static_cast<const double*>(row_lse), static_cast<const double*>(col_lse), dtotal,
+                             static_cast<const double*>(dtotal_dev), static_cast<double*>(dphi),
+                             static_cast<double*>(dpsi), ws, d->path, st);
+  else
+    infonce_backward<float>(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
+                            static_cast<const float*>(row_lse), static_cast<const float*>(col_lse), dtotal,
+                            static_cast<const float*>(dtotal_dev), static_cast<float*>(dphi),
+                            static_cast<float*>(dpsi), ws, d->path, st);
+  check_launch("infonce backward");
+}
+}  // namespace
+
+extern "C" {
+
 int crl_infonce_forward(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R, void* loss4,
                         void* row_lse, void* col_lse, void* ws, size_t ws_bytes, void* stream) {
   return guarded(nullptr, [&] {
-    const LossSpec ls = checked_loss(d);
-    CRL_REQUIRE(phi && psi && loss4 && row_lse && col_lse && ws && B >= 1 && R >= 1, CRL_E_INVALID_ARG,
-                "bad argument");
-    CRL_REQUIRE(ws_bytes >= (d->dtype == CRL_PREC_BF16 ? infonce_bf16_ws_bytes(ls, B, R)
-                                                       : infonce_ws_bytes(ls, B, R, dtype_size(d->dtype), d->path)),
-                CRL_E_SHAPE, "workspace too small");
-    CRL_REQUIRE(ls.loss != CRL_LOSS_FB || B >= 2, CRL_E_SHAPE, "the forward-backward objective needs B >= 2");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (d->dtype == CRL_PREC_BF16)
-      infonce_bf16_forward(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
-                           static_cast<float*>(loss4), static_cast<float*>(row_lse), static_cast<float*>(col_lse), ws,
-                           st);
-    else if (d->dtype == CRL_PREC_FP64)
-      infonce_forward<double>(ls, static_cast<const double*>(phi), static_cast<const double*>(psi), B, R,
-                              static_cast<double*>(loss4), static_cast<double*>(row_lse),
-                              static_cast<double*>(col_lse), ws, d->path, nullptr, nullptr, st);
-    else
-      infonce_forward<float>(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
-                             static_cast<float*>(loss4), static_cast<float*>(row_lse), static_cast<float*>(col_lse),
-                             ws, d->path, nullptr, nullptr, st);
-    check_launch("infonce forward");
+    infonce_forward_call(d, phi, psi, B, R, loss4, nullptr, row_lse, col_lse, ws, ws_bytes, stream);
+  });
+}
+
+int crl_infonce_forward_total(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
+                              void* loss4, void* total, void* row_lse, void* col_lse, void* ws, size_t ws_bytes,
+                              void* stream) {
+  return guarded(nullptr, [&] {
+    CRL_REQUIRE(total, CRL_E_INVALID_ARG, "bad argument");
+    infonce_forward_call(d, phi, psi, B, R, loss4, total, row_lse, col_lse, ws, ws_bytes, stream);
   });
 }
 
@@ -1182,27 +1232,16 @@ int crl_infonce_backward(const crl_loss_desc* d, const void* phi, const void* ps
                          const void* row_lse, const void* col_lse, double dtotal, void* dphi, void* dpsi, void* ws,
                          size_t ws_bytes, void* stream) {
   return guarded(nullptr, [&] {
-    const LossSpec ls = checked_loss(d);
-    CRL_REQUIRE(phi && psi && row_lse && col_lse && dphi && dpsi && ws && B >= 1 && R >= 1, CRL_E_INVALID_ARG,
-                "bad argument");
-    CRL_REQUIRE(ws_bytes >= (d->dtype == CRL_PREC_BF16 ? infonce_bf16_ws_bytes(ls, B, R)
-                                                       : infonce_ws_bytes(ls, B, R, dtype_size(d->dtype), d->path)),
-                CRL_E_SHAPE, "workspace too small");
-    CRL_REQUIRE(ls.loss != CRL_LOSS_FB || B >= 2, CRL_E_SHAPE, "the forward-backward objective needs B >= 2");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (d->dtype == CRL_PREC_BF16)
-      infonce_bf16_backward(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
-                            static_cast<const float*>(row_lse), static_cast<const float*>(col_lse), dtotal,
-                            static_cast<float*>(dphi), static_cast<float*>(dpsi), ws, st);
-    else if (d->dtype == CRL_PREC_FP64)
-      infonce_backward<double>(ls, static_cast<const double*>(phi), static_cast<const double*>(psi), B, R,
-                               static_cast<const double*>(row_lse), static_cast<const double*>(col_lse), dtotal,
-                               static_cast<double*>(dphi), static_cast<double*>(dpsi), ws, d->path, st);
-    else
-      infonce_backward<float>(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
-                              static_cast<const float*>(row_lse), static_cast<const float*>(col_lse), dtotal,
-                              static_cast<float*>(dphi), static_cast<float*>(dpsi), ws, d->path, st);
-    check_launch("infonce backward");
+    infonce_backward_call(d, phi, psi, B, R, row_lse, col_lse, dtotal, nullptr, dphi, dpsi, ws, ws_bytes, stream);
+  });
+}
+
+int crl_infonce_backward_device_scale(const crl_loss_desc* d, const void* phi, const void* psi, int32_t B, int32_t R,
+                                      const void* row_lse, const void* col_lse, const void* dtotal, void* dphi,
+                                      void* dpsi, void* ws, size_t ws_bytes, void* stream) {
+  return guarded(nullptr, [&] {
+    CRL_REQUIRE(dtotal, CRL_E_INVALID_ARG, "bad argument");
+    infonce_backward_call(d, phi, psi, B, R, row_lse, col_lse, 1.0, dtotal, dphi, dpsi, ws, ws_bytes, stream);
   });
 }
 

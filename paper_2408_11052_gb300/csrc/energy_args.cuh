@@ -65,6 +65,7 @@ struct FwdArgs {
   float* r_out;
   float* c_out;
   float* loss4;
+  float* total_out;   // may be null: a second copy of the total
   int* t_bump;
   unsigned* tickets;  // [2 n + 1]: per row tile (chunks), per column tile (row tiles), final (zero between launches)
   float* tile_part;   // [2][n][3]: per row / column tile (sum of (lse - diag), sum of lse^2, objective value)
@@ -90,7 +91,14 @@ struct BwdArgs {
   unsigned* status;
   float* d_out_f32;        // non-null: the gradient as FP32 [B][R] here instead of d_out
   const float* other_f32;  // [B][R] FP32 representation of the other side (the -L1 energy)
+  const float* dtotal_dev;  // non-null: the multiplier is read here instead of dtotal / scale
 };
+// The backward's multiplier and multiplier / B.  The quotient of two floats rounded
+// to float is the same whether or not it passes through a double first.
+__device__ __forceinline__ float bwd_dtotal(const BwdArgs& a) { return a.dtotal_dev ? __ldg(a.dtotal_dev) : a.dtotal; }
+__device__ __forceinline__ float bwd_scale(const BwdArgs& a, float dtotal) {
+  return a.dtotal_dev ? __fdiv_rn(dtotal, (float)a.B) : a.scale;
+}
 
 struct HCoef {
   float a_own;    // own auxiliary (|x|^2 for the L2 energies)

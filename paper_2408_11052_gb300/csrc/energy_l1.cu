@@ -350,12 +350,13 @@ __global__ void __launch_bounds__(kBwdT, 1) l1_bwd_kernel(const __grid_constant_
   // row penalty own; column pass: backward direction and column penalty own)
   const float w_own = a.transposed ? a.w.wb : a.w.wf, p_own = a.transposed ? a.w.pc : a.w.pr;
   const float w_oth = a.transposed ? a.w.wf : a.w.wb, p_oth = a.transposed ? a.w.pr : a.w.pc;
-  const float k_diag = a.scale * (a.w.wf + a.w.wb);
+  const float dtotal = bwd_dtotal(a), scale = bwd_scale(a, dtotal);
+  const float k_diag = scale * (a.w.wf + a.w.wb);
   HCoef hc = {};
-  hc.dtotal = a.dtotal;
-  hc.c_bb = a.dtotal / ((float)B * (float)B);
-  hc.c_b = a.dtotal / (float)B;
-  hc.c_fb = B > 1 ? a.dtotal / ((float)B * (float)(B - 1)) : 0.f;
+  hc.dtotal = dtotal;
+  hc.c_bb = dtotal / ((float)B * (float)B);
+  hc.c_b = dtotal / (float)B;
+  hc.c_fb = B > 1 ? dtotal / ((float)B * (float)(B - 1)) : 0.f;
   constexpr bool kAnchored = OBJ == kObjDPO || OBJ == kObjIPO;
   float l_own2[4], k_own[4], d_own[4], kd_own[4];
 #pragma unroll
@@ -363,11 +364,11 @@ __global__ void __launch_bounds__(kBwdT, 1) l1_bwd_kernel(const __grid_constant_
     const int u = u0 + 16 * wa + la + 4 * al;
     const float l = u < B ? a.lse_own[u] : 0.f;
     l_own2[al] = l * kLog2eF;
-    k_own[al] = a.scale * (w_own + 2.f * a.beta * p_own * l);
+    k_own[al] = scale * (w_own + 2.f * a.beta * p_own * l);
     d_own[al] = (kAnchored && u < B) ? a.dpre[u] : 0.f;
     kd_own[al] = (kAnchored && u < B) ? a.kd[u] : 0.f;
   }
-  const float kb_oth = a.scale * w_oth, k2_oth = 2.f * a.scale * a.beta * p_oth;
+  const float kb_oth = scale * w_oth, k2_oth = 2.f * scale * a.beta * p_oth;
 
   // sign-sum roles: own rows w + 16 a, float4 columns lane + 32 c
   bool kv[2];

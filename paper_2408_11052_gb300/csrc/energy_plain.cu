@@ -294,7 +294,7 @@ inline bool has_rows_pass(int obj) { return obj >= CRL_LOSS_FB; }
 template <typename T>
 __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__ F, int ldf, const T* __restrict__ r,
                                                    const T* __restrict__ c, const T* __restrict__ ov, DirWeights w,
-                                                   double beta, T* __restrict__ loss4, unsigned* status,
+                                                   double beta, T* __restrict__ loss4, T* total_out, unsigned* status,
                                                    int* t_bump) {
   pdl_enter();
   __shared__ T sm[5][32];   // 1024 threads: 32 warps
@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__
     loss4[1] = lf;
     loss4[2] = lb;
     loss4[3] = pen;
+    if (total_out) *total_out = total;
     if (status && !finite_val(total)) atomicOr(status, CRL_STATUS_NONFINITE);
     if (t_bump) *t_bump += 1;
   }
@@ -346,14 +347,17 @@ template <typename T>
 __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ F, const T* __restrict__ r,
                                                         const T* __restrict__ c, const T* __restrict__ dg,
                                                         const T* __restrict__ kd, DirWeights w, double beta,
-                                                        double dtotal, int energy, double tau, T* __restrict__ rsum) {
+                                                        double dtotal, const T* __restrict__ dtotal_dev, int energy, double tau,
+                                                        T* __restrict__ rsum) {
   pdl_enter();
   __shared__ T sm[32];
   const int i = blockIdx.x;
   T* __restrict__ row = F + (size_t)i * B;
   const T ri = r[i];
   T sum = 0;
-  const T scale = T(dtotal / B);
+  // (a quotient of two T values rounds the same through a double)
+  const T dt = dtotal_dev ? *dtotal_dev : T(dtotal);
+  const T scale = dtotal_dev ? dt / T(B) : T(dtotal / B);
   const T bb = T(B) * T(B);
   for (int j = threadIdx.x; j < B; j += blockDim.x) {
     const T f = row[j];
@@ -371,7 +375,7 @@ __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ 
         case CRL_LOSS_SPPO: o = T(2) * (f + T(1)) / bb + dlt * T(2) * (f - T(1)) / T(B); break;
         default: o = (sigmoid(f) - dlt) / bb; break;  // NCE-binary
       }
-      g += T(dtotal) * o;
+      g += dt * o;
     }
     T h;
     switch (energy) {
@@ -471,8 +475,8 @@ size_t infonce_ws_bytes(const LossSpec& ls, int B, int R, size_t elem, int path)
 }
 
 template <typename T>
-void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, T* loss4, T* row_lse, T* col_lse,
-                     void* ws, int path, unsigned* status, int* t_bump, cudaStream_t st) {
+void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, T* loss4, T* total, T* row_lse,
+                     T* col_lse, void* ws, int path, unsigned* status, int* t_bump, cudaStream_t st) {
   (void)path;
   PlainWs<T> w = carve_plain<T>(B, R, ws);
   const int nb = ceil_div(B, 8);
@@ -499,13 +503,14 @@ void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int 
   {
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
     launch_k(loss_kernel<T>, dim3(1), dim3(1024), 0, st, B, (const T*)w.F, B, (const T*)row_lse, (const T*)col_lse,
-             rows ? (const T*)w.ov : nullptr, weights(ls), ls.beta, loss4, status, t_bump);
+             rows ? (const T*)w.ov : nullptr, weights(ls), ls.beta, loss4, total, status, t_bump);
   }
 }
 
 template <typename T>
 void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, const T* row_lse,
-                      const T* col_lse, double dtotal, T* dphi, T* dpsi, void* ws, int path, cudaStream_t st) {
+                      const T* col_lse, double dtotal, const T* dtotal_dev, T* dphi, T* dpsi, void* ws, int path,
+                      cudaStream_t st) {
   (void)path;
   PlainWs<T> w = carve_plain<T>(B, R, ws);
   const int nb = ceil_div(B, 8);
@@ -533,7 +538,7 @@ void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int
   {
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
     launch_k(grad_coeff_kernel<T>, dim3(B), dim3(256), 0, st, B, w.F, row_lse, col_lse, (const T*)w.dg,
-             (const T*)w.kd, weights(ls), ls.beta, dtotal, ls.energy, ls.tau, diff ? w.rsum : (T*)nullptr);
+             (const T*)w.kd, weights(ls), ls.beta, dtotal, dtotal_dev, ls.energy, ls.tau, diff ? w.rsum : (T*)nullptr);
   }
   const T* H = w.F;
   if (diff) {
@@ -562,12 +567,12 @@ void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int
 }
 
 template void infonce_forward<float>(const LossSpec&, const float*, const float*, int, int, float*, float*, float*,
-                                     void*, int, unsigned*, int*, cudaStream_t);
-template void infonce_forward<double>(const LossSpec&, const double*, const double*, int, int, double*, double*,
+                                     float*, void*, int, unsigned*, int*, cudaStream_t);
+template void infonce_forward<double>(const LossSpec&, const double*, const double*, int, int, double*, double*, double*,
                                       double*, void*, int, unsigned*, int*, cudaStream_t);
 template void infonce_backward<float>(const LossSpec&, const float*, const float*, int, int, const float*,
-                                      const float*, double, float*, float*, void*, int, cudaStream_t);
+                                      const float*, double, const float*, float*, float*, void*, int, cudaStream_t);
 template void infonce_backward<double>(const LossSpec&, const double*, const double*, int, int, const double*,
-                                       const double*, double, double*, double*, void*, int, cudaStream_t);
+                                       const double*, double, const double*, double*, double*, void*, int, cudaStream_t);
 
 }  // namespace crl

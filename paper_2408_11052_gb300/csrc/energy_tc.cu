@@ -128,60 +128,51 @@ __device__ __forceinline__ float energy_of(int energy, float s, float ax, float 
 }
 
 // ---- representation preparation ------------------------------------------------
-// y [B][R] FP32 -> X [B][R] BF16 (normalised for cos), X^T [R][ldt] BF16, aux [B],
-// for phi and psi in one launch.  Block = 32 rows, one warp per row; the
-// transposed copy goes through a shared tile.
+// y [B][R] FP32 -> X [B][R] BF16 (normalised for cos) and aux [B], for phi and psi
+// in one launch.  Block = 32 rows, one warp per row; the row stays in registers
+// between its norm and its operand (one read; R <= 256).
 struct PrepSide {
   const float* y;
   bf16* X;
-  bf16* XT;
   float* aux;
 };
 // lb: block of 32 rows.
-__device__ __forceinline__ void prep_body(int B, int R, int energy, int ldt, const PrepSide& p, int lb) {
-  const float* __restrict__ y = p.y;
-  bf16* __restrict__ X = p.X;
-  bf16* __restrict__ XT = p.XT;
-  float* __restrict__ aux = p.aux;
-  __shared__ float tile[32][33];
-  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
-  const int row = lb * 32 + w;
-  float scale = 1.f;
-  if (row < B) {
-    const float* yr = y + (size_t)row * R;
-    float q = 0.f;
-    for (int c = lane; c < R; c += 32) {
-      const float v = yr[c];
-      if (energy == CRL_ENERGY_COS) {
-        q += v * v;
-      } else {
-        const float b = __bfloat162float(__float2bfloat16_rn(v));
-        q += b * b;
-      }
+__device__ __forceinline__ void prep_body(int B, int R, int energy, const PrepSide& p, int lb) {
+  const int lane = threadIdx.x % 32, row = lb * 32 + threadIdx.x / 32;
+  if (row >= B) return;
+  const float* __restrict__ yr = p.y + (size_t)row * R;
+  float v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = lane + 32 * k < R ? yr[lane + 32 * k] : 0.f;
+  float q = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    if (lane + 32 * k >= R) break;
+    if (energy == CRL_ENERGY_COS) {
+      q += v[k] * v[k];
+    } else {
+      const float b = __bfloat162float(__float2bfloat16_rn(v[k]));
+      q += b * b;
     }
-    q = warp_sum(q);
-    if (energy == CRL_ENERGY_COS) scale = rsqrtf(q);
-    if (lane == 0) aux[row] = (energy == CRL_ENERGY_COS) ? scale : q;
   }
-  for (int c0 = 0; c0 < R; c0 += 32) {
-    const int c = c0 + lane;
-    float v = 0.f;
-    if (row < B && c < R) {
-      v = y[(size_t)row * R + c] * scale;
-      X[(size_t)row * R + c] = __float2bfloat16_rn(v);
-    }
-    tile[w][lane] = v;
-    __syncthreads();
-    const int cc = c0 + w, rr = lb * 32 + lane;
-    if (XT && cc < R && rr < B) XT[(size_t)cc * ldt + rr] = __float2bfloat16_rn(tile[lane][w]);
-    __syncthreads();
-  }
+  q = warp_sum(q);
+  const float scale = (energy == CRL_ENERGY_COS) ? rsqrtf(q) : 1.f;
+  if (lane == 0) p.aux[row] = (energy == CRL_ENERGY_COS) ? scale : q;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (lane + 32 * k < R) p.X[(size_t)row * R + lane + 32 * k] = __float2bfloat16_rn(v[k] * scale);
 }
 
-// blockIdx.y = 0: phi -> X, 1: psi -> Y.
-__global__ void __launch_bounds__(1024) prep_kernel(int B, int R, int energy, int ldt, PrepSide s0, PrepSide s1) {
+// blockIdx.y = 0: phi -> X, 1: psi -> Y.  z0 / z1: words that the forward wants
+// cleared first (an op-level workspace's status and tickets).
+__global__ void __launch_bounds__(1024) prep_kernel(int B, int R, int energy, PrepSide s0, PrepSide s1, unsigned* z0,
+                                                    int n0, unsigned* z1, int n1) {
   pdl_enter();
-  prep_body(B, R, energy, ldt, blockIdx.y ? s1 : s0, blockIdx.x);
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    for (int i = threadIdx.x; i < n0; i += blockDim.x) z0[i] = 0u;
+    for (int i = threadIdx.x; i < n1; i += blockDim.x) z1[i] = 0u;
+  }
+  prep_body(B, R, energy, blockIdx.y ? s1 : s0, blockIdx.x);
 }
 
 // ---- forward ----------------------------------------------------------------------
@@ -331,6 +322,7 @@ __device__ void finalize_loss(const FwdArgs& a, int n) {
   a.loss4[1] = lf;
   a.loss4[2] = lb;
   a.loss4[3] = pen;
+  if (a.total_out) *a.total_out = total;
   if (a.status && !isfinite(total)) atomicOr(a.status, CRL_STATUS_NONFINITE);
   if (a.t_bump) *a.t_bump += 1;
 }
@@ -1250,9 +1242,10 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
     hc.a_own = a_own;
     hc.l_own = l_own;
     hc.l_own2 = l_own * kLog2e;
-    hc.k_own = a.scale * (w_own + 2.f * a.beta * p_own * l_own);
+    const float dtotal = bwd_dtotal(a), scale = bwd_scale(a, dtotal);
+    hc.k_own = scale * (w_own + 2.f * a.beta * p_own * l_own);
     hc.k_own_tau = hc.k_own * a.inv_tau;
-    hc.k_diag = a.scale * (a.w.wf + a.w.wb);
+    hc.k_diag = scale * (a.w.wf + a.w.wb);
     const bool own_live = w_own != 0.f || (a.beta != 0.f && p_own != 0.f);
     const bool oth_live = w_oth != 0.f || (a.beta != 0.f && p_oth != 0.f);
     const int live = (own_live && oth_live) ? 0 : (oth_live ? 2 : 1);
@@ -1263,13 +1256,13 @@ __device__ __forceinline__ void bwd_body(const CUtensorMap* tmX, const CUtensorM
     hc.kd_own = (kAnchored && u < a.B) ? a.kd[u] : 0.f;
     hc.dpre = a.dpre;
     hc.kd = a.kd;
-    hc.dtotal = a.dtotal;
-    hc.c_bb = a.dtotal / ((float)a.B * (float)a.B);
-    hc.c_b = a.dtotal / (float)a.B;
-    hc.c_fb = a.B > 1 ? a.dtotal / ((float)a.B * (float)(a.B - 1)) : 0.f;
+    hc.dtotal = dtotal;
+    hc.c_bb = dtotal / ((float)a.B * (float)a.B);
+    hc.c_b = dtotal / (float)a.B;
+    hc.c_fb = a.B > 1 ? dtotal / ((float)a.B * (float)(a.B - 1)) : 0.f;
     hc.transposed = a.transposed;
     const int ek = a.energy == CRL_ENERGY_L2 ? 0 : (a.energy == CRL_ENERGY_L2SQ ? 1 : 2);
-    const float kb_oth = a.scale * w_oth, k2_oth = 2.f * a.scale * a.beta * p_oth;
+    const float kb_oth = scale * w_oth, k2_oth = 2.f * scale * a.beta * p_oth;
     // this lane's share of the inputs of columns v0 + 64 h + 16 q ..: the auxiliary
     // of column lane (lanes 0 .. 15) or the logsumexp of column lane - 16
     const float* cin_src = lane < 16 ? a.aux_other : a.lse_other;
@@ -1369,7 +1362,7 @@ struct EnergyTask {   // 128-byte aligned by its tensor maps
   FwdArgs f;
   BwdArgs row, col;
   PrepSide s0, s1;
-  int B, R, energy, ldt, n;
+  int B, R, energy, n;
 };
 
 __global__ void __launch_bounds__(1024) prep_multi_kernel(const EnergyTask* __restrict__ tasks,
@@ -1378,7 +1371,7 @@ __global__ void __launch_bounds__(1024) prep_multi_kernel(const EnergyTask* __re
   int lb, nb;
   const EnergyTask& t = tasks[segment_of(begin, n, blockIdx.x, lb, nb)];
   const int half = nb / 2;
-  prep_body(t.B, t.R, t.energy, t.ldt, lb < half ? t.s0 : t.s1, lb < half ? lb : lb - half);
+  prep_body(t.B, t.R, t.energy, lb < half ? t.s0 : t.s1, lb < half ? lb : lb - half);
 }
 
 template <bool OBJ>
@@ -1481,6 +1474,7 @@ FwdArgs fwd_args(const EnergyTc& e, const LossSpec& ls, int B, void* ws, float* 
   f.r_out = r;
   f.c_out = c;
   f.loss4 = loss4;
+  f.total_out = nullptr;
   f.t_bump = t_bump;
   f.tickets = tickets;
   f.tile_part = tile_part;
@@ -1564,17 +1558,20 @@ const char* energy_tc_maps(EnergyTc& e, int B) {
   return nullptr;
 }
 
-void energy_tc_prepare(EnergyTc& e, const LossSpec& ls, const float* phi, const float* psi, int B, cudaStream_t st) {
+void energy_tc_prepare(EnergyTc& e, const LossSpec& ls, const float* phi, const float* psi, int B, unsigned* status,
+                       void* ws, cudaStream_t st) {
+  const int words = status ? 64 : 0, tickets = status ? (int)(energy_tc_ticket_bytes(B) / 4) : 0;
   if (ls.energy == CRL_ENERGY_L1) return;   // the -L1 tiles read the FP32 rows themselves
   TraceLaunch tr(CRL_TRACE_ENERGY, st, 0.0);
-  launch_k(prep_kernel, dim3(ceil_div(B, 32), 2), dim3(1024), 0, st, B, e.R, ls.energy, e.ldt,
-           PrepSide{phi, e.X, e.XT, e.auxX}, PrepSide{psi, e.Y, e.YT, e.auxY});
+  launch_k(prep_kernel, dim3(ceil_div(B, 32), 2), dim3(1024), 0, st, B, e.R, ls.energy, PrepSide{phi, e.X, e.auxX},
+           PrepSide{psi, e.Y, e.auxY}, status, words, static_cast<unsigned*>(ws), tickets);
 }
 
 void energy_tc_forward(EnergyTc& e, const LossSpec& ls, int B, const float* phi, const float* psi, float* loss4,
-                       float* r, float* c, void* ws, unsigned* status, int* t_bump, cudaStream_t st) {
+                       float* total, float* r, float* c, void* ws, unsigned* status, int* t_bump, cudaStream_t st) {
   const int n = (B + kTile - 1) / kTile;
   FwdArgs a = fwd_args(e, ls, B, ws, loss4, r, c, t_bump, status);
+  a.total_out = total;
   if (ls.energy == CRL_ENERGY_L1) {
     // SIMT tiles, one column tile per chunk
     a.C = 1;
@@ -1682,10 +1679,12 @@ void energy_tc_backward(EnergyTc& e, const LossSpec& ls, int B, const float* phi
 }
 
 void energy_tc_backward_f32(EnergyTc& e, const LossSpec& ls, int B, const float* phi, const float* psi,
-                            const float* r, const float* c, double dtotal, float* dphi, float* dpsi, void* ws,
+                            const float* r, const float* c, double dtotal, const float* dtotal_dev, float* dphi,
+                            float* dpsi, void* ws,
                             unsigned* status, cudaStream_t st) {
   const FwdArgs f = fwd_args(e, ls, B, ws, nullptr, nullptr, nullptr, nullptr, status);
   BwdArgs a = bwd_args(e, ls, B, phi, r, c, dtotal, nullptr, status, f);
+  a.dtotal_dev = dtotal_dev;
   a.d_out_f32 = dphi;
   BwdArgs b = column_args(e, a, psi, r, c);
   b.d_out_f32 = dpsi;
@@ -1704,7 +1703,7 @@ const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& al
     if (g.ls.energy != CRL_ENERGY_L1) {
       agents.push_back(g);
     } else if (stage == 1) {
-      energy_tc_forward(*g.e, g.ls, g.B, g.phi, g.psi, g.loss4, g.r, g.c, g.ws, g.status, g.t_bump, st);
+      energy_tc_forward(*g.e, g.ls, g.B, g.phi, g.psi, g.loss4, nullptr, g.r, g.c, g.ws, g.status, g.t_bump, st);
     } else if (stage == 2) {
       energy_tc_backward(*g.e, g.ls, g.B, g.phi, g.psi, g.r, g.c, 1.0, g.dphi, g.dpsi, g.ws, g.status, st);
     }
@@ -1725,10 +1724,9 @@ const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& al
     t.B = g.B;
     t.R = e.R;
     t.energy = g.ls.energy;
-    t.ldt = e.ldt;
     t.n = (g.B + kTile - 1) / kTile;
-    t.s0 = PrepSide{g.phi, e.X, e.XT, e.auxX};
-    t.s1 = PrepSide{g.psi, e.Y, e.YT, e.auxY};
+    t.s0 = PrepSide{g.phi, e.X, e.auxX};
+    t.s1 = PrepSide{g.psi, e.Y, e.auxY};
     t.f = fwd_args(e, g.ls, g.B, g.ws, g.loss4, g.r, g.c, g.t_bump, g.status);
     t.row = bwd_args(e, g.ls, g.B, g.phi, g.r, g.c, 1.0, g.dphi, g.status, t.f);
     t.col = t.row;

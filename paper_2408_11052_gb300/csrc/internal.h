@@ -111,14 +111,14 @@ struct LossSpec {
   double tau, beta;
 };
 size_t infonce_ws_bytes(const LossSpec& ls, int B, int R, size_t elem, int path);
-// loss4 = {total, fwd, bwd, penalty}.  t_bump: if non-null, ++*t_bump (Adam step counter).
+// loss4 = {total, fwd, bwd, penalty}.  total: if non-null, a second copy of the total.  t_bump: if non-null, ++*t_bump (Adam step counter).
 template <typename T>
-void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, T* loss4, T* row_lse,
+void infonce_forward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, T* loss4, T* total, T* row_lse,
                      T* col_lse, void* ws, int path, unsigned* status, int* t_bump, cudaStream_t st);
 template <typename T>
 void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int R, const T* row_lse,
-                      const T* col_lse, double dtotal, T* dphi, T* dpsi, void* ws, int path,
-                      cudaStream_t st);
+                      const T* col_lse, double dtotal, const T* dtotal_dev, T* dphi, T* dpsi, void* ws, int path,
+                      cudaStream_t st);   // dtotal_dev non-null: the multiplier is that device scalar
 
 // ---------------------------------------------------------------- op-level BF16 (ops_bf16.cu)
 // One encoder on the tensor-core path: params FP32 (flat layout), x0 / x1 /
@@ -132,10 +132,10 @@ void mlp_bf16_backward(const MlpShape& s, const float* params, int M, const void
 // The fused energy stage on FP32 representations phi, psi [B][R]; ws
 // (infonce_bf16_ws_bytes) carries the BF16 operands from a forward to its backward.
 size_t infonce_bf16_ws_bytes(const LossSpec& ls, int B, int R);
-void infonce_bf16_forward(const LossSpec& ls, const float* phi, const float* psi, int B, int R, float* loss4,
+void infonce_bf16_forward(const LossSpec& ls, const float* phi, const float* psi, int B, int R, float* loss4, float* total,
                           float* row_lse, float* col_lse, void* ws, cudaStream_t st);
 void infonce_bf16_backward(const LossSpec& ls, const float* phi, const float* psi, int B, int R, const float* row_lse,
-                           const float* col_lse, double dtotal, float* dphi, float* dpsi, void* ws, cudaStream_t st);
+                           const float* col_lse, double dtotal, const float* dtotal_dev, float* dphi, float* dpsi, void* ws, cudaStream_t st);
 
 // ---------------------------------------------------------------- actor head
 // Entropy-coefficient auto-tuning (the rule is a reading; the paper only says the

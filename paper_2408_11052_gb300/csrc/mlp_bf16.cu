@@ -35,67 +35,61 @@ constexpr float kLnEpsF = 1e-6f;
 inline int pad8(int x) { return (x + 7) / 8 * 8; }
 
 // ---- element kernels ----------------------------------------------------------------
-// 32 x 32 tile transpose-and-pack: src = concat(s0 [rows][n0], s1 [rows][n1]) (FP32)
-// -> dst [rows][ld] (BF16, optional) and dstT [n0 + n1][ldt] (BF16, optional).
-__global__ void __launch_bounds__(256) pack_kernel(int rows, const float* __restrict__ s0, int ld0, int n0,
-                                                  const float* __restrict__ s1, int ld1, int n1, bf16* __restrict__ dst,
-                                                  int ld, bf16* __restrict__ dstT, int ldt) {
+// FP32 rows [rows][n] -> BF16 rows [rows][ld]; four columns per thread where the rows are aligned.
+// gaps: block 0 clears the padding words between the tensors of a flat gradient
+// array (at most 63 after each).
+struct GradGaps {
+  float* grads;   // may be null
+  int n;
+  int64_t off[4 * (CRL_MAX_LAYERS + 1)];
+  int len[4 * (CRL_MAX_LAYERS + 1)];
+};
+__global__ void __launch_bounds__(256) pack_rows_kernel(int rows, int n, const float* __restrict__ src,
+                                                       bf16* __restrict__ dst, int ld, int vec,
+                                                       const __grid_constant__ GradGaps gaps) {
   pdl_enter();
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  const int ncol = n0 + n1;
-  for (int r = ty; r < 32; r += 8) {
-    const int row = r0 + r, col = c0 + tx;
-    float v = 0.f;
-    if (row < rows && col < ncol) v = col < n0 ? s0[(size_t)row * ld0 + col] : s1[(size_t)row * ld1 + (col - n0)];
-    tile[r][tx] = v;
-    if (dst && row < rows && col < ncol) dst[(size_t)row * ld + col] = __float2bfloat16_rn(v);
-  }
-  __syncthreads();
-  if (dstT) {
-    for (int c = ty; c < 32; c += 8) {
-      const int col = c0 + c, row = r0 + tx;
-      if (col < ncol && row < rows) dstT[(size_t)col * ldt + row] = __float2bfloat16_rn(tile[tx][c]);
+  if (blockIdx.x == 0 && gaps.grads)
+    for (int e = threadIdx.x; e < 64 * gaps.n; e += blockDim.x)
+      if (e % 64 < gaps.len[e / 64]) gaps.grads[gaps.off[e / 64] + e % 64] = 0.f;
+  if (vec) {
+    const long long total = (long long)rows * (n / 4);
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+      const long long r = e / (n / 4);
+      const int c = 4 * (int)(e - r * (n / 4));
+      const float4 v = *reinterpret_cast<const float4*>(src + r * n + c);
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+      *reinterpret_cast<uint2*>(dst + r * ld + c) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    }
+  } else {
+    const long long total = (long long)rows * n;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+      const long long r = e / n;
+      dst[r * ld + (e - r * n)] = __float2bfloat16_rn(src[e]);
     }
   }
 }
 
-// Split pack of the network input: x = concat(s0, s1) [rows][ncol] (FP32) ->
-// dst [rows][ld] = (hi_0, lo_0, hi_1, lo_1, ...) and dstT [2 ncol][ldt], with
-// hi = bf16(x), lo = bf16(x - hi).
-__global__ void __launch_bounds__(256) pack_split_kernel(int rows, const float* __restrict__ s0, int ld0, int n0,
-                                                        const float* __restrict__ s1, int ld1, int n1,
-                                                        bf16* __restrict__ dst, int ld, bf16* __restrict__ dstT,
-                                                        int ldt) {
+// One row of the split network input: x = concat(s0, s1) (FP32) -> (hi_0, lo_0,
+// hi_1, lo_1, ...) with hi = bf16(x), lo = bf16(x - hi); one warp, a pair per lane.
+__device__ __forceinline__ void split_row(const float* __restrict__ s0, int n0, const float* __restrict__ s1, int n1,
+                                          bf16* __restrict__ dst, int lane) {
+  for (int c = lane; c < n0 + n1; c += kWarp) {
+    const float v = c < n0 ? s0[c] : s1[c - n0];
+    const bf16 hi = __float2bfloat16_rn(v);
+    __nv_bfloat162 p;
+    p.x = hi;
+    p.y = __float2bfloat16_rn(v - __bfloat162float(hi));
+    reinterpret_cast<__nv_bfloat162*>(dst)[c] = p;
+  }
+}
+__global__ void __launch_bounds__(256) pack_split_kernel(int rows, const float* __restrict__ s0, int n0,
+                                                        const float* __restrict__ s1, int n1, bf16* __restrict__ dst,
+                                                        int ld) {
   pdl_enter();
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  const int ncol = n0 + n1;
-  for (int r = ty; r < 32; r += 8) {
-    const int row = r0 + r, col = c0 + tx;
-    float v = 0.f;
-    if (row < rows && col < ncol) v = col < n0 ? s0[(size_t)row * ld0 + col] : s1[(size_t)row * ld1 + (col - n0)];
-    tile[r][tx] = v;
-    if (row < rows && col < ncol) {
-      const bf16 hi = __float2bfloat16_rn(v);
-      const bf16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-      dst[(size_t)row * ld + 2 * col] = hi;
-      dst[(size_t)row * ld + 2 * col + 1] = lo;
-    }
-  }
-  __syncthreads();
-  if (!dstT) return;
-  for (int c = ty; c < 32; c += 8) {
-    const int col = c0 + c, row = r0 + tx;
-    if (col < ncol && row < rows) {
-      const float v = tile[tx][c];
-      const bf16 hi = __float2bfloat16_rn(v);
-      dstT[(size_t)(2 * col) * ldt + row] = hi;
-      dstT[(size_t)(2 * col + 1) * ldt + row] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
-  }
+  const int row = blockIdx.x * 8 + threadIdx.x / kWarp;
+  if (row >= rows) return;
+  split_row(s0 + (size_t)row * n0, n0, s1 + (size_t)row * n1, n1, dst + (size_t)row * ld, threadIdx.x % kWarp);
 }
 
 // Weight shadows: W [out][ncol] (FP32) -> W2 [out][(nhi + 1) kp] = nhi copies
@@ -103,40 +97,116 @@ __global__ void __launch_bounds__(256) pack_split_kernel(int rows, const float* 
 // `rep` times (first layer: rep = 2 matching the split input, nhi = 1; later
 // layers: rep = 1, nhi = 2 for the hi / lo activations), and the single BF16
 // transpose Wt [ncol][ldt] for the input-gradient product.
-__global__ void __launch_bounds__(256) pack_weights_kernel(int rows, int ncol, int rep, int nhi,
-                                                          const float* __restrict__ W, bf16* __restrict__ W2, int kp,
-                                                          bf16* __restrict__ Wt, int ldt) {
-  pdl_enter();
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+struct ShadowTile {
+  const float* W;   // [rows][ncol]
+  bf16* W2;         // [rows][(nhi + 1) kp]
+  bf16* Wt;         // [ncol][ldt]
+  int rows, ncol, rep, nhi, kp, ldt;
+};
+// A 64 x 64 tile of one layer's shadows, columns up to kp / rep (the padding
+// columns are written as zeros: the tensor cores read them as K).  Two columns per
+// thread and row: 128-byte rows of W2; the transpose leaves by row pairs.
+__device__ __forceinline__ void shadow_tile(const ShadowTile& t, int r0, int c0, float (&tile)[64][65]) {
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int r = ty; r < 32; r += 8) {
-    const int row = r0 + r, col = c0 + tx;
-    float v = 0.f;
-    if (row < rows && col < ncol) {
-      v = W[(size_t)row * ncol + col];
-      const bf16 hi = __float2bfloat16_rn(v);
-      const bf16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-      bf16* d = W2 + (size_t)row * (nhi + 1) * kp;
-      for (int q = 0; q < rep; ++q) {
-        for (int c = 0; c < nhi; ++c) d[c * kp + rep * col + q] = hi;
-        d[nhi * kp + rep * col + q] = lo;
+  const int c = c0 + 2 * tx;
+  for (int r = ty; r < 64; r += 8) {
+    const int row = r0 + r;
+    float v0 = 0.f, v1 = 0.f;
+    if (row < t.rows) {
+      const float* w = t.W + (size_t)row * t.ncol;
+      if (c < t.ncol) v0 = w[c];
+      if (c + 1 < t.ncol) v1 = w[c + 1];
+      if (c < t.kp / t.rep) {   // (a multiple of 32: both columns of the pair)
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
+        bf16* d = t.W2 + (size_t)row * (t.nhi + 1) * t.kp;
+        if (t.rep == 1) {
+          for (int q = 0; q < t.nhi; ++q) *reinterpret_cast<__nv_bfloat162*>(d + q * t.kp + c) = hi;
+          *reinterpret_cast<__nv_bfloat162*>(d + t.nhi * t.kp + c) = lo;
+        } else {   // every column twice
+          __nv_bfloat162 h2[2], l2[2];
+          h2[0] = __bfloat162bfloat162(hi.x), h2[1] = __bfloat162bfloat162(hi.y);
+          l2[0] = __bfloat162bfloat162(lo.x), l2[1] = __bfloat162bfloat162(lo.y);
+          for (int q = 0; q < t.nhi; ++q) *reinterpret_cast<uint2*>(d + q * t.kp + 2 * c) = *reinterpret_cast<uint2*>(h2);
+          *reinterpret_cast<uint2*>(d + t.nhi * t.kp + 2 * c) = *reinterpret_cast<uint2*>(l2);
+        }
       }
     }
-    tile[r][tx] = v;
+    tile[r][2 * tx] = v0;
+    tile[r][2 * tx + 1] = v1;
   }
   __syncthreads();
-  for (int c = ty; c < 32; c += 8) {
-    const int col = c0 + c, row = r0 + tx;
-    if (col < ncol && row < rows) Wt[(size_t)col * ldt + row] = __float2bfloat16_rn(tile[tx][c]);
+  const int row = r0 + 2 * tx;
+  for (int k = ty; k < 64; k += 8) {
+    const int col = c0 + k;
+    if (col >= t.ncol || row >= t.rows) continue;
+    bf16* d = t.Wt + (size_t)col * t.ldt + row;   // (ldt and row are even)
+    const __nv_bfloat162 p = __floats2bfloat162_rn(tile[2 * tx][k], tile[2 * tx + 1][k]);
+    if (row + 1 < t.rows) *reinterpret_cast<__nv_bfloat162*>(d) = p;
+    else *d = p.x;
   }
 }
+__host__ __device__ inline int shadow_tiles_x(const ShadowTile& t) { return (t.kp / t.rep + 63) / 64; }
+__host__ __device__ inline int shadow_tiles(const ShadowTile& t) { return shadow_tiles_x(t) * ((t.rows + 63) / 64); }
 
-void pack(int rows, const float* s0, int ld0, int n0, const float* s1, int ld1, int n1, bf16* dst, int ld, bf16* dstT,
-          int ldt, cudaStream_t st) {
-  TraceLaunch tr(CRL_TRACE_AUX, st, (double)rows * (n0 + n1) * (4.0 + (dst ? 2 : 0) + (dstT ? 2 : 0)));
-  dim3 grid(ceil_div(n0 + n1, 32), ceil_div(rows, 32));
-  launch_k(pack_kernel, grid, dim3(256), 0, st, rows, s0, ld0, n0, s1, ld1, n1, dst, ld, dstT, ldt);
+__global__ void __launch_bounds__(256) pack_weights_kernel(const __grid_constant__ ShadowTile t) {
+  pdl_enter();
+  __shared__ float tile[64][65];
+  const int nx = shadow_tiles_x(t);
+  shadow_tile(t, 64 * ((int)blockIdx.x / nx), 64 * ((int)blockIdx.x % nx), tile);
+}
+
+// Everything an op-level forward needs before its first product, in one launch
+// (it was a memset of the whole workspace and 2 + 2 (layers + 1) launches): the
+// weight shadows of every layer, the split input with its ones column, the ones
+// column and the K padding of every hidden activation, the status word and the
+// split-K tickets.  Blocks [0, wtiles): weight tiles; then 8 rows per block.
+struct NetPrep {
+  ShadowTile L[CRL_MAX_LAYERS + 1];
+  int tile_begin[CRL_MAX_LAYERS + 2];
+  int nl, M;
+  const float *s0, *s1;
+  int n0, n1;
+  bf16* x0;
+  int x0_ld;
+  bf16* h[CRL_MAX_LAYERS];
+  int ldh, hlo, H, kp;   // kp: H rounded up to 64
+  unsigned* status;      // 64 words
+  unsigned* tick[CRL_MAX_LAYERS + 1];
+  int ntick[CRL_MAX_LAYERS + 1];
+};
+__global__ void __launch_bounds__(256) net_prep_kernel(const __grid_constant__ NetPrep p) {
+  pdl_enter();
+  __shared__ float tile[64][65];
+  const int wtiles = p.tile_begin[p.nl], b = blockIdx.x;
+  if (b < wtiles) {
+    int l = 0;
+    while (p.tile_begin[l + 1] <= b) ++l;
+    const ShadowTile& t = p.L[l];
+    const int k = b - p.tile_begin[l], nx = shadow_tiles_x(t);
+    shadow_tile(t, 64 * (k / nx), 64 * (k % nx), tile);
+    return;
+  }
+  const int lane = threadIdx.x % kWarp, row = (b - wtiles) * 8 + threadIdx.x / kWarp;
+  if (b == wtiles) {
+    if (threadIdx.x < 64) p.status[threadIdx.x] = 0u;
+    for (int l = 0; l < p.nl; ++l)
+      for (int i = threadIdx.x; i < p.ntick[l]; i += blockDim.x) p.tick[l][i] = 0u;
+  }
+  if (row >= p.M) return;
+  bf16* x = p.x0 + (size_t)row * p.x0_ld;
+  split_row(p.s0 + (size_t)row * p.n0, p.n0, p.s1 + (size_t)row * p.n1, p.n1, x, lane);
+  const bf16 one = __float2bfloat16_rn(1.f), zero = __float2bfloat16_rn(0.f);
+  if (lane == 0) x[2 * (p.n0 + p.n1)] = one;
+  for (int l = 0; l + 1 < p.nl; ++l) {
+    bf16* h = p.h[l] + (size_t)row * p.ldh;
+    for (int c = p.H + lane; c < p.kp; c += kWarp) {
+      h[c] = zero;
+      h[p.hlo + c] = zero;
+    }
+    __syncwarp();
+    if (lane == 0) h[p.H] = one;
+  }
 }
 
 // LayerNorm kernels: one warp per row, 8 rows per 256-thread block.  Rows of
@@ -473,14 +543,16 @@ const char* mk(CUtensorMap* m, const void* base, int inner, int rows, int stride
   return nullptr;
 }
 
-
-
+static_assert(sizeof(tc::GemmProblem) % 8 == 0, "hashed in 8-byte words");
+// FNV-1a over 8-byte words.
 uint64_t fnv1a(const void* data, size_t n) {
   const unsigned char* p = static_cast<const unsigned char*>(data);
   uint64_t h = 1469598103934665603ull;
-  for (size_t i = 0; i < n; ++i) {
-    h ^= p[i];
-    h *= 1099511628211ull;
+  for (size_t i = 0; i + 8 <= n; i += 8) {
+    uint64_t w;
+    memcpy(&w, p + i, 8);
+    h = (h ^ w) * 1099511628211ull;
+    h ^= h >> 32;   // a word's high bits reach the low ones
   }
   return h;
 }
@@ -834,6 +906,14 @@ void GemmGroups::reset() {
   used_ = cap_ = 0;
 }
 
+namespace {
+// Arrival counters of a layer's weight-gradient product (one per 128 x 64 tile).
+int split_tickets(const BfLayer& L, int l) {
+  const int N = (l == 0) ? 2 * L.in + 1 : L.in + 1;
+  return (int)round_up(ceil_div(L.out, 128) * ceil_div(N, 64), 64);
+}
+}  // namespace
+
 const char* bf_net_carve(BfNet& n, const MlpShape& s, int Mmax, DevAlloc alloc, void* owner, bool weight_maps) {
   n.s = s;
   n.Mmax = Mmax;
@@ -876,7 +956,7 @@ const char* bf_net_carve(BfNet& n, const MlpShape& s, int Mmax, DevAlloc alloc, 
     if (cap < 2) continue;
     const int N = (l == 0) ? 2 * L.in + 1 : L.in + 1;   // the weight-gradient product's columns
     L.wpart = static_cast<float*>(A((size_t)cap * round_up(L.out, 128) * round_up(N, 256) * 4));
-    L.wtick = static_cast<unsigned*>(A((size_t)round_up(ceil_div(L.out, 128) * ceil_div(N, 64), 64) * 4));
+    L.wtick = static_cast<unsigned*>(A((size_t)split_tickets(L, l) * 4));
     if (!L.wpart || !L.wtick) return "device allocation failed";
   }
   const int in = s.in(), out = s.out;
@@ -937,9 +1017,7 @@ const char* bf_net_init(BfNet& n, const MlpShape& s, int Mmax, DevAlloc alloc, v
         cudaMemset(L.Wt, 0, (size_t)L.in * L.out_pad * 2) != cudaSuccess)
       return "cudaMemset failed";
     if (L.wtick) {
-      const int N = (l == 0) ? 2 * L.in + 1 : L.in + 1;
-      if (cudaMemset(L.wtick, 0, (size_t)round_up(ceil_div(L.out, 128) * ceil_div(N, 64), 64) * 4) != cudaSuccess)
-        return "cudaMemset failed";
+      if (cudaMemset(L.wtick, 0, (size_t)split_tickets(L, l) * 4) != cudaSuccess) return "cudaMemset failed";
     }
   }
   for (int l = 0; l <= s.layers; ++l) {
@@ -974,14 +1052,51 @@ const char* bf_net_maps(BfNet& n, int M) {
   return nullptr;
 }
 
+namespace {
+ShadowTile shadow_of(const BfNet& n, int l, const float* params) {
+  const BfLayer& L = n.L[l];
+  return ShadowTile{params + L.oW, L.W, L.Wt, L.out, L.in, l == 0 ? 2 : 1, L.nhi, L.kp, L.out_pad};
+}
+}  // namespace
+
 void bf_net_shadow(BfNet& n, const float* params, cudaStream_t st) {
   for (int l = 0; l <= n.layers; ++l) {
-    BfLayer& L = n.L[l];
-    TraceLaunch tr(CRL_TRACE_AUX, st, (double)L.out * L.in * 10.0);
-    dim3 grid(ceil_div(L.in, 32), ceil_div(L.out, 32));
-    launch_k(pack_weights_kernel, grid, dim3(256), 0, st, L.out, L.in, l == 0 ? 2 : 1, L.nhi, params + L.oW, L.W, L.kp,
-             L.Wt, L.out_pad);
+    TraceLaunch tr(CRL_TRACE_AUX, st, (double)n.L[l].out * n.L[l].in * 10.0);
+    const ShadowTile t = shadow_of(n, l, params);
+    launch_k(pack_weights_kernel, dim3(shadow_tiles(t)), dim3(256), 0, st, t);
   }
+}
+
+void bf_net_prepare(BfNet& n, const float* params, const float* x0, const float* x1, int M, unsigned* status,
+                    cudaStream_t st) {
+  NetPrep p;
+  memset(&p, 0, sizeof(p));
+  p.nl = n.layers + 1;
+  p.M = M;
+  double bytes = (double)M * n.s.in() * 8.0;
+  for (int l = 0; l <= n.layers; ++l) {
+    p.L[l] = shadow_of(n, l, params);
+    p.tile_begin[l + 1] = p.tile_begin[l] + shadow_tiles(p.L[l]);
+    if (n.L[l].wtick) {
+      p.tick[l] = n.L[l].wtick;
+      p.ntick[l] = split_tickets(n.L[l], l);
+    }
+    bytes += (double)n.L[l].out * n.L[l].in * 10.0;
+  }
+  p.s0 = x0;
+  p.s1 = x1;
+  p.n0 = n.s.in0;
+  p.n1 = n.s.in1;
+  p.x0 = n.x0;
+  p.x0_ld = bf_net_x0_ld(n);
+  for (int l = 0; l < n.layers; ++l) p.h[l] = n.h[l];
+  p.ldh = n.ldh;
+  p.hlo = n.hlo;
+  p.H = n.s.hidden;
+  p.kp = (n.s.hidden + 63) / 64 * 64;
+  p.status = status;
+  TraceLaunch tr(CRL_TRACE_AUX, st, bytes);
+  launch_k(net_prep_kernel, dim3(p.tile_begin[p.nl] + ceil_div(M, 8)), dim3(256), 0, st, p);
 }
 
 int bf_net_x0_ld(const BfNet& n) { return pad8(2 * n.s.in() + 1); }
@@ -989,14 +1104,31 @@ int bf_net_x0_ld(const BfNet& n) { return pad8(2 * n.s.in() + 1); }
 void bf_net_pack_input(BfNet& n, const float* x0, const float* x1, int M, cudaStream_t st) {
   const int in = n.s.in();
   TraceLaunch tr(CRL_TRACE_AUX, st, (double)M * in * 12.0);
-  dim3 grid(ceil_div(in, 32), ceil_div(M, 32));
-  launch_k(pack_split_kernel, grid, dim3(256), 0, st, M, x0, n.s.in0, n.s.in0, x1, n.s.in1, n.s.in1, n.x0,
-           bf_net_x0_ld(n), (bf16*)nullptr, 0);
+  launch_k(pack_split_kernel, dim3(ceil_div(M, 8)), dim3(256), 0, st, M, x0, n.s.in0, x1, n.s.in1, n.x0, bf_net_x0_ld(n));
 }
 
-void bf_net_load_dy(BfNet& n, const float* dy, int M, cudaStream_t st) {
+void bf_net_load_dy(BfNet& n, const float* dy, int M, float* grads, cudaStream_t st) {
   const int out = n.s.out;
-  pack(M, dy, out, out, nullptr, 0, 0, n.dz[n.layers], pad8(out), nullptr, 0, st);
+  GradGaps gaps;
+  gaps.grads = grads;
+  gaps.n = 0;
+  auto pad = [&](int64_t off, int64_t len) {
+    const int rest = (int)(round_up(len, 64) - len);
+    if (off < 0 || rest == 0) return;
+    gaps.off[gaps.n] = off + len;
+    gaps.len[gaps.n++] = rest;
+  };
+  for (int l = 0; grads && l <= n.layers; ++l) {
+    const BfLayer& L = n.L[l];
+    pad(L.oW, (int64_t)L.in * L.out);
+    pad(L.ob, L.out);
+    pad(L.og, L.out);
+    pad(L.obeta, L.out);
+  }
+  TraceLaunch tr(CRL_TRACE_AUX, st, (double)M * out * 6.0);
+  const int vec = out % 4 == 0 && (reinterpret_cast<uintptr_t>(dy) & 15) == 0 ? 1 : 0;
+  const int blocks = (int)std::min<int64_t>(ceil_div((int64_t)M * out / (vec ? 4 : 1) + 1, 256), 152 * 8);
+  launch_k(pack_rows_kernel, dim3(blocks), dim3(256), 0, st, M, out, dy, n.dz[n.layers], pad8(out), vec, gaps);
 }
 
 namespace {

@@ -91,11 +91,11 @@ extern "C" int crl_infonce_forward_noalloc(const crl_loss_desc* d, const void* p
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (d->dtype == CRL_PREC_FP64)
       infonce_forward<double>(ls, static_cast<const double*>(phi), static_cast<const double*>(psi), B, R,
-                              static_cast<double*>(loss4), static_cast<double*>(row_lse),
+                              static_cast<double*>(loss4), nullptr, static_cast<double*>(row_lse),
                               static_cast<double*>(col_lse), ws, d->path, nullptr, nullptr, st);
     else
       infonce_forward<float>(ls, static_cast<const float*>(phi), static_cast<const float*>(psi), B, R,
-                             static_cast<float*>(loss4), static_cast<float*>(row_lse), static_cast<float*>(col_lse),
+                             static_cast<float*>(loss4), nullptr, static_cast<float*>(row_lse), static_cast<float*>(col_lse),
                              ws, d->path, nullptr, nullptr, st);
     check_launch("allocation-free infonce forward");
   });

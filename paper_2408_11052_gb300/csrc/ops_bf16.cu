@@ -50,8 +50,17 @@ GemmGroups& ops_groups() {
   return *g;
 }
 
+// Tensor maps are encoded by the driver API, which wants a current context: a
+// thread that has made no runtime call yet (an autograd worker) has none.
+void bind_context() {
+  int dev = 0;
+  CRL_CHECK_CUDA(cudaGetDevice(&dev));
+  CRL_CHECK_CUDA(cudaSetDevice(dev));
+}
+
 // The network's BF16 buffers laid out in `saved` (after the status word) for M rows.
 const char* carve_net(BfNet& n, const MlpShape& s, int M, void* saved) {
+  bind_context();
   Carver c{static_cast<char*>(saved) + kStatusBytes, 0};
   if (const char* e = bf_net_carve(n, s, M, carve_piece, &c, true)) return e;
   return bf_net_maps(n, M);
@@ -69,13 +78,8 @@ void mlp_bf16_forward(const MlpShape& s, const float* params, const float* x0, c
   std::lock_guard<std::mutex> lock(g_ops_mutex);
   BfNet n;
   if (const char* e = carve_net(n, s, M, saved)) throw Failure(CRL_E_INVALID_ARG, e);
-  // a fresh workspace: zero it (padding columns of the weight shadows are read
-  // as K by the tensor cores; the LayerNorm ticket starts at zero), then the
-  // ones rows, the weight shadows and the split input
-  CRL_CHECK_CUDA(cudaMemsetAsync(saved, 0, mlp_bf16_saved_bytes(s, M), st));
-  bf_net_fill_ones(n, st);
-  bf_net_shadow(n, params, st);
-  bf_net_pack_input(n, x0, x1, M, st);
+  // a fresh workspace holds anything: what the products read is written here
+  bf_net_prepare(n, params, x0, x1, M, static_cast<unsigned*>(saved), st);
   n.y = y;
   BfPass p{&n, params, nullptr, nullptr, M};
   if (const char* e = bf_forward(ops_groups(), &p, 1, static_cast<unsigned*>(saved), st))
@@ -88,7 +92,7 @@ void mlp_bf16_backward(const MlpShape& s, const float* params, int M, const void
   BfNet n;
   void* sv = const_cast<void*>(saved);   // the backward writes its dz buffers there
   if (const char* e = carve_net(n, s, M, sv)) throw Failure(CRL_E_INVALID_ARG, e);
-  bf_net_load_dy(n, dy, M, st);
+  bf_net_load_dy(n, dy, M, dparams, st);
   BfPass p{&n, params, dparams, dx1, M};
   p.dx0 = dx0;
   if (const char* e = bf_backward(ops_groups(), &p, 1, static_cast<unsigned*>(sv), st))
@@ -105,16 +109,15 @@ struct EnergyWs {
   unsigned* status;
 };
 const char* carve_energy(EnergyWs& w, const LossSpec& ls, int B, int R, void* ws) {
+  bind_context();
   char* base = static_cast<char*>(ws);
   w.status = reinterpret_cast<unsigned*>(base);
   Carver c{base + kStatusBytes, 0};
   w.ews = carve_piece(&c, energy_tc_ws_bytes(ls, B, R));
   w.e.R = R;
   w.e.Bmax = B;
-  w.e.ldt = 0;
   w.e.X = static_cast<__nv_bfloat16*>(carve_piece(&c, (size_t)B * R * 2));
   w.e.Y = static_cast<__nv_bfloat16*>(carve_piece(&c, (size_t)B * R * 2));
-  w.e.XT = w.e.YT = nullptr;
   w.e.auxX = static_cast<float*>(carve_piece(&c, (size_t)B * 4));
   w.e.auxY = static_cast<float*>(carve_piece(&c, (size_t)B * 4));
   w.e.tm_B = -1;
@@ -142,27 +145,30 @@ size_t infonce_bf16_ws_bytes(const LossSpec& ls, int B, int R) {
 }
 
 void infonce_bf16_forward(const LossSpec& ls, const float* phi, const float* psi, int B, int R, float* loss4,
-                          float* row_lse, float* col_lse, void* ws, cudaStream_t st) {
+                          float* total, float* row_lse, float* col_lse, void* ws, cudaStream_t st) {
   const char* why = nullptr;
   if (!energy_tc_supported(ls, B, R, &why)) throw Failure(CRL_E_UNSUPPORTED, why);
   check_l1_alignment(ls, phi, psi, nullptr, nullptr);
   EnergyWs w;
   if (const char* e = carve_energy(w, ls, B, R, ws)) throw Failure(CRL_E_INVALID_ARG, e);
-  // status word and tickets start at zero
-  CRL_CHECK_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
-  CRL_CHECK_CUDA(cudaMemsetAsync(w.ews, 0, energy_tc_ticket_bytes(B), st));
-  energy_tc_prepare(w.e, ls, phi, psi, B, st);
-  energy_tc_forward(w.e, ls, B, phi, psi, loss4, row_lse, col_lse, w.ews, w.status, nullptr, st);
+  // status word and tickets start at zero: cleared by the operand launch, which -L1 does not have
+  if (ls.energy == CRL_ENERGY_L1) {
+    CRL_CHECK_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
+    CRL_CHECK_CUDA(cudaMemsetAsync(w.ews, 0, energy_tc_ticket_bytes(B), st));
+  }
+  energy_tc_prepare(w.e, ls, phi, psi, B, w.status, w.ews, st);
+  energy_tc_forward(w.e, ls, B, phi, psi, loss4, total, row_lse, col_lse, w.ews, w.status, nullptr, st);
 }
 
 void infonce_bf16_backward(const LossSpec& ls, const float* phi, const float* psi, int B, int R, const float* row_lse,
-                           const float* col_lse, double dtotal, float* dphi, float* dpsi, void* ws, cudaStream_t st) {
+                           const float* col_lse, double dtotal, const float* dtotal_dev, float* dphi, float* dpsi,
+                           void* ws, cudaStream_t st) {
   const char* why = nullptr;
   if (!energy_tc_supported(ls, B, R, &why)) throw Failure(CRL_E_UNSUPPORTED, why);
   check_l1_alignment(ls, phi, psi, dphi, dpsi);
   EnergyWs w;
   if (const char* e = carve_energy(w, ls, B, R, ws)) throw Failure(CRL_E_INVALID_ARG, e);
-  energy_tc_backward_f32(w.e, ls, B, phi, psi, row_lse, col_lse, dtotal, dphi, dpsi, w.ews, w.status, st);
+  energy_tc_backward_f32(w.e, ls, B, phi, psi, row_lse, col_lse, dtotal, dtotal_dev, dphi, dpsi, w.ews, w.status, st);
 }
 
 }  // namespace crl
