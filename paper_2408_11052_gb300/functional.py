@@ -13,6 +13,7 @@ saved with the graph, so several forwards may precede their backwards.
 """
 
 from ctypes import byref, c_size_t
+from functools import lru_cache
 
 import torch
 
@@ -31,6 +32,30 @@ def _dtype_code(t, precision=None):
     raise TypeError("parameters must be float32 or float64")
 
 
+# Descriptors and workspace sizes depend on shapes and options alone: kept per value (typed: 17.0 and
+# numpy.int64(17) are refused as field values whether or not 17 was seen).
+@lru_cache(maxsize=256, typed=True)
+def _mlp_plan(in0, in1, hidden, layers, out, layernorm, dtype, M):
+    desc = api.CrlMlpDesc(in0, in1, hidden, layers, out, layernorm, dtype)
+    nbytes = c_size_t()
+    api.check(api.lib().crl_mlp_saved_bytes(byref(desc), M, byref(nbytes)))
+    # elements of the flat layout: every tensor padded to 64
+    dims = [in0 + in1] + [hidden] * layers + [out]
+    count = sum(-(-n // 64) * 64 for a, b in zip(dims, dims[1:]) for n in (a * b, b))
+    if layernorm:
+        count += 2 * layers * (-(-hidden // 64) * 64)
+    return desc, nbytes.value, count
+
+
+@lru_cache(maxsize=256, typed=True)
+def _loss_plan(energy, loss, sym_reduction, penalty_axis, temperature, beta, dtype, path, B, R):
+    desc = api.CrlLossDesc(api.ENERGY[energy], api.LOSS[loss], api.SYM[sym_reduction], api.PENALTY[penalty_axis],
+                           temperature, beta, dtype, api.PATH[path])
+    nbytes = c_size_t()
+    api.check(api.lib().crl_infonce_workspace_bytes(byref(desc), B, R, byref(nbytes)))
+    return desc, nbytes.value
+
+
 class EncoderMLP(torch.autograd.Function):
     """y = MLP(concat(x0, x1)) with params in the flat layout of include/crl.h.
 
@@ -42,19 +67,19 @@ class EncoderMLP(torch.autograd.Function):
     @staticmethod
     def forward(ctx, params, x0, x1, in0, in1, hidden, layers, out, layernorm, precision=None):
         L = api.lib()
-        desc = api.CrlMlpDesc(in0, in1, hidden, layers, out, int(layernorm), _dtype_code(params, precision))
         M = x0.shape[0]
-        nbytes = c_size_t()
-        api.check(L.crl_mlp_saved_bytes(byref(desc), M, byref(nbytes)))
-        saved = torch.empty(nbytes.value, dtype=torch.uint8, device=params.device)
+        desc, nbytes, count = _mlp_plan(in0, in1, hidden, layers, out, int(layernorm),
+                                        _dtype_code(params, precision), M)
+        saved = torch.empty(nbytes, dtype=torch.uint8, device=params.device)
         y = torch.empty(M, out, dtype=params.dtype, device=params.device)
         x0c = x0.detach().contiguous().float()
         x1c = None if x1 is None else x1.detach().contiguous().float()
         api.check(L.crl_mlp_forward(byref(desc), params.data_ptr(), x0c.data_ptr(),
                                     None if x1c is None else x1c.data_ptr(), M, y.data_ptr(), saved.data_ptr(),
                                     api.stream_handle()))
-        ctx.desc = (in0, in1, hidden, layers, out, int(layernorm))
-        ctx.precision = precision
+        ctx.desc = desc
+        # the BF16 backward writes the whole layout, its padding too
+        ctx.whole = desc.dtype == api.PREC["bf16"] and params.numel() == count
         ctx.has_x1 = x1 is not None
         ctx.save_for_backward(params, x0c, x1c if x1c is not None else x0c, saved)
         return y
@@ -65,11 +90,11 @@ class EncoderMLP(torch.autograd.Function):
         params, x0c, x1c, saved = ctx.saved_tensors
         if not ctx.has_x1:
             x1c = None
-        desc = api.CrlMlpDesc(*ctx.desc, _dtype_code(params, ctx.precision))
+        desc = ctx.desc
         M = x0c.shape[0]
-        dparams = torch.zeros_like(params) if ctx.needs_input_grad[0] else None
-        dx0 = torch.empty(M, ctx.desc[0], dtype=params.dtype, device=params.device) if ctx.needs_input_grad[1] else None
-        dx1 = (torch.empty(M, ctx.desc[1], dtype=params.dtype, device=params.device)
+        dparams = (torch.empty_like if ctx.whole else torch.zeros_like)(params) if ctx.needs_input_grad[0] else None
+        dx0 = torch.empty(M, desc.in0, dtype=params.dtype, device=params.device) if ctx.needs_input_grad[1] else None
+        dx1 = (torch.empty(M, desc.in1, dtype=params.dtype, device=params.device)
                if (x1c is not None and ctx.needs_input_grad[2]) else None)
         dyc = dy.contiguous().to(params.dtype)
         api.check(L.crl_mlp_backward(byref(desc), params.data_ptr(), x0c.data_ptr(),
@@ -82,7 +107,8 @@ class InfoNCELoss(torch.autograd.Function):
     """Critic loss (energy + InfoNCE + logsumexp penalty); returns (total, parts[4]).
 
     parts = {total, InfoNCE-fwd, InfoNCE-bwd, penalty} (not differentiable).
-    The backward takes the incoming gradient of ``total`` as a host scalar.
+    The backward reads the incoming gradient of ``total`` on the device: it does not
+    wait for the stream.
     path "fused": float32 representations on the BF16 fused kernels (B a
     multiple of 8, repr 64 / 128 / 192 / 256; the L1 energy runs on FP32 SIMT
     tiles, the others on the tensor cores).
@@ -92,34 +118,42 @@ class InfoNCELoss(torch.autograd.Function):
     def forward(ctx, phi, psi, energy, loss, sym_reduction, penalty_axis, temperature, beta, path):
         L = api.lib()
         dtype = _dtype_code(phi, "bf16" if path == "fused" else None)
-        desc = api.CrlLossDesc(api.ENERGY[energy], api.LOSS[loss], api.SYM[sym_reduction],
-                               api.PENALTY[penalty_axis], temperature, beta, dtype, api.PATH[path])
         B, R = phi.shape
-        nbytes = c_size_t()
-        api.check(L.crl_infonce_workspace_bytes(byref(desc), B, R, byref(nbytes)))
-        ws = torch.empty(nbytes.value, dtype=torch.uint8, device=phi.device)
+        desc, nbytes = _loss_plan(energy, loss, sym_reduction, penalty_axis, temperature, beta, dtype, path, B, R)
+        # one allocation: the kernels' workspace, then the row and the column logsumexps
+        at_r = -(-nbytes // 256) * 256
+        at_c = at_r + -(-B * phi.element_size() // 256) * 256
+        ws = torch.empty(2 * at_c - at_r, dtype=torch.uint8, device=phi.device)
+        base = ws.data_ptr()
         phi_c, psi_c = phi.detach().contiguous(), psi.detach().contiguous()
         parts = torch.empty(4, dtype=phi.dtype, device=phi.device)
-        r = torch.empty(B, dtype=phi.dtype, device=phi.device)
-        c = torch.empty(B, dtype=phi.dtype, device=phi.device)
-        api.check(L.crl_infonce_forward(byref(desc), phi_c.data_ptr(), psi_c.data_ptr(), B, R, parts.data_ptr(),
-                                        r.data_ptr(), c.data_ptr(), ws.data_ptr(), nbytes.value, api.stream_handle()))
+        total = torch.empty((), dtype=phi.dtype, device=phi.device)
+        api.check(L.crl_infonce_forward_total(byref(desc), phi_c.data_ptr(), psi_c.data_ptr(), B, R, parts.data_ptr(),
+                                              total.data_ptr(), base + at_r, base + at_c, base, nbytes,
+                                              api.stream_handle()))
         ctx.desc = desc
-        ctx.ws_bytes = nbytes.value
-        ctx.save_for_backward(phi_c, psi_c, r, c, ws)
+        ctx.layout = nbytes, at_r, at_c
+        ctx.save_for_backward(phi_c, psi_c, ws)
         ctx.mark_non_differentiable(parts)
-        return parts[0].clone(), parts
+        ctx.set_materialize_grads(False)
+        return total, parts
 
     @staticmethod
     def backward(ctx, dtotal, _dparts):
         L = api.lib()
-        phi, psi, r, c, ws = ctx.saved_tensors
+        phi, psi, ws = ctx.saved_tensors
+        nbytes, at_r, at_c = ctx.layout
+        base = ws.data_ptr()
         B, R = phi.shape
+        stream = torch.cuda.current_stream()
+        # the kernels read the multiplier after this returns, on a stream that need not be the one it was allocated on
+        dtotal = torch.zeros_like(phi[0, 0]) if dtotal is None else dtotal.to(phi.dtype)
+        dtotal.record_stream(stream)
         dphi = torch.empty_like(phi)
         dpsi = torch.empty_like(psi)
-        api.check(L.crl_infonce_backward(byref(ctx.desc), phi.data_ptr(), psi.data_ptr(), B, R, r.data_ptr(),
-                                         c.data_ptr(), float(dtotal.item()), dphi.data_ptr(), dpsi.data_ptr(),
-                                         ws.data_ptr(), ctx.ws_bytes, api.stream_handle()))
+        api.check(L.crl_infonce_backward_device_scale(byref(ctx.desc), phi.data_ptr(), psi.data_ptr(), B, R,
+                                                      base + at_r, base + at_c, dtotal.data_ptr(), dphi.data_ptr(),
+                                                      dpsi.data_ptr(), base, nbytes, api.stream_handle(stream)))
         return dphi, dpsi, None, None, None, None, None, None, None
 
 
