@@ -93,6 +93,7 @@ struct LayerOffsets {
   int64_t W, b, g, beta;            // g/beta = -1 without LayerNorm
   int in, out;
 };
+constexpr double kLnEps = 1e-6;   // LayerNorm, FP32 / FP64 paths
 // Layout of the flat parameter array; returns the element count (64-element aligned tensors).
 int64_t mlp_layout(const MlpShape& s, LayerOffsets* lay /* layers + 1 entries */);
 size_t mlp_saved_bytes(const MlpShape& s, int M, size_t elem);

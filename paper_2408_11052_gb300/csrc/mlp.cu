@@ -18,7 +18,6 @@
 
 namespace crl {
 
-constexpr double kLnEps = 1e-6;
 
 int64_t mlp_layout(const MlpShape& s, LayerOffsets* lay) {
   int64_t off = 0;

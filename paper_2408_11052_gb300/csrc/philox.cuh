@@ -74,4 +74,19 @@ __device__ T philox_normal(unsigned long long step, int b, unsigned long long wo
   }
 }
 
+// Both elements 2 p and 2 p + 1 of the same draw (float): one block and one
+// Box-Muller for the two.
+__device__ __forceinline__ float2 philox_normal_pair(unsigned long long step, int b, unsigned long long word, int p,
+                                                     unsigned long long seed, unsigned long long agent) {
+  constexpr double kTwoPi = 6.28318530717958647693;
+  const Philox4 r = philox4x64_10(step, (unsigned long long)b, word, (unsigned long long)(p / 2), seed, agent);
+  const bool hi = p % 2 != 0;
+  const double u1 = u64_to_unit_open(hi ? r.w[2] : r.w[0]);
+  const double u2 = u64_to_unit_open(hi ? r.w[3] : r.w[1]);
+  const float rad = sqrtf(-2.0f * logf((float)u1));
+  float s, c;
+  sincosf((float)(kTwoPi * u2), &s, &c);
+  return make_float2(rad * c, rad * s);
+}
+
 }  // namespace crl
