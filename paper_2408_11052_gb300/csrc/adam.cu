@@ -15,10 +15,20 @@ namespace crl {
 namespace {
 
 template <typename T>
-__global__ void __launch_bounds__(256) adam_kernel(T* __restrict__ p, const T* __restrict__ g, T* __restrict__ m,
-                                                  T* __restrict__ v, long long n, const int* __restrict__ t_dev,
-                                                  int t_host, float lr, float b1, float b2, float eps) {
+struct AdamPair {
+  AdamArrays<T> a[2];
+};
+// blockIdx.y: the network.
+template <typename T>
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamPair<T> pair,
+                                                  const int* __restrict__ t_dev, int t_host, float lr, float b1,
+                                                  float b2, float eps) {
   pdl_enter();
+  T* __restrict__ p = pair.a[blockIdx.y].p;
+  const T* __restrict__ g = pair.a[blockIdx.y].g;
+  T* __restrict__ m = pair.a[blockIdx.y].m;
+  T* __restrict__ v = pair.a[blockIdx.y].v;
+  const long long n = pair.a[blockIdx.y].n;
   // Bias corrections in double (1 - b^t loses most of its digits in float for
   // small t), computed once per block.
   // b^t by repeated squaring (at most 31 double products; pow() took several us of
@@ -50,17 +60,27 @@ __global__ void __launch_bounds__(256) adam_kernel(T* __restrict__ p, const T* _
 }  // namespace
 
 template <typename T>
-void adam_update(T* p, const T* g, T* m, T* v, int64_t n, const int* t_dev, int t_host, float lr, float b1, float b2,
+void adam_update(const AdamArrays<T>* a, int count, const int* t_dev, int t_host, float lr, float b1, float b2,
                  float eps, cudaStream_t st) {
-  if (n <= 0) return;
-  const int blocks = (int)std::min<int64_t>(ceil_div(n, 256), 152 * 8);
-  TraceLaunch tr(CRL_TRACE_ADAM, st, 7.0 * sizeof(T) * n);  // read p, g, m, v; write p, m, v
-  launch_k(adam_kernel<T>, dim3(blocks), dim3(256), 0, st, p, g, m, v, n, t_dev, t_host, lr, b1, b2, eps);
+  AdamPair<T> pair;
+  int64_t longest = 0, total = 0;
+  int live = 0;
+  for (int i = 0; i < count; ++i) {
+    if (a[i].n <= 0) continue;
+    pair.a[live++] = a[i];
+    longest = std::max(longest, a[i].n);
+    total += a[i].n;
+  }
+  if (live == 0) return;
+  if (live == 1) pair.a[1] = pair.a[0];
+  const int blocks = (int)std::min<int64_t>(ceil_div(longest, 256), 152 * 8 / live);
+  TraceLaunch tr(CRL_TRACE_ADAM, st, 7.0 * sizeof(T) * total);  // read p, g, m, v; write p, m, v
+  launch_k(adam_kernel<T>, dim3(blocks, live), dim3(256), 0, st, pair, t_dev, t_host, lr, b1, b2, eps);
 }
 
-template void adam_update<float>(float*, const float*, float*, float*, int64_t, const int*, int, float, float, float,
-                                 float, cudaStream_t);
-template void adam_update<double>(double*, const double*, double*, double*, int64_t, const int*, int, float, float,
-                                  float, float, cudaStream_t);
+template void adam_update<float>(const AdamArrays<float>*, int, const int*, int, float, float, float, float,
+                                 cudaStream_t);
+template void adam_update<double>(const AdamArrays<double>*, int, const int*, int, float, float, float, float,
+                                  cudaStream_t);
 
 }  // namespace crl

@@ -178,24 +178,30 @@ void critic_impl(crl_ctx* c, const float* s, const float* a, const float* g, int
   T* rl = static_cast<T*>(c->row_lse);
   T* cl = static_cast<T*>(c->col_lse);
   T* loss = static_cast<T*>(c->loss);
-  mlp_forward<T, float>(c->shapes[CRL_NET_PHI], pphi, s, a, B, phi, c->saved[CRL_NET_PHI], st);
-  mlp_forward<T, float>(c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, psi, c->saved[CRL_NET_PSI], st);
+  const MlpForward<T, float> fwd[2] = {
+      {&c->shapes[CRL_NET_PHI], pphi, s, a, B, phi, c->saved[CRL_NET_PHI]},
+      {&c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, psi, c->saved[CRL_NET_PSI]}};
+  mlp_forward<T, float>(fwd, 2, st);
   const LossSpec ls = loss_spec(cf);
   infonce_forward<T>(ls, phi, psi, B, cf.repr, loss, nullptr, rl, cl, c->ws, cf.path, &c->ctr->status,
                      apply ? &c->ctr->t_critic : nullptr, st);
   logit_stats_launch(c, phi, psi, B, sizeof(T) == 8, st);
   infonce_backward<T>(ls, phi, psi, B, cf.repr, rl, cl, 1.0, nullptr, dphi, dpsi, c->ws, cf.path, st);
-  mlp_backward<T, float>(c->shapes[CRL_NET_PHI], pphi, s, a, B, c->saved[CRL_NET_PHI], dphi,
-                         static_cast<T*>(c->nets[CRL_NET_PHI].grads), nullptr, nullptr, st);
-  mlp_backward<T, float>(c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, c->saved[CRL_NET_PSI], dpsi,
-                         static_cast<T*>(c->nets[CRL_NET_PSI].grads), nullptr, nullptr, st);
+  const MlpBackward<T, float> bwd[2] = {
+      {&c->shapes[CRL_NET_PHI], pphi, s, a, B, c->saved[CRL_NET_PHI], dphi,
+       static_cast<T*>(c->nets[CRL_NET_PHI].grads), nullptr, nullptr},
+      {&c->shapes[CRL_NET_PSI], ppsi, g, nullptr, B, c->saved[CRL_NET_PSI], dpsi,
+       static_cast<T*>(c->nets[CRL_NET_PSI].grads), nullptr, nullptr}};
+  mlp_backward<T, float>(bwd, 2, st);
   if (apply) {
-    for (int net : {CRL_NET_PHI, CRL_NET_PSI}) {
+    AdamArrays<T> arr[2];
+    for (int i = 0; i < 2; ++i) {
+      const int net = i == 0 ? CRL_NET_PHI : CRL_NET_PSI;
       const crl_net_ptrs& np = c->nets[net];
-      adam_update<T>(static_cast<T*>(np.params), static_cast<const T*>(np.grads), static_cast<T*>(np.adam_m),
-                     static_cast<T*>(np.adam_v), c->counts[net], &c->ctr->t_critic, 0, cf.lr_critic, cf.adam_beta1,
-                     cf.adam_beta2, cf.adam_eps, st);
+      arr[i] = {static_cast<T*>(np.params), static_cast<const T*>(np.grads), static_cast<T*>(np.adam_m),
+                static_cast<T*>(np.adam_v), c->counts[net]};
     }
+    adam_update<T>(arr, 2, &c->ctr->t_critic, 0, cf.lr_critic, cf.adam_beta1, cf.adam_beta2, cf.adam_eps, st);
   }
   if constexpr (sizeof(T) != sizeof(float)) {
     TraceLaunch tr(CRL_TRACE_AUX, st, 4.0 * (sizeof(T) + 4));

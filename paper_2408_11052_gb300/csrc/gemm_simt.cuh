@@ -196,9 +196,25 @@ struct F32Ring {
   }
 };
 
+// One product; a launch takes one or two that do not depend on each other (the two
+// networks of the critic: blockIdx.z).  At its sizes a product is a few tiles per SM
+// at most, and half the launches halve the time.
+template <class LA, class LB, class EP>
+struct GemmSet {
+  int M, N, K;
+  LA la;
+  LB lb;
+  EP ep;
+  int vec_a = 0, vec_b = 0;   // 16-byte copies (set by the launch)
+};
+template <class LA, class LB, class EP>
+struct GemmSets {
+  GemmSet<LA, LB, EP> s[2];
+};
+
 template <InnerOp OP, int BM, int BN, int TM, int TN, class LA, class LB, class EP>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    gemm_f32_kernel(int M, int N, int K, LA la, LB lb, EP ep, int vec_a, int vec_b) {
+    gemm_f32_kernel(const __grid_constant__ GemmSets<LA, LB, EP> sets) {
   constexpr int kThreads = (BM / TM) * (BN / TN);
   static_assert(BM * kF32K % kThreads == 0 && BN * kF32K % kThreads == 0, "copies per thread");
   using RA = F32Ring<LA::kContigK, BM, TM>;
@@ -206,9 +222,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
   __shared__ __align__(16) RA As;
   __shared__ __align__(16) RB Bs;
   pdl_enter();
+  const GemmSet<LA, LB, EP>& set = sets.s[blockIdx.z];
+  const int M = set.M, N = set.N, K = set.K, vec_a = set.vec_a, vec_b = set.vec_b;
+  const LA la = set.la;
+  const LB lb = set.lb;
+  const EP ep = set.ep;
   const int tid = threadIdx.x;
   const int tx = tid % (BN / TN), ty = tid / (BN / TN);
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  if (m0 >= M || n0 >= N) return;   // (the grid covers the larger product)
   auto load = [&](int buf, int k0) {
     As.template load<kThreads>(buf, k0, m0, M, K, vec_a != 0, [&](int m, int k) { return la.addr(m, k); });
     Bs.template load<kThreads>(buf, k0, n0, N, K, vec_b != 0, [&](int n, int k) { return lb.addr(k, n); });
@@ -271,36 +293,61 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 }
 
 template <InnerOp OP, int BM, int BN, int TM, int TN, class LA, class LB, class EP>
-void launch_gemm_f32(int M, int N, int K, const LA& la, const LB& lb, const EP& ep, cudaStream_t st) {
-  launch_k(gemm_f32_kernel<OP, BM, BN, TM, TN, LA, LB, EP>, dim3(ceil_div(N, BN), ceil_div(M, BM)),
-           dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, la, lb, ep, la.vec4(M, K) ? 1 : 0, lb.vec4(N, K) ? 1 : 0);
+void launch_gemm_f32(const GemmSets<LA, LB, EP>& g, int n, int M, int N, cudaStream_t st) {
+  launch_k(gemm_f32_kernel<OP, BM, BN, TM, TN, LA, LB, EP>, dim3(ceil_div(N, BN), ceil_div(M, BM), n),
+           dim3((BM / TM) * (BN / TN)), 0, st, g);
 }
 
-// Launch; traced as class `cls` (CRL_TRACE_*) with 2 M N K flops of work.  FP32
-// takes the tile whose waves over the 152 SMs cost least: outputs per SM, weighted
-// by the shared reads per FMA of its thread tile (a 2 x 2 tile reads twice what a
-// 4 x 4 tile does).  FP64 keeps the 32 x 32 tile of the kernel above.
+// Launch of n products (one or two); traced as class `cls` (CRL_TRACE_*) with
+// 2 M N K flops of work each.  FP32 takes the tile whose waves over the 152 SMs cost
+// least: outputs per SM, weighted by the shared reads per FMA of its thread tile (a
+// 2 x 2 tile reads twice what a 4 x 4 tile does).  FP64 keeps the 32 x 32 tile of the
+// kernel above, a launch per product.
 template <typename T, InnerOp OP = InnerOp::kMul, class LA, class LB, class EP>
-void gemm(int M, int N, int K, const LA& la, const LB& lb, const EP& ep, cudaStream_t st, int cls = CRL_TRACE_GEMM) {
-  if (M <= 0 || N <= 0) return;
-  TraceLaunch tr(cls, st, 2.0 * M * N * K);
+void gemm_sets(const GemmSet<LA, LB, EP>* set, int n, cudaStream_t st, int cls = CRL_TRACE_GEMM) {
   if constexpr (sizeof(T) == 8) {
-    // (its 64 x 64 double buffers would exceed 48 KiB of static shared memory)
-    dim3 grid(ceil_div(N, 32), ceil_div(M, 32));
-    launch_k(gemm_tile_kernel<T, OP, 32, 32, LA, LB, EP>, dim3(grid), dim3(256), 0, st, M, N, K, la, lb, ep);
+    for (int i = 0; i < n; ++i) {
+      const GemmSet<LA, LB, EP>& p = set[i];
+      if (p.M <= 0 || p.N <= 0) continue;
+      TraceLaunch tr(cls, st, 2.0 * p.M * p.N * p.K);
+      // (its 64 x 64 double buffers would exceed 48 KiB of static shared memory)
+      dim3 grid(ceil_div(p.N, 32), ceil_div(p.M, 32));
+      launch_k(gemm_tile_kernel<T, OP, 32, 32, LA, LB, EP>, dim3(grid), dim3(256), 0, st, p.M, p.N, p.K, p.la, p.lb, p.ep);
+    }
   } else {
+    GemmSets<LA, LB, EP> g;
+    int live = 0, M = 0, N = 0;
+    double flops = 0;
+    for (int i = 0; i < n; ++i) {
+      if (set[i].M <= 0 || set[i].N <= 0) continue;
+      GemmSet<LA, LB, EP>& p = g.s[live++];
+      p = set[i];
+      p.vec_a = p.la.vec4(p.M, p.K) ? 1 : 0;
+      p.vec_b = p.lb.vec4(p.N, p.K) ? 1 : 0;
+      M = std::max(M, p.M), N = std::max(N, p.N);
+      flops += 2.0 * p.M * p.N * p.K;
+    }
+    if (live == 0) return;
+    if (live == 1) g.s[1] = g.s[0];
+    TraceLaunch tr(cls, st, flops);
     auto cost = [&](int bm, int bn, double w) {
       if (bm < 64 && ceil_div(M, bm) > 65535) return 1e300;   // grid.y
-      const long long ctas = (long long)ceil_div(M, bm) * ceil_div(N, bn);
+      long long ctas = 0;
+      for (int i = 0; i < live; ++i) ctas += (long long)ceil_div(g.s[i].M, bm) * ceil_div(g.s[i].N, bn);
       return (double)((ctas + 151) / 152) * bm * bn * w;
     };
     const double c64 = cost(64, 64, 1.0), c32w = cost(32, 64, 1.05), c32 = cost(32, 32, 1.2), c16 = cost(16, 32, 1.5);
     const double best = std::min(std::min(c64, c32w), std::min(c32, c16));
-    if (best == c64) launch_gemm_f32<OP, 64, 64, 4, 4>(M, N, K, la, lb, ep, st);
-    else if (best == c32w) launch_gemm_f32<OP, 32, 64, 4, 4>(M, N, K, la, lb, ep, st);
-    else if (best == c32) launch_gemm_f32<OP, 32, 32, 2, 4>(M, N, K, la, lb, ep, st);
-    else launch_gemm_f32<OP, 16, 32, 2, 2>(M, N, K, la, lb, ep, st);
+    if (best == c64) launch_gemm_f32<OP, 64, 64, 4, 4>(g, live, M, N, st);
+    else if (best == c32w) launch_gemm_f32<OP, 32, 64, 4, 4>(g, live, M, N, st);
+    else if (best == c32) launch_gemm_f32<OP, 32, 32, 2, 4>(g, live, M, N, st);
+    else launch_gemm_f32<OP, 16, 32, 2, 2>(g, live, M, N, st);
   }
+}
+template <typename T, InnerOp OP = InnerOp::kMul, class LA, class LB, class EP>
+void gemm(int M, int N, int K, const LA& la, const LB& lb, const EP& ep, cudaStream_t st, int cls = CRL_TRACE_GEMM) {
+  const GemmSet<LA, LB, EP> one{M, N, K, la, lb, ep};
+  gemm_sets<T, OP>(&one, 1, st, cls);
 }
 
 // ---- loaders ---------------------------------------------------------------

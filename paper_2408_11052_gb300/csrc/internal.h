@@ -98,13 +98,45 @@ constexpr double kLnEps = 1e-6;   // LayerNorm, FP32 / FP64 paths
 int64_t mlp_layout(const MlpShape& s, LayerOffsets* lay /* layers + 1 entries */);
 size_t mlp_saved_bytes(const MlpShape& s, int M, size_t elem);
 
+// One network's forward / backward; dparams / dx0 / dx1 may be null.
+template <typename T, typename TX1>
+struct MlpForward {
+  const MlpShape* s;
+  const T* params;
+  const float* x0;
+  const TX1* x1;
+  int M;
+  T* y;
+  void* saved;
+};
+template <typename T, typename TX1>
+struct MlpBackward {
+  const MlpShape* s;
+  const T* params;
+  const float* x0;
+  const TX1* x1;
+  int M;
+  const void* saved;
+  const T* dy;
+  T *dparams, *dx0, *dx1;
+};
+// n networks that do not depend on each other (one or two), a launch for each layer of all.
+template <typename T, typename TX1>
+void mlp_forward(const MlpForward<T, TX1>* net, int n, cudaStream_t st);
+template <typename T, typename TX1>
+void mlp_backward(const MlpBackward<T, TX1>* net, int n, cudaStream_t st);
 template <typename T, typename TX1>
 void mlp_forward(const MlpShape& s, const T* params, const float* x0, const TX1* x1, int M, T* y,
-                 void* saved, cudaStream_t st);
-// dparams / dx0 / dx1 may be null.
+                 void* saved, cudaStream_t st) {
+  const MlpForward<T, TX1> one{&s, params, x0, x1, M, y, saved};
+  mlp_forward<T, TX1>(&one, 1, st);
+}
 template <typename T, typename TX1>
 void mlp_backward(const MlpShape& s, const T* params, const float* x0, const TX1* x1, int M,
-                  const void* saved, const T* dy, T* dparams, T* dx0, T* dx1, cudaStream_t st);
+                  const void* saved, const T* dy, T* dparams, T* dx0, T* dx1, cudaStream_t st) {
+  const MlpBackward<T, TX1> one{&s, params, x0, x1, M, saved, dy, dparams, dx0, dx1};
+  mlp_backward<T, TX1>(&one, 1, st);
+}
 
 // ---------------------------------------------------------------- energy + InfoNCE
 struct LossSpec {
@@ -229,9 +261,24 @@ const char* actor_head_backward_multi(BlobCache& cache, const std::vector<HeadBw
                                       cudaStream_t st);
 
 // ---------------------------------------------------------------- Adam
+// One network's arrays of n elements.
 template <typename T>
-void adam_update(T* p, const T* g, T* m, T* v, int64_t n, const int* t_dev, int t_host, float lr,
-                 float b1, float b2, float eps, cudaStream_t st);
+struct AdamArrays {
+  T* p;
+  const T* g;
+  T *m, *v;
+  int64_t n;
+};
+// `count` networks (one or two) in one launch.
+template <typename T>
+void adam_update(const AdamArrays<T>* a, int count, const int* t_dev, int t_host, float lr, float b1, float b2,
+                 float eps, cudaStream_t st);
+template <typename T>
+void adam_update(T* p, const T* g, T* m, T* v, int64_t n, const int* t_dev, int t_host, float lr, float b1, float b2,
+                 float eps, cudaStream_t st) {
+  const AdamArrays<T> one{p, g, m, v, n};
+  adam_update<T>(&one, 1, t_dev, t_host, lr, b1, b2, eps, st);
+}
 
 // Small device utilities.
 void launch_bump_u64(unsigned long long* ctr, cudaStream_t st);

@@ -88,11 +88,25 @@ Saved<T> carve(const MlpShape& s, int M, void* base) {
 // Row-wise LayerNorm + ReLU: z (in zhat, overwritten by zhat), rstd, h = ReLU(zhat*g + beta).
 // One warp per row.
 template <typename T>
-__global__ void __launch_bounds__(256) layernorm_relu_kernel(int M, int N, T* __restrict__ zhat,
-                                                            T* __restrict__ rstd, T* __restrict__ h,
-                                                            const T* __restrict__ gain,
-                                                            const T* __restrict__ bias) {
+struct LnFwd {   // one network's; blockIdx.y picks the network
+  int M, N;
+  T *zhat, *rstd, *h;
+  const T *gain, *bias;
+};
+template <typename T>
+struct LnFwds {
+  LnFwd<T> a[2];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) layernorm_relu_kernel(const __grid_constant__ LnFwds<T> args) {
   pdl_enter();
+  const LnFwd<T>& p = args.a[blockIdx.y];
+  const int M = p.M, N = p.N;
+  T* __restrict__ zhat = p.zhat;
+  T* __restrict__ rstd = p.rstd;
+  T* __restrict__ h = p.h;
+  const T* __restrict__ gain = p.gain;
+  const T* __restrict__ bias = p.bias;
   const int lane = threadIdx.x % kWarp;
   const int row = blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp;
   if (row >= M) return;
@@ -118,11 +132,25 @@ __global__ void __launch_bounds__(256) layernorm_relu_kernel(int M, int N, T* __
 
 // Row-wise LayerNorm backward: du (already masked by ReLU) -> dz.
 template <typename T>
-__global__ void __launch_bounds__(256) layernorm_bwd_kernel(int M, int N, const T* __restrict__ du,
-                                                           const T* __restrict__ zhat,
-                                                           const T* __restrict__ rstd,
-                                                           const T* __restrict__ gain, T* __restrict__ dz) {
+struct LnBwd {
+  int M, N;
+  const T *du, *zhat, *rstd, *gain;
+  T* dz;
+};
+template <typename T>
+struct LnBwds {
+  LnBwd<T> a[2];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) layernorm_bwd_kernel(const __grid_constant__ LnBwds<T> args) {
   pdl_enter();
+  const LnBwd<T>& p = args.a[blockIdx.y];
+  const int M = p.M, N = p.N;
+  const T* __restrict__ du = p.du;
+  const T* __restrict__ zhat = p.zhat;
+  const T* __restrict__ rstd = p.rstd;
+  const T* __restrict__ gain = p.gain;
+  T* __restrict__ dz = p.dz;
   const int lane = threadIdx.x % kWarp;
   const int row = blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp;
   if (row >= M) return;
@@ -143,20 +171,32 @@ __global__ void __launch_bounds__(256) layernorm_bwd_kernel(int M, int N, const 
   }
 }
 
-// Column sums over M rows: out1[n] = sum X, out2[n] = sum X*Y (Y optional),
-// out3[n] = sum Z (Z optional).  Block = 32 columns x 32 row groups (eight groups
+// Column sums over M rows: out1[n] = sum X, out2[n] = sum X*Y (Y optional).  Block = 32 columns x 32 row groups (eight groups
 // left M / 8 dependent loads per thread: 9 us at M = 256 against 4 now).
 constexpr int kSumRows = 32;
 template <typename T>
-__global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(int M, int N, const T* __restrict__ X,
-                                                    const T* __restrict__ Y, const T* __restrict__ Z,
-                                                    T* __restrict__ out1, T* __restrict__ out2,
-                                                    T* __restrict__ out3) {
+struct ColSum {
+  int M, N;
+  const T *X, *Y;
+  T *out1, *out2;
+};
+template <typename T>
+struct ColSums {
+  ColSum<T> a[2];
+};
+template <typename T>
+__global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(const __grid_constant__ ColSums<T> args) {
   pdl_enter();
-  __shared__ T sm[3][kSumRows][33];
+  const ColSum<T>& p = args.a[blockIdx.y];
+  const int M = p.M, N = p.N;
+  const T* __restrict__ X = p.X;
+  const T* __restrict__ Y = p.Y;
+  T* __restrict__ out1 = p.out1;
+  T* __restrict__ out2 = p.out2;
+  __shared__ T sm[2][kSumRows][33];
   const int cx = threadIdx.x % 32, ry = threadIdx.x / 32;
   const int n = blockIdx.x * 32 + cx;
-  T a1 = 0, a2 = 0, a3 = 0;
+  T a1 = 0, a2 = 0;
   if (n < N) {
 #pragma unroll 4
     for (int m = ry; m < M; m += kSumRows) {
@@ -164,134 +204,187 @@ __global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(int M, int N, con
       const T x = X[o];
       a1 += x;
       if (Y) a2 += x * Y[o];
-      if (Z) a3 += Z[o];
     }
   }
   sm[0][ry][cx] = a1;
   sm[1][ry][cx] = a2;
-  sm[2][ry][cx] = a3;
   __syncthreads();
   if (ry == 0 && n < N) {
-    T s1 = 0, s2 = 0, s3 = 0;
+    T s1 = 0, s2 = 0;
 #pragma unroll 8
     for (int r = 0; r < kSumRows; ++r) {
       s1 += sm[0][r][cx];
       s2 += sm[1][r][cx];
-      s3 += sm[2][r][cx];
     }
     if (out1) out1[n] = s1;
     if (out2) out2[n] = s2;
-    if (out3) out3[n] = s3;
   }
 }
 
 template <typename T>
-void colsum(int M, int N, const T* X, const T* Y, const T* Z, T* o1, T* o2, T* o3, cudaStream_t st) {
-  TraceLaunch tr(CRL_TRACE_AUX, st, (double)M * N * sizeof(T) * (1 + (Y != nullptr) + (Z != nullptr)));
-  launch_k(colsum_kernel<T>, dim3(ceil_div(N, 32)), dim3(32 * kSumRows), 0, st, M, N, X, Y, Z, o1, o2, o3);
+void colsum(const ColSum<T>* c, int n, cudaStream_t st) {
+  ColSums<T> a;
+  double bytes = 0;
+  int N = 0;
+  for (int i = 0; i < 2; ++i) {
+    a.a[i] = c[i < n ? i : 0];
+    if (i >= n) continue;
+    bytes += (double)c[i].M * c[i].N * sizeof(T) * (1 + (c[i].Y != nullptr));
+    N = std::max(N, c[i].N);
+  }
+  TraceLaunch tr(CRL_TRACE_AUX, st, bytes);
+  launch_k(colsum_kernel<T>, dim3(ceil_div(N, 32), n), dim3(32 * kSumRows), 0, st, a);
 }
 
 }  // namespace
 
+// Networks of one call share each launch (blockIdx.z of a product, blockIdx.y of the
+// others); they need the same number of layers and the same LayerNorm setting.
 template <typename T, typename TX1>
-void mlp_forward(const MlpShape& s, const T* params, const float* x0, const TX1* x1, int M, T* y, void* saved,
-                 cudaStream_t st) {
-  LayerOffsets lay[CRL_MAX_LAYERS + 1];
-  mlp_layout(s, lay);
-  Saved<T> sv = carve<T>(s, M, saved);
-  const int H = s.hidden;
-  for (int l = 0; l <= s.layers; ++l) {
-    const LayerOffsets& L = lay[l];
-    const bool last = (l == s.layers);
-    T* out = last ? y : (s.layernorm ? sv.zhat[l] : sv.h[l]);
-    const int ldo = last ? s.out : H;
-    EpiBias<T> ep{out, ldo, params + L.b, (!last && !s.layernorm) ? 1 : 0};
-    LoadNK<T> lb{params + L.W, L.in};
-    if (l == 0) {
-      LoadRowsSplit<T, float, TX1> la{x0, x1, s.in0, s.in1, s.in0};
-      gemm<T>(M, L.out, L.in, la, lb, ep, st);
-    } else {
-      LoadRowsSplit<T, T, T> la{sv.h[l - 1], nullptr, H, 0, H};
-      gemm<T>(M, L.out, L.in, la, lb, ep, st);
+void mlp_forward(const MlpForward<T, TX1>* net, int n, cudaStream_t st) {
+  const int layers = net[0].s->layers, layernorm = net[0].s->layernorm;
+  if (n == 2 && (net[1].s->layers != layers || net[1].s->layernorm != layernorm)) {
+    mlp_forward<T, TX1>(net, 1, st);
+    mlp_forward<T, TX1>(net + 1, 1, st);
+    return;
+  }
+  LayerOffsets lay[2][CRL_MAX_LAYERS + 1];
+  Saved<T> sv[2];
+  for (int i = 0; i < n; ++i) {
+    mlp_layout(*net[i].s, lay[i]);
+    sv[i] = carve<T>(*net[i].s, net[i].M, net[i].saved);
+  }
+  for (int l = 0; l <= layers; ++l) {
+    const bool last = (l == layers);
+    GemmSet<LoadRowsSplit<T, float, TX1>, LoadNK<T>, EpiBias<T>> first[2];
+    GemmSet<LoadRowsSplit<T, T, T>, LoadNK<T>, EpiBias<T>> later[2];
+    for (int i = 0; i < n; ++i) {
+      const MlpForward<T, TX1>& p = net[i];
+      const LayerOffsets& L = lay[i][l];
+      const int H = p.s->hidden;
+      T* out = last ? p.y : (layernorm ? sv[i].zhat[l] : sv[i].h[l]);
+      const int ldo = last ? p.s->out : H;
+      const EpiBias<T> ep{out, ldo, p.params + L.b, (!last && !layernorm) ? 1 : 0};
+      const LoadNK<T> lb{p.params + L.W, L.in};
+      if (l == 0)
+        first[i] = {p.M, L.out, L.in, LoadRowsSplit<T, float, TX1>{p.x0, p.x1, p.s->in0, p.s->in1, p.s->in0}, lb, ep};
+      else
+        later[i] = {p.M, L.out, L.in, LoadRowsSplit<T, T, T>{sv[i].h[l - 1], nullptr, H, 0, H}, lb, ep};
     }
-    if (!last && s.layernorm) {
-      TraceLaunch tr(CRL_TRACE_AUX, st, 4.0 * M * H * sizeof(T));
-      launch_k(layernorm_relu_kernel<T>, dim3(ceil_div(M, 8)), dim3(256), 0, st, M, H, sv.zhat[l], sv.rstd[l], sv.h[l],
-                                                               params + L.g, params + L.beta);
+    if (l == 0) gemm_sets<T>(first, n, st);
+    else gemm_sets<T>(later, n, st);
+    if (!last && layernorm) {
+      LnFwds<T> a;
+      double bytes = 0;
+      int M = 0;
+      for (int i = 0; i < 2; ++i) {
+        const int k = i < n ? i : 0;
+        const MlpForward<T, TX1>& p = net[k];
+        const LayerOffsets& L = lay[k][l];
+        a.a[i] = {p.M, p.s->hidden, sv[k].zhat[l], sv[k].rstd[l], sv[k].h[l], p.params + L.g, p.params + L.beta};
+        if (i < n) bytes += 4.0 * p.M * p.s->hidden * sizeof(T), M = std::max(M, p.M);
+      }
+      TraceLaunch tr(CRL_TRACE_AUX, st, bytes);
+      launch_k(layernorm_relu_kernel<T>, dim3(ceil_div(M, 8), n), dim3(256), 0, st, a);
     }
   }
 }
 
 template <typename T, typename TX1>
-void mlp_backward(const MlpShape& s, const T* params, const float* x0, const TX1* x1, int M, const void* saved,
-                  const T* dy, T* dparams, T* dx0, T* dx1, cudaStream_t st) {
-  LayerOffsets lay[CRL_MAX_LAYERS + 1];
-  mlp_layout(s, lay);
-  Saved<T> sv = carve<T>(s, M, const_cast<void*>(saved));
-  const int H = s.hidden;
-  // dcur holds dZ of the layer being processed ([M][out_l]).
-  const T* dcur = dy;
+void mlp_backward(const MlpBackward<T, TX1>* net, int n, cudaStream_t st) {
+  const int layers = net[0].s->layers, layernorm = net[0].s->layernorm;
+  const bool grads = net[0].dparams != nullptr;
+  const bool dx = net[0].dx0 || net[0].dx1;
+  if (n == 2 && (net[1].s->layers != layers || net[1].s->layernorm != layernorm ||
+                 (net[1].dparams != nullptr) != grads || (net[1].dx0 || net[1].dx1) != dx)) {
+    mlp_backward<T, TX1>(net, 1, st);
+    mlp_backward<T, TX1>(net + 1, 1, st);
+    return;
+  }
+  LayerOffsets lay[2][CRL_MAX_LAYERS + 1];
+  Saved<T> sv[2];
+  const T* dcur[2];   // dZ of the layer being processed ([M][out_l])
+  for (int i = 0; i < n; ++i) {
+    mlp_layout(*net[i].s, lay[i]);
+    sv[i] = carve<T>(*net[i].s, net[i].M, const_cast<void*>(net[i].saved));
+    dcur[i] = net[i].dy;
+  }
   int bufi = 0;
-  for (int l = s.layers; l >= 0; --l) {
-    const LayerOffsets& L = lay[l];
-    const int nout = L.out;
-    if (dparams) {
+  for (int l = layers; l >= 0; --l) {
+    if (grads) {
       // db_l = colsum(dZ_l);  dW_l[n][k] = sum_m dZ_l[m][n] * in_l[m][k]
-      colsum<T>(M, nout, dcur, nullptr, nullptr, dparams + L.b, nullptr, nullptr, st);
-      LoadTrans<T> la{dcur, nout};
-      EpiScale<T> ep{dparams + L.W, L.in, T(1)};
-      if (l == 0) {
-        LoadColsSplit<T, float, TX1> lb{x0, x1, s.in0, s.in1, s.in0};
-        gemm<T>(nout, L.in, M, la, lb, ep, st);
-      } else {
-        LoadColsSplit<T, T, T> lb{sv.h[l - 1], nullptr, H, 0, H};
-        gemm<T>(nout, L.in, M, la, lb, ep, st);
+      ColSum<T> db[2];
+      GemmSet<LoadTrans<T>, LoadColsSplit<T, float, TX1>, EpiScale<T>> first[2];
+      GemmSet<LoadTrans<T>, LoadColsSplit<T, T, T>, EpiScale<T>> later[2];
+      for (int i = 0; i < n; ++i) {
+        const MlpBackward<T, TX1>& p = net[i];
+        const LayerOffsets& L = lay[i][l];
+        const int H = p.s->hidden;
+        db[i] = {p.M, L.out, dcur[i], nullptr, p.dparams + L.b, nullptr};
+        const LoadTrans<T> la{dcur[i], L.out};
+        const EpiScale<T> ep{p.dparams + L.W, L.in, T(1)};
+        if (l == 0)
+          first[i] = {L.out, L.in, p.M, la, LoadColsSplit<T, float, TX1>{p.x0, p.x1, p.s->in0, p.s->in1, p.s->in0}, ep};
+        else
+          later[i] = {L.out, L.in, p.M, la, LoadColsSplit<T, T, T>{sv[i].h[l - 1], nullptr, H, 0, H}, ep};
       }
+      colsum<T>(db, n, st);
+      if (l == 0) gemm_sets<T>(first, n, st);
+      else gemm_sets<T>(later, n, st);
     }
-    LoadMK<T> la{dcur, nout};
-    LoadKN<T> lb{params + L.W, L.in};
-    if (l == 0) {
-      if (dx0 || dx1) {
-        EpiMaskSplit<T> ep{dx0, dx1, s.in0, s.in1, s.in0, nullptr, 0};
-        gemm<T>(M, L.in, nout, la, lb, ep, st);
+    if (l == 0 && !dx) break;
+    // dU_{l-1} = (dZ_l W_l) * [h_{l-1} > 0], or the input gradients
+    GemmSet<LoadMK<T>, LoadKN<T>, EpiMaskSplit<T>> prod[2];
+    for (int i = 0; i < n; ++i) {
+      const MlpBackward<T, TX1>& p = net[i];
+      const LayerOffsets& L = lay[i][l];
+      const int H = p.s->hidden;
+      const LoadMK<T> la{dcur[i], L.out};
+      const LoadKN<T> lb{p.params + L.W, L.in};
+      if (l == 0)
+        prod[i] = {p.M, L.in, L.out, la, lb, EpiMaskSplit<T>{p.dx0, p.dx1, p.s->in0, p.s->in1, p.s->in0, nullptr, 0}};
+      else
+        prod[i] = {p.M, H, L.out, la, lb,
+                   EpiMaskSplit<T>{sv[i].scratch[bufi], nullptr, H, 0, H, sv[i].h[l - 1], H}};
+    }
+    gemm_sets<T>(prod, n, st);
+    if (l == 0) break;
+    if (layernorm) {
+      LnBwds<T> a;
+      ColSum<T> dg[2];
+      double bytes = 0;
+      int M = 0;
+      for (int i = 0; i < 2; ++i) {
+        const int k = i < n ? i : 0;
+        const MlpBackward<T, TX1>& p = net[k];
+        const LayerOffsets& P = lay[k][l - 1];
+        T* du = sv[k].scratch[bufi];
+        a.a[i] = {p.M, p.s->hidden, du, sv[k].zhat[l - 1], sv[k].rstd[l - 1], p.params + P.g, sv[k].scratch[2]};
+        if (i >= n) continue;
+        dg[i] = {p.M, p.s->hidden, du, sv[i].zhat[l - 1], grads ? p.dparams + P.beta : nullptr,
+                 grads ? p.dparams + P.g : nullptr};
+        bytes += 3.0 * p.M * p.s->hidden * sizeof(T);
+        M = std::max(M, p.M);
+        // the next product reads dz (scratch[2]) and writes the other ping-pong buffer: no overlap
+        dcur[i] = sv[i].scratch[2];
       }
-      break;
-    }
-    // dU_{l-1} = (dZ_l W_l) * [h_{l-1} > 0]
-    T* du = sv.scratch[bufi];
-    bufi = (bufi + 1) % 2;
-    EpiMaskSplit<T> ep{du, nullptr, H, 0, H, sv.h[l - 1], H};
-    gemm<T>(M, H, nout, la, lb, ep, st);
-    if (s.layernorm) {
-      const LayerOffsets& P = lay[l - 1];
-      T* dz = sv.scratch[2];
       {
-        TraceLaunch tr(CRL_TRACE_AUX, st, 3.0 * M * H * sizeof(T));
-        launch_k(layernorm_bwd_kernel<T>, dim3(ceil_div(M, 8)), dim3(256), 0, st, M, H, du, sv.zhat[l - 1], sv.rstd[l - 1],
-                                                                params + P.g, dz);
+        TraceLaunch tr(CRL_TRACE_AUX, st, bytes);
+        launch_k(layernorm_bwd_kernel<T>, dim3(ceil_div(M, 8), n), dim3(256), 0, st, a);
       }
-      if (dparams)
-        colsum<T>(M, H, du, sv.zhat[l - 1], nullptr, dparams + P.beta, dparams + P.g, nullptr, st);
-      // move dz into the ping-pong buffer so scratch[2] is free for the next LayerNorm
-      dcur = dz;
-      // the next GEMM reads dz (scratch[2]) and writes scratch[bufi]: no overlap.
+      if (grads) colsum<T>(dg, n, st);
     } else {
-      dcur = du;
+      for (int i = 0; i < n; ++i) dcur[i] = sv[i].scratch[bufi];
     }
+    bufi = (bufi + 1) % 2;
   }
 }
 
-template void mlp_forward<float, float>(const MlpShape&, const float*, const float*, const float*, int, float*,
-                                        void*, cudaStream_t);
-template void mlp_forward<double, float>(const MlpShape&, const double*, const float*, const float*, int,
-                                         double*, void*, cudaStream_t);
-template void mlp_forward<double, double>(const MlpShape&, const double*, const float*, const double*, int,
-                                          double*, void*, cudaStream_t);
-template void mlp_backward<float, float>(const MlpShape&, const float*, const float*, const float*, int,
-                                         const void*, const float*, float*, float*, float*, cudaStream_t);
-template void mlp_backward<double, float>(const MlpShape&, const double*, const float*, const float*, int,
-                                          const void*, const double*, double*, double*, double*, cudaStream_t);
-template void mlp_backward<double, double>(const MlpShape&, const double*, const float*, const double*, int,
-                                           const void*, const double*, double*, double*, double*, cudaStream_t);
+template void mlp_forward<float, float>(const MlpForward<float, float>*, int, cudaStream_t);
+template void mlp_forward<double, float>(const MlpForward<double, float>*, int, cudaStream_t);
+template void mlp_forward<double, double>(const MlpForward<double, double>*, int, cudaStream_t);
+template void mlp_backward<float, float>(const MlpBackward<float, float>*, int, cudaStream_t);
+template void mlp_backward<double, float>(const MlpBackward<double, float>*, int, cudaStream_t);
+template void mlp_backward<double, double>(const MlpBackward<double, double>*, int, cudaStream_t);
 
 }  // namespace crl
