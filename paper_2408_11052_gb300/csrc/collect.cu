@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kUnrollThreads, 1) unroll_kernel(const __grid_
   for (int l = 0; l < p.layers; ++l) {
     const int K = l == 0 ? p.in : H, kb = (K + 15) / 16, nb = (nc + 7) / 8;
     const float* Wg = p.params + p.W[l];
-    const bool vec = (K & 3) == 0;   // tensors start on 256 bytes
+    const bool vec = (K & 3) == 0;   // tensors start 256 bytes apart in a 16-byte aligned array
     for (int b = wid; b < kb * nb; b += kUnrollThreads / kWarp) {
       const int n = 8 * (b % nb) + lane % 8, k = 16 * (b / nb) + 4 * (lane / 8);
       if (n >= nc || k >= K) continue;

@@ -33,6 +33,7 @@ def _mlp(desc, M, params, x0, x1, dy, fill):
 # tiles, odd row counts, one wide and one deep network, a batch that splits K
 @pytest.mark.parametrize("M,in0,in1,hidden,layers,out,layernorm", [
     (1, 3, 0, 8, 1, 8, 0),
+    (33, 5, 2, 40, 1, 19, 0),           # an output width off the 16-byte pitch
     (129, 29, 8, 72, 2, 64, 1),
     (257, 61, 3, 200, 3, 72, 1),
     (1000, 268, 17, 256, 4, 64, 0),
