@@ -307,70 +307,103 @@ __device__ __host__ __forceinline__ int pack_cols(int k, int D, int A, int G) {
   return k == 0 ? D + A : (k == 1 ? G : D + G);
 }
 
-// Relabel with the BF16 network-input packs (the update step): a block of 32
-// warps takes 32 consecutive samples, one per warp (lane 0 draws the indices,
-// the warp copies the row and writes its sample's split inputs row-major).
+// Relabel with the BF16 network-input packs (the update step): a block takes 16
+// consecutive samples.  Lanes of its first warp draw the indices side by side (a
+// draw is several hundred instructions: one lane per warp drawing its own sample
+// set the pace of large launches), then every warp copies two samples' rows, their
+// loads in flight together, and writes the split inputs row-major, a pair per store.
+constexpr int kPackSamples = 16, kPackThreads = 256;
+// lb: block index within this batch.
 __device__ __forceinline__ void relabel_pack_body(const BufferDev& bd, const RelabelArgs& ra, int lb) {
+  __shared__ long long s_row[2][kPackSamples];   // first floats of the (s, a) and the goal rows
   const int lane = threadIdx.x % kWarp, w = threadIdx.x / kWarp;
-  const int b0 = lb * kWarp;
-  const int b = b0 + w;
-  const unsigned long long step = (ra.step == CRL_STEP_AUTO) ? *ra.step_dev : ra.step;
-  if (lb == 0 && threadIdx.x == 0 && ra.last_step_dev != nullptr) *ra.last_step_dev = step;
+  const int b0 = lb * kPackSamples;
   const int size = bd.state[0];
-  const long long total = bd.state[1];
   if (size <= 0) {
     if (threadIdx.x == 0) atomicOr(ra.status, CRL_STATUS_BAD_INDEX);
     return;
   }
-  const int D = bd.D, DA = bd.D + bd.A;
-  if (b < ra.B) {
-    int e = 0, t = 0, k = 0;
-    if (lane == 0) {
+  const int D = bd.D, DA = bd.D + bd.A, G = ra.G;
+  if (w == 0) {
+    const unsigned long long step = (ra.step == CRL_STEP_AUTO) ? *ra.step_dev : ra.step;
+    if (lb == 0 && lane == 0 && ra.last_step_dev != nullptr) *ra.last_step_dev = step;
+    const long long total = bd.state[1];
+    const int b = b0 + lane;
+    if (lane < kPackSamples && b < ra.B) {
+      int e, t, k;
       sample_indices(bd, ra, step, b, size, total, e, t, k);
       if (ra.idx != nullptr) {
         ra.idx[3 * (size_t)b + 0] = e;
         ra.idx[3 * (size_t)b + 1] = t;
         ra.idx[3 * (size_t)b + 2] = k;
       }
+      const unsigned abs_t = (unsigned)(total - size + t), T = (unsigned)bd.T;   // (below 2^31)
+      s_row[0][lane] = ((long long)e * bd.T + abs_t % T) * bd.W;
+      s_row[1][lane] = ((long long)e * bd.T + (abs_t + (unsigned)k) % T) * bd.W;
     }
-    e = __shfl_sync(0xffffffffu, e, 0);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    k = __shfl_sync(0xffffffffu, k, 0);
-    const long long abs_t = total - size + t;
-    const float* row = bd.rows + ((size_t)e * bd.T + (size_t)(abs_t % bd.T)) * bd.W;
-    const float* grow = bd.rows + ((size_t)e * bd.T + (size_t)((abs_t + k) % bd.T)) * bd.W;
-    for (int c = lane; c < DA; c += kWarp) {
-      const float v = row[c];
-      if (c < D) ra.s[(size_t)b * D + c] = v;
-      else ra.a[(size_t)b * bd.A + (c - D)] = v;
-    }
-    if (lane < ra.G) ra.g[(size_t)b * ra.G + lane] = grow[ra.goal_idx[lane]];
-    for (int kk = 0; kk < 3; ++kk) {
-      const RelabelPack& pk = ra.pack[kk];
-      if (pk.x0 == nullptr) continue;
-      const int ncol = pack_cols(kk, D, bd.A, ra.G);
-      __nv_bfloat16* x0 = static_cast<__nv_bfloat16*>(pk.x0);
-      for (int c = lane; c < ncol; c += kWarp) {
-        float v;
-        if (kk == 0) v = row[c];
-        else if (kk == 1) v = grow[ra.goal_idx[c]];
-        else v = c < D ? row[c] : grow[ra.goal_idx[c - D]];
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-        x0[(size_t)b * pk.ld + 2 * c] = hi;
-        x0[(size_t)b * pk.ld + 2 * c + 1] = lo;
+  }
+  __syncthreads();
+  constexpr int kWarps = kPackThreads / kWarp, kPer = kPackSamples / kWarps;
+  const float *row[kPer], *grow[kPer];
+  bool live[kPer];
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int j = w + kWarps * i;
+    live[i] = b0 + j < ra.B;
+    row[i] = bd.rows + (live[i] ? s_row[0][j] : 0);
+    grow[i] = bd.rows + (live[i] ? s_row[1][j] : 0);
+  }
+  auto split = [](float v) {
+    __nv_bfloat162 p;
+    p.x = __float2bfloat16_rn(v);
+    p.y = __float2bfloat16_rn(v - __bfloat162float(p.x));
+    return p;
+  };
+  auto put = [&](int kk, int b, int c, __nv_bfloat162 p) {   // (rows and pairs are 4-byte aligned)
+    const RelabelPack& pk = ra.pack[kk];
+    if (pk.x0) *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(pk.x0) + (size_t)b * pk.ld + 2 * c) = p;
+  };
+  float gv[kPer];
+  const int gi = lane < G ? ra.goal_idx[lane] : 0;   // (G <= 16)
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) gv[i] = grow[i][gi];
+#pragma unroll 4
+  for (int c = lane; c < DA; c += kWarp) {
+    float v[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) v[i] = row[i][c];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      if (!live[i]) continue;
+      const int b = b0 + w + kWarps * i;
+      const __nv_bfloat162 p = split(v[i]);
+      put(0, b, c, p);
+      if (c < D) {
+        ra.s[(size_t)b * D + c] = v[i];
+        put(2, b, c, p);
+      } else {
+        ra.a[(size_t)b * bd.A + (c - D)] = v[i];
       }
     }
   }
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    if (!live[i] || lane >= G) continue;
+    const int b = b0 + w + kWarps * i;
+    const __nv_bfloat162 p = split(gv[i]);
+    ra.g[(size_t)b * G + lane] = gv[i];
+    put(1, b, lane, p);
+    put(2, b, D + lane, p);
+  }
 }
 
-__global__ void __launch_bounds__(1024) relabel_pack_kernel(const __grid_constant__ BufferDev bd,
+__global__ void __launch_bounds__(kPackThreads) relabel_pack_kernel(const __grid_constant__ BufferDev bd,
                                                            const __grid_constant__ RelabelArgs ra) {
   pdl_enter();
   relabel_pack_body(bd, ra, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(1024) relabel_pack_multi_kernel(const RelabelTask* __restrict__ tasks,
+__global__ void __launch_bounds__(kPackThreads) relabel_pack_multi_kernel(const RelabelTask* __restrict__ tasks,
                                                                  const int* __restrict__ begin, int n) {
   pdl_enter();
   int lb, nb;
@@ -396,7 +429,7 @@ __global__ void __launch_bounds__(256) relabel_multi_kernel(const RelabelTask* _
 int relabel_spw(int B) { return (int)std::min<long long>(32, std::max<long long>(1, (long long)B / (152 * 48))); }
 bool relabel_packs(const RelabelArgs& ra) { return ra.pack[0].x0 || ra.pack[1].x0 || ra.pack[2].x0; }
 int relabel_blocks(const RelabelArgs& ra) {
-  return relabel_packs(ra) ? ceil_div(ra.B, kWarp) : ceil_div(ra.B, 8 * ra.spw);
+  return relabel_packs(ra) ? ceil_div(ra.B, kPackSamples) : ceil_div(ra.B, 8 * ra.spw);
 }
 
 void launch_relabel_multi(const RelabelTask* tasks, const int* begin, int n, int blocks, double bytes, bool packs,
@@ -408,7 +441,7 @@ void launch_relabel_multi(const RelabelTask* tasks, const int* begin, int n, int
       cudaFuncSetAttribute(relabel_pack_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       attr = smem;
     }
-    launch_k(relabel_pack_multi_kernel, dim3(blocks), dim3(1024), smem, st, tasks, begin, n);
+    launch_k(relabel_pack_multi_kernel, dim3(blocks), dim3(kPackThreads), smem, st, tasks, begin, n);
   } else {
     launch_k(relabel_multi_kernel, dim3(blocks), dim3(256), 0, st, tasks, begin, n);
   }
@@ -422,7 +455,7 @@ void launch_relabel(const BufferDev& bd, const RelabelArgs& ra, cudaStream_t st)
   RelabelArgs r = ra;
   r.spw = relabel_spw(ra.B);
   if (relabel_packs(r)) {
-    launch_k(relabel_pack_kernel, dim3(relabel_blocks(r)), dim3(1024), 0, st, bd, r);
+    launch_k(relabel_pack_kernel, dim3(relabel_blocks(r)), dim3(kPackThreads), 0, st, bd, r);
   } else {
     launch_k(relabel_kernel, dim3(relabel_blocks(r)), dim3(256), 0, st, bd, r);
   }
