@@ -343,11 +343,17 @@ __global__ void __launch_bounds__(1024) loss_kernel(int B, const T* __restrict__
 // dg, kd: F_ii and k_i from objective_rows_kernel (objectives outside InfoNCE).
 // One block per row: the row's constants are read once, no index division, and the
 // row sums of H (rsum, may be null) cost no further pass over the matrix.
+// (scalars in T from the host: FP64 divisions and conversions per thread are slow)
+template <typename T>
+struct CoeffScalars {
+  T wf, wb, pr, pc, two_beta, tau, dtotal, scale;   // scale: dtotal / B
+  int obj;
+};
 template <typename T>
 __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ F, const T* __restrict__ r,
                                                         const T* __restrict__ c, const T* __restrict__ dg,
-                                                        const T* __restrict__ kd, DirWeights w, double beta,
-                                                        double dtotal, const T* __restrict__ dtotal_dev, int energy, double tau,
+                                                        const T* __restrict__ kd, const CoeffScalars<T> w,
+                                                        const T* __restrict__ dtotal_dev, int energy,
                                                         T* __restrict__ rsum) {
   pdl_enter();
   __shared__ T sm[32];
@@ -356,15 +362,15 @@ __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ 
   const T ri = r[i];
   T sum = 0;
   // (a quotient of two T values rounds the same through a double)
-  const T dt = dtotal_dev ? *dtotal_dev : T(dtotal);
-  const T scale = dtotal_dev ? dt / T(B) : T(dtotal / B);
+  const T dt = dtotal_dev ? *dtotal_dev : w.dtotal;
+  const T scale = dtotal_dev ? dt / T(B) : w.scale;
   const T bb = T(B) * T(B);
   for (int j = threadIdx.x; j < B; j += blockDim.x) {
     const T f = row[j];
     const T P = dev_exp(f - ri);
     const T Q = dev_exp(f - c[j]);
     const T dlt = (i == j) ? T(1) : T(0);
-    T g = T(w.wf) * (P - dlt) + T(w.wb) * (Q - dlt) + T(2.0 * beta) * (T(w.pr) * ri * P + T(w.pc) * c[j] * Q);
+    T g = w.wf * (P - dlt) + w.wb * (Q - dlt) + w.two_beta * (w.pr * ri * P + w.pc * c[j] * Q);
     g *= scale;
     if (w.obj >= CRL_LOSS_FB) {
       T o = 0;
@@ -380,12 +386,12 @@ __global__ void __launch_bounds__(256) grad_coeff_kernel(int B, T* __restrict__ 
     T h;
     switch (energy) {
       case CRL_ENERGY_L2: {
-        const T d = -f * T(tau);
-        h = (d >= T(1e-12)) ? g / (T(tau) * d) : T(0);
+        const T d = -f * w.tau;
+        h = (d >= T(1e-12)) ? g / (w.tau * d) : T(0);
         break;
       }
-      case CRL_ENERGY_L2SQ: h = T(2) * g / T(tau); break;
-      default: h = g / T(tau); break;  // dot, cos
+      case CRL_ENERGY_L2SQ: h = T(2) * g / w.tau; break;
+      default: h = g / w.tau; break;  // dot, cos
     }
     row[j] = h;
     sum += h;
@@ -537,8 +543,11 @@ void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int
   const bool diff = ls.energy == CRL_ENERGY_L2 || ls.energy == CRL_ENERGY_L2SQ;
   {
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0);
+    const DirWeights dw = weights(ls);
+    const CoeffScalars<T> cs{T(dw.wf),         T(dw.wb),  T(dw.pr),  T(dw.pc),
+                             T(2.0 * ls.beta), T(ls.tau), T(dtotal), T(dtotal / B), dw.obj};
     launch_k(grad_coeff_kernel<T>, dim3(B), dim3(256), 0, st, B, w.F, row_lse, col_lse, (const T*)w.dg,
-             (const T*)w.kd, weights(ls), ls.beta, dtotal, dtotal_dev, ls.energy, ls.tau, diff ? w.rsum : (T*)nullptr);
+             (const T*)w.kd, cs, dtotal_dev, ls.energy, diff ? w.rsum : (T*)nullptr);
   }
   const T* H = w.F;
   if (diff) {

@@ -196,7 +196,8 @@ void actor_head_forward(const ActorSpec& as, const T* pi_out, const float* eps,
 template <typename T>
 struct ActorLossArgs {
   int B, R, energy;
-  double tau, alpha;
+  T inv_tau, scale;           // 1 / tau and -1 / (B tau), from the host (actor_scalars)
+  double alpha;
   const T* phi;
   const T* psi;
   const T* logpi;
@@ -213,6 +214,12 @@ struct ActorLossArgs {
   const unsigned long long* last_step;
   AlphaTune tune;             // tune.state != null: alpha = exp(state[0]), updated at the end
 };
+// The scalars of ActorLossArgs, rounded as T(1.0 / tau) and T(-1.0 / B) * T(1.0 / tau).
+template <typename T>
+void actor_scalars(ActorLossArgs<T>& p, double tau) {
+  p.inv_tau = T(1.0 / tau);
+  p.scale = T(-1.0 / p.B) * p.inv_tau;
+}
 size_t actor_loss_ws_bytes(int B, size_t elem);
 template <typename T>
 struct HeadFwdArgs {
@@ -230,14 +237,14 @@ struct HeadFwdArgs {
 template <typename T>
 struct HeadBwdArgs {
   int B, A;
-  double alpha;
+  T alpha_over_b;                   // alpha / B, divided in double on the host
   const T* out;
   const T* eps_used;
   const T* da;
   T* dout;
   __nv_bfloat16* dz;                // optional BF16 output gradient (see actor_head_backward)
   int ldz;
-  const double* alpha_used;         // non-null: the alpha the actor loss used (overrides alpha)
+  const double* alpha_used;         // non-null: the alpha the actor loss used (overrides alpha_over_b)
 };
 // Diagonal energy, dphi (T, or BF16 into dz [B][ldz] when dz != null) and the
 // actor loss in one launch.  ws: actor_loss_ws_bytes(B, sizeof(T)); ticket: a

@@ -160,7 +160,9 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const __grid_constant
 // (it was a memset of the whole workspace and 2 + 2 (layers + 1) launches): the
 // weight shadows of every layer, the split input with its ones column, the ones
 // column and the K padding of every hidden activation, the status word and the
-// split-K tickets.  Blocks [0, wtiles): weight tiles; then 8 rows per block.
+// split-K tickets.  Blocks [0, wtiles): weight tiles; then 8 rows per block.  Memory
+// and latency bound: 8 us for 2 x 512 at 8192 rows (the memset alone took 18, the
+// packs 21), 14 us for 4 x 1024.
 struct NetPrep {
   ShadowTile L[CRL_MAX_LAYERS + 1];
   int tile_begin[CRL_MAX_LAYERS + 2];

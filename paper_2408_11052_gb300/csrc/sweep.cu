@@ -241,7 +241,7 @@ void body_grouped(crl_sweep* sw, cudaStream_t st) {
       t.B = cf.B;
       t.R = cf.repr;
       t.energy = cf.energy;
-      t.tau = (double)cf.temperature;
+      actor_scalars(t, (double)cf.temperature);
       t.alpha = (double)cf.alpha;
       t.phi = P.y;
       t.psi = Q.y;
@@ -272,7 +272,7 @@ void body_grouped(crl_sweep* sw, cudaStream_t st) {
       memset(&h, 0, sizeof(h));
       h.B = cf.B;
       h.A = cf.A;
-      h.alpha = (double)cf.alpha;
+      h.alpha_over_b = (float)((double)cf.alpha / cf.B);
       h.out = PI.y;
       h.eps_used = static_cast<const float*>(c->eps_used);
       h.da = static_cast<const float*>(c->da);
