@@ -590,12 +590,17 @@ __device__ __forceinline__ void epilogue_tile(const GemmProblem* P, const EpiDes
   const int row0 = m0 + 32 * eg;
   if (row0 >= M) return;
   const uint32_t lane_base = acc + ((uint32_t)(32 * eg) << 16);
+  const bool tma = NC == 64 && P->tma_out != 0;
+  // The staging block may still belong to the copies of the warp's last tile (in the
+  // kernels that walk a list: a policy's output that left as TMA stores, then an
+  // encoder's, or a policy's whose rows TMA does not take).  The steps that store
+  // through TMA wait for that before each write; nothing else does.
+  if (NC == 64 && !tma) stage_reclaim(lane);
   if (e.kind == kEpiFwdOutEnergy) {
     epilogue_energy(e, st, row0, lane, half, lane_base, N, M);
     return;
   }
   const int ncol = (N - n0 < BN) ? N - n0 : BN;
-  const bool tma = NC == 64 && P->tma_out != 0;
 #pragma unroll 1
   for (int c = NC * half; c < ncol; c += 2 * NC)
     epilogue_step<NC>(P, e, st, tma, row0, lane, lane_base + c, n0 + c, M, N);
