@@ -12,8 +12,9 @@ the B x B logits are never written).  Every workspace the backward needs is
 saved with the graph, so several forwards may precede their backwards.
 """
 
-from ctypes import byref, c_size_t
+from ctypes import byref, c_double, c_size_t
 from functools import lru_cache
+from operator import index
 
 import torch
 
@@ -32,10 +33,21 @@ def _dtype_code(t, precision=None):
     raise TypeError("parameters must be float32 or float64")
 
 
-# Descriptors and workspace sizes depend on shapes and options alone: kept per value (typed: 17.0 and
-# numpy.int64(17) are refused as field values whether or not 17 was seen).
-@lru_cache(maxsize=256, typed=True)
+# Descriptors and workspace sizes depend on shapes and options alone: kept per value.  Widths and
+# options may be any object that converts (0-d tensors and arrays, NumPy scalars), whose value may
+# change between calls: they become numbers before the lookup, by the rules of the descriptors' fields
+# (index() and c_double refuse what the fields refuse).
 def _mlp_plan(in0, in1, hidden, layers, out, layernorm, dtype, M):
+    return _mlp_plan_kept(index(in0), index(in1), index(hidden), index(layers), index(out), layernorm, dtype, M)
+
+
+def _loss_plan(energy, loss, sym_reduction, penalty_axis, temperature, beta, dtype, path, B, R):
+    return _loss_plan_kept(energy, loss, sym_reduction, penalty_axis, c_double(temperature).value,
+                           c_double(beta).value, dtype, path, B, R)
+
+
+@lru_cache(maxsize=256, typed=True)
+def _mlp_plan_kept(in0, in1, hidden, layers, out, layernorm, dtype, M):
     desc = api.CrlMlpDesc(in0, in1, hidden, layers, out, layernorm, dtype)
     nbytes = c_size_t()
     api.check(api.lib().crl_mlp_saved_bytes(byref(desc), M, byref(nbytes)))
@@ -48,7 +60,7 @@ def _mlp_plan(in0, in1, hidden, layers, out, layernorm, dtype, M):
 
 
 @lru_cache(maxsize=256, typed=True)
-def _loss_plan(energy, loss, sym_reduction, penalty_axis, temperature, beta, dtype, path, B, R):
+def _loss_plan_kept(energy, loss, sym_reduction, penalty_axis, temperature, beta, dtype, path, B, R):
     desc = api.CrlLossDesc(api.ENERGY[energy], api.LOSS[loss], api.SYM[sym_reduction], api.PENALTY[penalty_axis],
                            temperature, beta, dtype, api.PATH[path])
     nbytes = c_size_t()
