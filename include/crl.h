@@ -502,7 +502,8 @@ typedef struct crl_mlp_desc {
 /* Bytes of the activation workspace `saved` for M rows. */
 int crl_mlp_saved_bytes(const crl_mlp_desc* d, int32_t M, size_t* bytes);
 /* y [M][out] = MLP(concat(x0 [M][in0], x1 [M][in1])) with params in the flat
- * layout above; stores what backward needs in `saved`. */
+ * layout above; stores what backward needs in `saved`.  y (and dy, dparams, dx0,
+ * dx1 below) may start on any element boundary. */
 int crl_mlp_forward(const crl_mlp_desc* d, const void* params, const float* x0, const float* x1,
                     int32_t M, void* y, void* saved, void* stream);
 /* Given dy [M][out]: writes dparams (flat layout; overwritten) and, if not

@@ -278,6 +278,12 @@ __device__ __forceinline__ uint32_t mask_pair(uint32_t x, uint32_t m) {
   return x & (lo | hi);
 }
 
+// FP32 rows that take 16-byte accesses: the callers' own arrays (an op-level output
+// or gradient) may start on any 4-byte boundary.
+__device__ __forceinline__ bool rows_aligned16(const float* p, int ld) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld & 3) == 0;
+}
+
 // 32 columns of a gradient output (weights, split first-layer weights, first-layer inputs).
 __device__ __forceinline__ void epilogue_grad32(const EpiDesc& e, uint8_t* st, int row0, int lane, const float* v,
                                                 int col0, int M, int N) {
@@ -286,7 +292,7 @@ __device__ __forceinline__ void epilogue_grad32(const EpiDesc& e, uint8_t* st, i
     case kEpiBwdDW: {
       float* dW = static_cast<float*>(e.out0);
       if (col0 < e.kin) {
-        if ((e.kin & 3) == 0)
+        if (rows_aligned16(dW, e.kin))
           emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
             if (row0 + r < M && col0 + k < e.kin)
               *reinterpret_cast<float4*>(dW + (size_t)(row0 + r) * e.kin + col0 + k) = x;
@@ -393,7 +399,7 @@ __device__ __forceinline__ void epilogue_f32x32(const GemmProblem* P, const EpiD
           *reinterpret_cast<float4*>(st + stage128(lane, q)) =
               make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         stage_publish(&P->o0, st, lane, col0, row0);
-      } else if ((e.ld0 & 3) == 0 && (N & 3) == 0) {
+      } else if (rows_aligned16(z, e.ld0) && (N & 3) == 0) {
         emit_f32x4(st, lane, v, [&](int r, int k, float4 x) {
           if (row0 + r < M && col0 + k < N) *reinterpret_cast<float4*>(z + (size_t)(row0 + r) * e.ld0 + col0 + k) = x;
         });
