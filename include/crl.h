@@ -508,8 +508,9 @@ int crl_mlp_forward(const crl_mlp_desc* d, const void* params, const float* x0, 
                     int32_t M, void* y, void* saved, void* stream);
 /* Given dy [M][out]: writes dparams (flat layout; overwritten) and, if not
  * NULL, dx0 [M][in0] / dx1 [M][in1].  dparams may be NULL (input gradient only).
- * The padding between the layout's tensors is set to 0 for CRL_PREC_BF16 and left
- * as it was for the other dtypes. */
+ * dparams holds the whole layout, every tensor padded to 64 elements, the last bias
+ * too: the padding is set to 0 for CRL_PREC_BF16 (including after the last tensor)
+ * and left as it was for the other dtypes. */
 int crl_mlp_backward(const crl_mlp_desc* d, const void* params, const float* x0, const float* x1,
                      int32_t M, const void* saved, const void* dy, void* dparams, void* dx0,
                      void* dx1, void* stream);

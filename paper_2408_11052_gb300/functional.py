@@ -90,8 +90,8 @@ class EncoderMLP(torch.autograd.Function):
                                     None if x1c is None else x1c.data_ptr(), M, y.data_ptr(), saved.data_ptr(),
                                     api.stream_handle()))
         ctx.desc = desc
-        # the BF16 backward writes the whole layout, its padding too
-        ctx.whole = desc.dtype == api.PREC["bf16"] and params.numel() == count
+        # the BF16 backward writes the whole layout, the padding after every tensor too
+        ctx.count = count if desc.dtype == api.PREC["bf16"] else 0
         ctx.has_x1 = x1 is not None
         ctx.save_for_backward(params, x0c, x1c if x1c is not None else x0c, saved)
         return y
@@ -104,7 +104,15 @@ class EncoderMLP(torch.autograd.Function):
             x1c = None
         desc = ctx.desc
         M = x0c.shape[0]
-        dparams = (torch.empty_like if ctx.whole else torch.zeros_like)(params) if ctx.needs_input_grad[0] else None
+        dparams = None
+        if ctx.needs_input_grad[0]:
+            n = params.numel()
+            if n == ctx.count:
+                dparams = torch.empty_like(params)
+            elif n < ctx.count:   # parameters that end with the last bias, short of its padding
+                dparams = params.new_empty(ctx.count)[:n].view(params.shape)
+            else:
+                dparams = torch.zeros_like(params)
         dx0 = torch.empty(M, desc.in0, dtype=params.dtype, device=params.device) if ctx.needs_input_grad[1] else None
         dx1 = (torch.empty(M, desc.in1, dtype=params.dtype, device=params.device)
                if (x1c is not None and ctx.needs_input_grad[2]) else None)
