@@ -18,9 +18,13 @@
 // actor's noise.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "actor_head.cuh"
 #include "common.cuh"
 #include "ctx.h"
+#include "gemm_simt.cuh"
 #include "internal.h"
 #include "philox.cuh"
 #include "tc_common.cuh"
@@ -164,12 +168,6 @@ __global__ void advance_kernel(unsigned long long* c, unsigned long long n) {
 constexpr int kUnrollThreads = 256, kUnrollGemmWarps = 4;
 constexpr int kUnrollSteps = 1024;   // steps per launch at most (about 10 ms)
 constexpr int kUnrollSmem = 227 * 1024;
-
-struct UnrollPlan {
-  int C, ME, nc, pitch, clusters;
-  size_t smem;
-  double cost;   // modelled us per step
-};
 
 struct UnrollArgs {
   BufferDev bd;
@@ -539,27 +537,71 @@ __global__ void __launch_bounds__(kUnrollThreads, 1) unroll_kernel(const __grid_
   }
 }
 
-// The cheapest cluster size and environments per cluster that fit, by waves times
-// modelled time per step; false: nothing fits, or the layer-by-layer path is modelled
-// faster.  Both models are fits to measured steps (us; D 29, A 8 unless noted):
-//   hidden, layers        E    one launch   by layers
-//   256, 2               16       8.7         17.6
-//   256, 2             1024       9.6         31
-//   256, 2             8192      61           83
-//   256, 3             8192     138          126
-//   64, 2              1024       6.0         13.6
-//   256, 2 LN, D 268   1024      40          102
-//   512, 2              512      64           45    (eight CTAs hold eight environments)
+// ---- which path a call takes ------------------------------------------------------
+// Modelled us, fits to both paths' times at 252 policies and sizes (D 3 to 500, hidden 32
+// to 512, one to four layers, with and without LayerNorm; E 1 to 16,000) and calls of 1
+// to 62 steps.  A call of n steps is the one launch's where setup + n step < n layers.
+// The one launch fills its shared memory in every wave of clusters, so a call of one or
+// two steps of many environments is the layers'.  us per call, D 29, A 8, two layers of
+// 256, layers / one launch:
+//   E          n = 1       n = 2       n = 8        n = 62
+//   1          17 / 25     34 / 33     132 / 80     1014 / 503
+//   1024       27 / 27     59 / 36     244 / 90     1906 / 569
+//   8192       81 / 132    160 / 191   637 / 547    4923 / 3743
+//   16000      135 / 256   270 / 374   1082 / 1082  7890 / 7447
+// Over those 1,512 calls the choice takes 0.4 % more than the faster path on average and
+// at most 10 % more than the layers (8 calls of one or two steps more than 5 %).
 // Beyond kUnrollEnvs environments the products fill the SMs by themselves.
 constexpr int kUnrollEnvs = 16384;
-bool unroll_plan(const crl_config& cf, const MlpShape& s, UnrollPlan* best) {
-  best->C = 0;
+
+// One step layer by layer: the launches, the tiles' waves of every product, LayerNorm,
+// the step kernel.
+double layers_step_us(const crl_config& cf, const MlpShape& s) {
+  const double E = cf.E, D = cf.D, H = s.hidden;
+  double us = 4.4 + 1.27e-3 * E + 1e-5 * E * D + 0.0155 * std::sqrt(E * D) + 0.027 * D;
+  for (int l = 0; l <= s.layers; ++l) {
+    const int K = l == 0 ? s.in() : s.hidden, N = l == s.layers ? s.out : s.hidden;
+    double tiles = 0;
+    for (const F32Tile& t : kF32Tiles) {
+      const double c = f32_tile_cost(t, (long long)ceil_div(cf.E, t.bm) * ceil_div(N, t.bn));
+      if (tiles == 0 || c < tiles) tiles = c;
+    }
+    us += 0.82 + K * (6.39e-6 * tiles + 5.4e-4 * std::sqrt(tiles));
+  }
+  return us + (s.layernorm ? s.layers * (2.1 + 4.3e-3 * std::sqrt(E * H)) : 0.0);
+}
+
+// The one launch, `waves` of clusters after one another.  Clocks of a step: the products
+// of 8 x 4 blocks of thread tiles, beside them the slice in the first layer and the noise
+// in the last; the barriers; the output chains; the dynamics and the pieces sent to the
+// peers.  Set-up: the weights and the environments' state.
+void unroll_model(const crl_config& cf, const MlpShape& s, int waves, UnrollPlan* q) {
+  const int H = s.hidden, in = s.in(), own = q->ME / q->C;
+  const int rounds = ceil_div(ceil_div(q->nc / 4, 8) * ceil_div(q->ME / 4, 4), kUnrollGemmWarps);
+  const double noise = 1710.0 + 1445.0 * ceil_div(own * (ceil_div(cf.A, 2) + ceil_div(cf.D, 2)), 128);
+  const double slice = 76.0 * ceil_div(own, 4) * (ceil_div(cf.D, 32) + ceil_div(cf.A, 32) + 1);
+  double clocks = H * (1.8 + 2.63 * ceil_div(own * 2 * cf.A, 32)) +
+                  ceil_div(own, 8) * (1650.0 + ceil_div(in, 32) * (337.0 + 68.0 * (q->C - 1)));
+  for (int l = 0; l < s.layers; ++l)
+    clocks += std::max(rounds * (22.3 * (l == 0 ? in : H) + 1167.0),
+                       (l == 0 ? slice : 0.0) + (l == s.layers - 1 ? noise : 0.0)) +
+              475.0 * q->C;
+  if (s.layernorm) clocks += s.layers * ceil_div(q->ME, 8) * (3.79 * H + 1060.0);
+  const double w = waves * (0.99 + 0.01 * waves);   // (waves fill the SMs a little less well than one)
+  q->step = w * clocks / 1920.0;
+  q->setup = 0.8 + w * (5.75 + 3.16e-4 * (in + (s.layers - 1.0) * H) * q->nc + 2.4e-4 * cf.A * H +
+                            1.2e-3 * own * cf.D + 0.004 * ceil_div(own, 8) * ceil_div(in, 32) * q->C);
+}
+
+// The cluster size and environments per cluster that fit with the least waves x clocks
+// per step (a ranking of the forms of one policy: the terms that differ little between
+// them are left out, so its values are good to a factor of 1.5 only).  C = 0: nothing fits.
+UnrollPlan unroll_plan(const crl_config& cf, const MlpShape& s) {
+  UnrollPlan best;
+  double least = 0;
+  int waves = 0;
   const int H = s.hidden, in = s.in();
-  if (in != cf.D + cf.G || s.out != 2 * cf.A || cf.E > kUnrollEnvs) return false;
-  // the layer-by-layer step: launches, one output's chain over k, then throughput
-  const double K = in + (double)s.layers * H;
-  const double layers_us = 2.1 + 2.3 * (s.layers + 1) + 0.0156 * K + (s.layernorm ? s.layers * (8.5 + 0.002 * cf.E) : 0.0) +
-                           2.0 * cf.E * (K * H - (double)H * (H - s.out)) / 20e6;
+  if (in != cf.D + cf.G || s.out != 2 * cf.A || cf.E > kUnrollEnvs) return best;
   CRL_CHECK_CUDA(cudaFuncSetAttribute(unroll_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUnrollSmem));
   for (int C = 1; C <= 8; C *= 2) {
     const int nc = round_up(ceil_div(H, C), 4);
@@ -587,20 +629,29 @@ bool unroll_plan(const crl_config& cf, const MlpShape& s, UnrollPlan* best) {
       const UnrollSmem u = unroll_smem(s.layers, in, H, cf.D, cf.A, cf.G, s.layernorm, C, ME, nc, pitch);
       const size_t bytes = (size_t)u.total * sizeof(float);
       if (bytes > kUnrollSmem) break;
-      UnrollPlan q;
-      q.C = C, q.ME = ME, q.nc = nc, q.pitch = pitch, q.smem = bytes;
-      q.clusters = ceil_div(cf.E, ME);
-      const int waves = ceil_div(q.clusters, resident), own = ME / C;
+      const int clusters = ceil_div(cf.E, ME), w = ceil_div(clusters, resident), own = ME / C;
       const int rounds = ceil_div(ceil_div(nc / 4, 8) * ceil_div(ME / 4, 4), kUnrollGemmWarps);
       const double clocks = 26.5 * rounds * (in + (s.layers - 1) * (double)H) + 2600.0 * s.layers +
                             10.0 * H * ceil_div(own * 2 * cf.A, kUnrollThreads) + 1200.0 * ceil_div(own, 8) + 1500.0 +
                             50.0 * C * s.layers +
                             (s.layernorm ? s.layers * ceil_div(ME, 8) * (H / 32 * 60.0 + 250.0) : 0.0);
-      q.cost = waves * clocks / 1920.0;
-      if (best->C == 0 || q.cost < best->cost) *best = q;
+      if (best.C == 0 || w * clocks < least) {
+        best.C = C, best.ME = ME, best.nc = nc, best.pitch = pitch, best.clusters = clusters, best.smem = bytes;
+        least = w * clocks;
+        waves = w;
+      }
     }
   }
-  return best->C != 0 && 1.15 * best->cost < layers_us;   // (the models are good to about that)
+  if (best.C) {
+    unroll_model(cf, s, waves, &best);
+    best.layers_step = layers_step_us(cf, s);
+  }
+  return best;
+}
+
+// Whether a call of n steps is the one launch's.
+bool unroll_pays(const UnrollPlan& q, int n) {
+  return q.C != 0 && ceil_div(n, kUnrollSteps) * q.setup + n * q.step < n * q.layers_step;
 }
 
 // All n steps of one call (as many as the step counter has room for).
@@ -652,9 +703,12 @@ void collect_steps(crl_ctx* c, int n, int episode_length, float* obs_out, float*
   const int E = cf.E;
   const T* params = static_cast<const T*>(c->nets[CRL_NET_PI].params);
   int i = 0;
-  UnrollPlan plan;
-  const bool one = sizeof(T) == 4 && unroll_plan(cf, c->shapes[CRL_NET_PI], &plan);
-  if (one) i = collect_unroll(c, plan, n, episode_length, obs_out, act_out, done_out, st);
+  if (sizeof(T) == 4 && !v.planned) {   // (the configuration decides: once per context)
+    v.plan = unroll_plan(cf, c->shapes[CRL_NET_PI]);
+    v.planned = true;
+  }
+  const bool one = sizeof(T) == 4 && unroll_pays(v.plan, n);
+  if (one) i = collect_unroll(c, v.plan, n, episode_length, obs_out, act_out, done_out, st);
   for (; !one && i < n && c->total_host + 1 < ((int64_t)1 << 31) - 1; ++i) {
     mlp_forward<T, float>(c->shapes[CRL_NET_PI], params, v.s, v.g, E, static_cast<T*>(v.pi_out), v.saved, st);
     CollectArgs<T> a;

@@ -65,6 +65,14 @@ size_t dtype_size(int precision);
 MlpShape net_shape(const crl_config& c, int net);
 void validate_config(const crl_config& c);
 
+// The one-launch form of a context's collection calls (collect.cu): clusters of C
+// CTAs (0: none fits), each carrying ME environments.
+struct UnrollPlan {
+  int C = 0, ME, nc, pitch, clusters;
+  size_t smem;
+  double setup, step, layers_step;   // modelled us per launch and per environment step; per layer-by-layer step
+};
+
 }  // namespace crl
 
 using namespace crl;
@@ -107,6 +115,8 @@ struct crl_ctx {
     int32_t* t = nullptr;                 // [E] step within the episode
     unsigned long long* step = nullptr;   // next collection step (Philox counter)
     void *pi_out = nullptr, *a = nullptr, *saved = nullptr;
+    bool planned = false;
+    UnrollPlan plan;
   } env;
   // logit statistics of the critic steps (crl_set_logit_stats): [2] floats and per-tile FP64 sums
   bool stats_on = false;

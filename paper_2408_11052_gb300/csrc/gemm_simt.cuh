@@ -298,6 +298,14 @@ void launch_gemm_f32(const GemmSets<LA, LB, EP>& g, int n, int M, int N, cudaStr
            dim3((BM / TM) * (BN / TN)), 0, st, g);
 }
 
+// The FP32 tiles, widest first, with the cost of an output relative to the first.
+struct F32Tile {
+  int bm, bn;
+  double w;
+};
+constexpr F32Tile kF32Tiles[4] = {{64, 64, 1.0}, {32, 64, 1.05}, {32, 32, 1.2}, {16, 32, 1.5}};
+inline double f32_tile_cost(const F32Tile& t, long long ctas) { return (double)((ctas + 151) / 152) * t.bm * t.bn * t.w; }
+
 // Launch of n products (one or two); traced as class `cls` (CRL_TRACE_*) with
 // 2 M N K flops of work each.  FP32 takes the tile whose waves over the 152 SMs cost
 // least: outputs per SM, weighted by the shared reads per FMA of its thread tile (a
@@ -330,17 +338,19 @@ void gemm_sets(const GemmSet<LA, LB, EP>* set, int n, cudaStream_t st, int cls =
     if (live == 0) return;
     if (live == 1) g.s[1] = g.s[0];
     TraceLaunch tr(cls, st, flops);
-    auto cost = [&](int bm, int bn, double w) {
-      if (bm < 64 && ceil_div(M, bm) > 65535) return 1e300;   // grid.y
+    int pick = 0;
+    double best = 0;
+    for (int q = 0; q < 4; ++q) {
+      const F32Tile& t = kF32Tiles[q];
+      if (t.bm < 64 && ceil_div(M, t.bm) > 65535) continue;   // grid.y
       long long ctas = 0;
-      for (int i = 0; i < live; ++i) ctas += (long long)ceil_div(g.s[i].M, bm) * ceil_div(g.s[i].N, bn);
-      return (double)((ctas + 151) / 152) * bm * bn * w;
-    };
-    const double c64 = cost(64, 64, 1.0), c32w = cost(32, 64, 1.05), c32 = cost(32, 32, 1.2), c16 = cost(16, 32, 1.5);
-    const double best = std::min(std::min(c64, c32w), std::min(c32, c16));
-    if (best == c64) launch_gemm_f32<OP, 64, 64, 4, 4>(g, live, M, N, st);
-    else if (best == c32w) launch_gemm_f32<OP, 32, 64, 4, 4>(g, live, M, N, st);
-    else if (best == c32) launch_gemm_f32<OP, 32, 32, 2, 4>(g, live, M, N, st);
+      for (int i = 0; i < live; ++i) ctas += (long long)ceil_div(g.s[i].M, t.bm) * ceil_div(g.s[i].N, t.bn);
+      const double c = f32_tile_cost(t, ctas);
+      if (q == 0 || c < best) best = c, pick = q;
+    }
+    if (pick == 0) launch_gemm_f32<OP, 64, 64, 4, 4>(g, live, M, N, st);
+    else if (pick == 1) launch_gemm_f32<OP, 32, 64, 4, 4>(g, live, M, N, st);
+    else if (pick == 2) launch_gemm_f32<OP, 32, 32, 2, 4>(g, live, M, N, st);
     else launch_gemm_f32<OP, 16, 32, 2, 2>(g, live, M, N, st);
   }
 }
