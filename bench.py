@@ -20,7 +20,10 @@ on the 32-agent sweep.  "relabel" reports the standalone sample + relabel
 kernel at 2^20 and 2^22 samples per launch on Humanoid-shaped rows (its HBM
 roofline).
 
-Prints one JSON line (rank 0).  Under torchrun (N > 1) every rank runs its own
+Prints one JSON line (rank 0) of a few KB on standard output: the headline and a
+summary of the rest; everything (per-tensor errors, per-class breakdowns, every
+autotuner candidate) goes to standard error as one line, "bench detail: {...}".
+Under torchrun (N > 1) every rank runs its own
 independent agent (its own Philox key and buffer): weak scaling, no data-path
 collective; timing takes the max over ranks.
 """
@@ -736,6 +739,78 @@ def run_sweep(args, dev, flush):
     return line
 
 
+def rounded(x, digits=5):
+    """x with every float at `digits` significant digits, cosines at 9 (containers walked)."""
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}")
+    if isinstance(x, dict):
+        return {k: rounded(v, 9 if k.endswith("_cos") else digits) for k, v in x.items()}
+    return [rounded(v, digits) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def pick(d, *keys):
+    return {k: d[k] for k in keys if k in d}
+
+
+def error_summary(err):
+    arms = {k: pick(v, "status", "grad_worst_rel_err", "grad_worst_cos") |
+            {"loss_worst_rel_err": max(v["loss_rel_err"].values())}
+            for k, v in err.items() if isinstance(v, dict) and "loss_rel_err" in v}
+    return {"bars": err["bars"]} | arms if arms else err
+
+
+def summary_line(line):
+    """The line as printed: the contract's keys whole, the rest by its figures.  The whole
+    line is tens of KB (the autotuner's candidates, per-tensor errors), more than a reader
+    of a log's tail gets back."""
+    out = dict(line)
+    for k in ("breakdown", "gemm_tuning", "error", "workloads", "relabel", "collect_loop", "comparator", "cpu_baseline",
+              "roofline"):
+        out.pop(k, None)
+    if "roofline" in line:
+        r = {k: v for k, v in line["roofline"].items() if k not in ("note", "timing")}
+        if "issued" in r:
+            r["issued"] = pick(r["issued"], "tflops", "frac")
+        out["roofline"] = r
+    if "breakdown" in line:
+        out["us_per_step"] = {k: v["us_per_step"] for k, v in line["breakdown"].items() if isinstance(v, dict)}
+    comps = line.get("comparator")
+    if comps is not None:
+        keys = ("precision", "path", "grouped", "autotune", "value", "unit", "ms_per_step", "speedup")
+        out["comparator"] = [pick(c, *keys) for c in comps] if isinstance(comps, list) else pick(comps, *keys)
+    if "error" in line:
+        out["error"] = error_summary(line["error"])
+    if "workloads" in line:
+        out["workloads"] = {}
+        for k, w in line["workloads"].items():
+            o = pick(w, "value", "unit", "ms_per_step")
+            o["e2e"] = w["e2e"]["value"]
+            o["roofline_frac"] = w["roofline"]["frac"]
+            o["sm_mhz"], o["reasons"] = w["clocks"]["sm_mhz"], w["clocks"]["reasons"]
+            if isinstance(w.get("comparator"), dict):
+                o["speedup_over_fp32_plain"] = w["comparator"]["speedup"]
+            if "error" in w:
+                o["error"] = {a: pick(v, "grad_worst_rel_err", "grad_worst_cos")
+                              for a, v in error_summary(w["error"]).items() if a != "bars"}
+            out["workloads"][k] = o
+    if "relabel" in line:
+        out["relabel"] = {"workload": line["relabel"]["workload"], "results": [
+            pick(r, "samples_per_launch", "value", "unit", "us_per_launch", "achieved_gbs") |
+            {"frac": r["roofline"]["frac"]} for r in line["relabel"]["results"]]}
+    if "collect_loop" in line:
+        out["collect_loop"] = pick(line["collect_loop"], "env_steps_per_s", "update_steps_per_s", "envs", "unroll",
+                                   "collect_ms_per_round", "update_ms_per_round")
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = pick(line["cpu_baseline"], "value", "unit", "cores", "kind", "sample")
+    whole = ("value", "ms_per_step")
+    return {k: v if k in whole else rounded(v, 7) if k in ("e2e", "samples_per_s") else rounded(v) for k, v in out.items()}
+
+
+def print_line(line):
+    print("bench detail: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(summary_line(line)), flush=True)
+
+
 def api_losses():
     from paper_2408_11052_gb300 import api as _api
     return _api.LOSS
@@ -804,7 +879,7 @@ def main():
     torch.cuda.set_stream(torch.cuda.Stream(device=dev))
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     if args.workload == "sweep":
-        print(json.dumps(run_sweep(args, dev, flush)), flush=True)
+        print_line(run_sweep(args, dev, flush))
         return
     if args.only_relabel:
         rw, res = relabel_throughput(dev, flush)
@@ -907,7 +982,7 @@ def main():
     if cpu is not None:
         line["cpu_baseline"] = cpu
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print_line(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
