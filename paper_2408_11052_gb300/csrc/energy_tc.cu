@@ -1361,18 +1361,8 @@ struct EnergyTask {   // 128-byte aligned by its tensor maps
   CUtensorMap tmX, tmY;
   FwdArgs f;
   BwdArgs row, col;
-  PrepSide s0, s1;
-  int B, R, energy, n;
+  int n;
 };
-
-__global__ void __launch_bounds__(1024) prep_multi_kernel(const EnergyTask* __restrict__ tasks,
-                                                         const int* __restrict__ begin, int n) {
-  pdl_enter();
-  int lb, nb;
-  const EnergyTask& t = tasks[segment_of(begin, n, blockIdx.x, lb, nb)];
-  const int half = nb / 2;
-  prep_body(t.B, t.R, t.energy, lb < half ? t.s0 : t.s1, lb < half ? lb : lb - half);
-}
 
 template <bool OBJ>
 __global__ void __launch_bounds__(kFwdThreads, 1) fwd_multi_kernel(const EnergyTask* __restrict__ tasks,
@@ -1696,15 +1686,15 @@ size_t energy_tc_ticket_bytes(int B) {
   return (size_t)(2 * n + 1) * 4;
 }
 
-const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& all, int stage, cudaStream_t st) {
-  // the -L1 agents run their own SIMT launches; the rest share one launch per stage
+const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& all, bool backward, cudaStream_t st) {
+  // the -L1 agents run their own SIMT launches; the rest share one launch
   std::vector<EnergyAgent> agents;
   for (const EnergyAgent& g : all) {
     if (g.ls.energy != CRL_ENERGY_L1) {
       agents.push_back(g);
-    } else if (stage == 1) {
+    } else if (!backward) {
       energy_tc_forward(*g.e, g.ls, g.B, g.phi, g.psi, g.loss4, nullptr, g.r, g.c, g.ws, g.status, g.t_bump, st);
-    } else if (stage == 2) {
+    } else {
       energy_tc_backward(*g.e, g.ls, g.B, g.phi, g.psi, g.r, g.c, 1.0, g.dphi, g.dpsi, g.ws, g.status, st);
     }
   }
@@ -1721,12 +1711,7 @@ const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& al
     const EnergyTc& e = *g.e;
     t.tmX = e.tmX;
     t.tmY = e.tmY;
-    t.B = g.B;
-    t.R = e.R;
-    t.energy = g.ls.energy;
     t.n = (g.B + kTile - 1) / kTile;
-    t.s0 = PrepSide{g.phi, e.X, e.auxX};
-    t.s1 = PrepSide{g.psi, e.Y, e.auxY};
     t.f = fwd_args(e, g.ls, g.B, g.ws, g.loss4, g.r, g.c, g.t_bump, g.status);
     t.row = bwd_args(e, g.ls, g.B, g.phi, g.r, g.c, 1.0, g.dphi, g.status, t.f);
     t.col = t.row;
@@ -1737,20 +1722,16 @@ const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& al
     t.col.lse_other = g.r;
     t.col.own_f32 = g.psi;
     t.col.d_out = g.dpsi;
-    const int nb = stage == 0 ? 2 * ceil_div(g.B, 32) : (stage == 1 ? t.n * t.f.nC : 2 * t.n);
-    begin[i + 1] = begin[i] + nb;
+    begin[i + 1] = begin[i] + (backward ? 2 * t.n : t.n * t.f.nC);
     Rmax = std::max(Rmax, e.R);
-    work += (stage == 1 ? 2.0 : 8.0) * g.B * g.B * e.R * (stage == 0 ? 0.0 : 1.0);
+    work += (backward ? 8.0 : 2.0) * g.B * g.B * e.R;
   }
   const char* err = nullptr;
   const EnergyTask* dt = cache.get(tasks, st, &err);
   if (!dt) return err;
   const int* db = cache.get(begin, st, &err);
   if (!db) return err;
-  if (stage == 0) {
-    TraceLaunch tr(CRL_TRACE_ENERGY, st, work);
-    launch_k(prep_multi_kernel, dim3(begin[na]), dim3(1024), 0, st, dt, db, na);
-  } else if (stage == 1) {
+  if (!backward) {
     static bool attr = false;
     if (!attr) {
       cudaFuncSetAttribute(fwd_multi_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem(256));

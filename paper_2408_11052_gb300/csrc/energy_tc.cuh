@@ -68,7 +68,8 @@ struct EnergyAgent {
   __nv_bfloat16* dpsi;
   unsigned* status;
 };
-// stage 0: prepare, 1: forward (+ loss), 2: backward -- one launch over all agents.
-const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& agents, int stage, cudaStream_t st);
+// The forward (with the loss) or the backward of every agent, whose operands the
+// encoders' output layers have written.
+const char* energy_tc_multi(BlobCache& cache, const std::vector<EnergyAgent>& agents, bool backward, cudaStream_t st);
 
 }  // namespace crl

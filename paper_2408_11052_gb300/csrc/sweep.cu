@@ -158,7 +158,7 @@ void body_grouped(crl_sweep* sw, cudaStream_t st) {
                              &c->ctr->t_critic, P.dz[P.layers], Q.dz[Q.layers], &c->ctr->status});
   }
   // (the operands were written by the encoders' output layers: no prepare stage)
-  for (int stage = 1; stage < 3; ++stage) sweep_check(energy_tc_multi(sw->tables, ea, stage, st));
+  for (bool backward : {false, true}) sweep_check(energy_tc_multi(sw->tables, ea, backward, st));
   sweep_check(bf_backward(sw->groups, bwd.data(), (int)bwd.size(), status, st));
   // Adam for every phi and psi; the actors' head forwards (a' into phi's input:
   // they read only the policies' outputs) run as extra blocks of the same launch

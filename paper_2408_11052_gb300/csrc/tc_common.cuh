@@ -173,15 +173,6 @@ __device__ __forceinline__ uint32_t mapa_shared(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
 }
-// Bulk copy of `bytes` (a multiple of 16; both addresses 16-byte aligned) from
-// this CTA's shared memory to shared memory of another CTA of the cluster,
-// completing the bytes on that CTA's barrier (dst and bar: mapa_shared addresses).
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "r"(smem_u32(src)), "r"(bytes), "r"(bar)
-      : "memory");
-}
 // Named barrier `id` over `nthreads` threads (a multiple of 32) that also
 // returns the AND of every participant's pred: a decision all of them share.
 __device__ __forceinline__ bool named_barrier_and(uint32_t id, uint32_t nthreads, bool pred) {
