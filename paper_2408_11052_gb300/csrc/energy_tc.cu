@@ -11,19 +11,20 @@
 // 1 / |phi| (cos).  S = X Y^T is formed 128 x 128 at a time in TMEM; the L2
 // energies use d^2 = |x|^2 + |y|^2 - 2 S (clamped at 0).
 //
-// forward:  one CTA per (row tile I, column tile J): S -> F tile in shared
-//           memory -> per-row (max, sum) over the tile's columns and per-column
-//           (max, sum) over the tile's rows, written as partials; the diagonal
-//           entries F_ii.  A one-block finalize merges the partials into
-//           r_i = LSE_j F_ij, c_j = LSE_i F_ij and the loss parts.
+// forward:  one CTA per row tile and chunk of column tiles: S (TMEM) -> F in
+//           registers -> per-row (max, sum) over the chunk's columns and
+//           per-column (max, sum) over the tile's rows, written as partials;
+//           the diagonal entries F_ii.  A finalize of 2 n blocks (n row tiles, n
+//           column tiles) merges the partials into r_i = LSE_j F_ij and c_j =
+//           LSE_i F_ij; its last block forms the loss parts.
 // backward: the "row pass" (one CTA per 128 rows of phi) loops over column
 //           tiles: S -> coefficient tile H (dL/dF times the energy's chain-rule
 //           factor) written as a BF16 K-major operand in shared memory ->
 //           acc += H psi (TMEM).  dphi = acc - rowsum(H) phi (L2, L2^2), acc
 //           (dot), or the tangent projection of acc (cos).  The "column pass"
 //           is the same kernel with the roles of phi and psi (and of r and c)
-//           exchanged.  Both write their result as BF16 dy [B][R] and dy^T
-//           [R][B], the layout the encoder backward consumes.
+//           exchanged.  Both write their result as BF16 dy [B][R], which the
+//           encoder backward reads, or as FP32 (the op-level calls).
 //
 // The other objectives of App. A.2 / §5.2 (FlatNCE, forward-backward, DPO, IPO,
 // SPPO, NCE-binary; definitions and readings as in the plain path) ride on the

@@ -36,8 +36,8 @@ inline int pad8(int x) { return (x + 7) / 8 * 8; }
 
 // ---- element kernels ----------------------------------------------------------------
 // FP32 rows [rows][n] -> BF16 rows [rows][ld]; four columns per thread where the rows are aligned.
-// gaps: block 0 clears the padding words between the tensors of a flat gradient
-// array (at most 63 after each).
+// gaps: block 0 clears the padding words after the tensors of a flat gradient array
+// (at most 63 after each, the last too).
 struct GradGaps {
   float* grads;   // may be null
   int n;

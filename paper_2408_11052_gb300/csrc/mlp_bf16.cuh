@@ -180,14 +180,14 @@ const char* bf_net_maps(BfNet& n, int M);
 void bf_net_shadow(BfNet& n, const float* params, cudaStream_t st);
 // Row length of x0 (the split input and the ones column): pad8(2 in + 1).
 int bf_net_x0_ld(const BfNet& n);
-// Pack the FP32 input concat(x0 [M][in0], x1 [M][in1]) into x0.
 // Everything an op-level forward needs in a fresh workspace, in one launch: the
 // shadows, the split input, the ones columns and K padding, a cleared status word and tickets.
 void bf_net_prepare(BfNet& n, const float* params, const float* x0, const float* x1, int M, unsigned* status,
                     cudaStream_t st);
+// Pack the FP32 input concat(x0 [M][in0], x1 [M][in1]) into x0.
 void bf_net_pack_input(BfNet& n, const float* x0, const float* x1, int M, cudaStream_t st);
 // Store an FP32 gradient dy [M][out] into dz[layers] (BF16).
-// grads (may be null): a flat gradient array whose padding between tensors is set to 0.
+// grads (may be null): a flat gradient array, the padding after every tensor of which is set to 0.
 void bf_net_load_dy(BfNet& n, const float* dy, int M, float* grads, cudaStream_t st);
 
 // The fused energy's BF16 operand written by an encoder's output layer (see

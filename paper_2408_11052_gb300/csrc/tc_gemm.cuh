@@ -983,15 +983,15 @@ __global__ void __launch_bounds__(kPersistentThreads, 1)
 // BN / 2 rows of B (columns BN / 2 r .. of the tile), so a pair moves half the
 // operand bytes of two one-SM tiles of the same work.  The even CTA issues
 // every MMA; its accumulator rows live in the even CTA's TMEM, the others in
-// the odd CTA's.  No multicast: the CTAs exchange plain mbarrier arrivals.
+// the odd CTA's.  No operand load is multicast; the CTAs exchange mbarrier
+// arrivals, the MMA commits among them on both CTAs' barriers at once.
 //   warp 0 / lane 0 -- TMA producer of this CTA's ring;
-//   warp 1 / lane 0 -- even CTA: MMA issuer (waits for its own slot and the
-//                      odd CTA's `pfull` arrival); odd CTA: reports each
+//   warp 1 / lane 0 -- even CTA: MMA issuer.  It waits for its own slot and the
+//                      odd CTA's `pfull` arrival; its commits free each slot
+//                      (`empty`) and announce each finished accumulator (`accf`)
+//                      in both CTAs (a relay warp cost about 0.5 us per slot:
+//                      more than one slot's MMA time).  Odd CTA: reports each
 //                      landed slot to the even CTA's `pfull`;
-//                      its commits free each slot (`empty`) and announce each
-//                      finished accumulator (`accf`) in both CTAs at once (a
-//                      relay warp cost about 0.5 us per slot: more than one
-//                      slot's MMA time);
 //   warps 2..9      -- epilogue of this CTA's 128 rows from TMEM buffer i % 2;
 //                      the pair's sixteen warps release it on the even CTA's `acce`.
 // The epilogue is the one-tile kernel's, so every kernel gives identical outputs
