@@ -684,6 +684,8 @@ def run_sweep(args, dev, flush):
     29 / 64 / 268, repr 64 / 128, 512 envs x 1000 steps each) per update step;
     the grouped BF16 sweep, with the same agents stepped one after another in
     BF16 and in FP32 as comparators."""
+    if args.trace == "auto":   # the sweep's largest class
+        args = argparse.Namespace(**dict(vars(args), trace="gemm"))
     ws = workload.sweep_agents(32)
     B_total = sum(w.B for w in ws)
     main_arm = run_sweep_arm(args, ws, "bf16", "fused", True, dev, flush, args.steps, full=True)

@@ -64,3 +64,19 @@ def test_the_printed_line_is_short_and_keeps_the_contract(capsys):
     assert out["roofline"]["frac"] == 0.11696
     detail = [l for l in got.err.splitlines() if l.startswith("bench detail: ")]
     assert len(detail) == 1 and json.loads(detail[0][len("bench detail: "):]) == line
+
+
+def test_the_sweep_workload_runs_with_the_default_arguments(monkeypatch):
+    """`--workload sweep` alone: its traced pass takes a kernel class (the default, "auto", is not one)."""
+    from paper_2408_11052_gb300 import api
+    seen = []
+
+    def arm(args, ws, precision, path, grouped, dev, flush, steps, full):
+        seen.append(args.trace)
+        return {"ms": 1.0, "e2e_ms": 1.0, "clocks": {}, "launches_per_step": 24, "trace": (10, 1.0, 1e9)}
+
+    monkeypatch.setattr(bench, "run_sweep_arm", arm)
+    args = bench.build_parser().parse_args(["--workload", "sweep", "--no-comparator"])
+    line = bench.run_sweep(args, None, None)
+    assert seen and all(t in api.TRACE for t in seen)
+    assert line["roofline"]["kernel_class"] in api.TRACE
