@@ -149,20 +149,14 @@ __device__ __forceinline__ void shadow_tile(const ShadowTile& t, int r0, int c0,
 __host__ __device__ inline int shadow_tiles_x(const ShadowTile& t) { return (t.kp / t.rep + 63) / 64; }
 __host__ __device__ inline int shadow_tiles(const ShadowTile& t) { return shadow_tiles_x(t) * ((t.rows + 63) / 64); }
 
-__global__ void __launch_bounds__(256) pack_weights_kernel(const __grid_constant__ ShadowTile t) {
-  pdl_enter();
-  __shared__ float tile[64][65];
-  const int nx = shadow_tiles_x(t);
-  shadow_tile(t, 64 * ((int)blockIdx.x / nx), 64 * ((int)blockIdx.x % nx), tile);
-}
-
 // Everything an op-level forward needs before its first product, in one launch
 // (it was a memset of the whole workspace and 2 + 2 (layers + 1) launches): the
 // weight shadows of every layer, the split input with its ones column, the ones
 // column and the K padding of every hidden activation, the status word and the
 // split-K tickets.  Blocks [0, wtiles): weight tiles; then 8 rows per block.  Memory
 // and latency bound: 8 us for 2 x 512 at 8192 rows (the memset alone took 18, the
-// packs 21), 14 us for 4 x 1024.
+// packs 21), 14 us for 4 x 1024.  The weight tiles alone refresh a bound network's
+// shadows: a launch per layer takes 6 to 8 us each at these few tiles.
 struct NetPrep {
   ShadowTile L[CRL_MAX_LAYERS + 1];
   int tile_begin[CRL_MAX_LAYERS + 2];
@@ -1059,32 +1053,37 @@ ShadowTile shadow_of(const BfNet& n, int l, const float* params) {
   const BfLayer& L = n.L[l];
   return ShadowTile{params + L.oW, L.W, L.Wt, L.out, L.in, l == 0 ? 2 : 1, L.nhi, L.kp, L.out_pad};
 }
+
+// The weight tiles of p; returns the bytes they move.
+double shadow_prep(NetPrep& p, const BfNet& n, const float* params) {
+  memset(&p, 0, sizeof(p));
+  p.nl = n.layers + 1;
+  double bytes = 0.0;
+  for (int l = 0; l <= n.layers; ++l) {
+    p.L[l] = shadow_of(n, l, params);
+    p.tile_begin[l + 1] = p.tile_begin[l] + shadow_tiles(p.L[l]);
+    bytes += (double)n.L[l].out * n.L[l].in * 10.0;
+  }
+  return bytes;
+}
 }  // namespace
 
 void bf_net_shadow(BfNet& n, const float* params, cudaStream_t st) {
-  for (int l = 0; l <= n.layers; ++l) {
-    TraceLaunch tr(CRL_TRACE_AUX, st, (double)n.L[l].out * n.L[l].in * 10.0);
-    const ShadowTile t = shadow_of(n, l, params);
-    launch_k(pack_weights_kernel, dim3(shadow_tiles(t)), dim3(256), 0, st, t);
-  }
+  NetPrep p;
+  TraceLaunch tr(CRL_TRACE_AUX, st, shadow_prep(p, n, params));
+  launch_k(net_prep_kernel, dim3(p.tile_begin[p.nl]), dim3(256), 0, st, p);
 }
 
 void bf_net_prepare(BfNet& n, const float* params, const float* x0, const float* x1, int M, unsigned* status,
                     cudaStream_t st) {
   NetPrep p;
-  memset(&p, 0, sizeof(p));
-  p.nl = n.layers + 1;
+  const double bytes = shadow_prep(p, n, params) + (double)M * n.s.in() * 8.0;
   p.M = M;
-  double bytes = (double)M * n.s.in() * 8.0;
-  for (int l = 0; l <= n.layers; ++l) {
-    p.L[l] = shadow_of(n, l, params);
-    p.tile_begin[l + 1] = p.tile_begin[l] + shadow_tiles(p.L[l]);
+  for (int l = 0; l <= n.layers; ++l)
     if (n.L[l].wtick) {
       p.tick[l] = n.L[l].wtick;
       p.ntick[l] = split_tickets(n.L[l], l);
     }
-    bytes += (double)n.L[l].out * n.L[l].in * 10.0;
-  }
   p.s0 = x0;
   p.s1 = x1;
   p.n0 = n.s.in0;
@@ -1376,7 +1375,7 @@ struct AdamUnit {
 };
 
 // Adam on the FP32 master parameters and the refresh of the BF16 shadows:
-// W2 (nhi copies of W_hi, then W_lo; see pack_weights_kernel) row-major
+// W2 (nhi copies of W_hi, then W_lo; see ShadowTile) row-major
 // (coalesced along the tile's columns) and Wt
 // (the transposed single BF16, written through a shared-memory transpose).
 // Bias corrections 1 - b^t = -expm1(t ln b): accurate to a few float ulps
