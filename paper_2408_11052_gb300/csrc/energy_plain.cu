@@ -562,13 +562,15 @@ void infonce_backward(const LossSpec& ls, const T* phi, const T* psi, int B, int
     { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(project_rows_kernel<T>, dim3(nb), dim3(256), 0, st, B, R, w.xh, w.inx, dphi); }
     { TraceLaunch tr_(CRL_TRACE_ENERGY, st, 0.0); launch_k(project_rows_kernel<T>, dim3(nb), dim3(256), 0, st, B, R, w.yh, w.iny, dpsi); }
   } else if (ls.energy == CRL_ENERGY_L1) {
+    static std::atomic<uint64_t> allowed{0};
     const dim3 grid(ceil_div(R, 32), ceil_div(B, 32));
+    const size_t smem = spread_smem(l1_grad_kernel<T>, allowed, 2 * 32 * 33 * sizeof(T), (long long)grid.x * grid.y);
     {
       TraceLaunch tr_(CRL_TRACE_ENERGY, st, 2.0 * B * B * R);
-      launch_k(l1_grad_kernel<T>, grid, dim3(256), 0, st, B, R, H, 0, phi, psi, dphi);
+      launch_k(l1_grad_kernel<T>, grid, dim3(256), smem, st, B, R, H, 0, phi, psi, dphi);
     }
     TraceLaunch tr_(CRL_TRACE_ENERGY, st, 2.0 * B * B * R);
-    launch_k(l1_grad_kernel<T>, grid, dim3(256), 0, st, B, R, H, 1, psi, phi, dpsi);
+    launch_k(l1_grad_kernel<T>, grid, dim3(256), smem, st, B, R, H, 1, psi, phi, dpsi);
   } else {  // dot
     gemm<T>(B, R, B, LoadMK<T>{H, B}, LoadKN<T>{psi, R}, EpiScale<T>{dphi, R, T(1)}, st, CRL_TRACE_ENERGY);
     gemm<T>(B, R, B, LoadTrans<T>{H, B}, LoadKN<T>{phi, R}, EpiScale<T>{dpsi, R, T(1)}, st, CRL_TRACE_ENERGY);

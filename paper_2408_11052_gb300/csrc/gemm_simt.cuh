@@ -294,8 +294,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 
 template <InnerOp OP, int BM, int BN, int TM, int TN, class LA, class LB, class EP>
 void launch_gemm_f32(const GemmSets<LA, LB, EP>& g, int n, int M, int N, cudaStream_t st) {
-  launch_k(gemm_f32_kernel<OP, BM, BN, TM, TN, LA, LB, EP>, dim3(ceil_div(N, BN), ceil_div(M, BM), n),
-           dim3((BM / TM) * (BN / TN)), 0, st, g);
+  static std::atomic<uint64_t> allowed{0};
+  const auto kernel = gemm_f32_kernel<OP, BM, BN, TM, TN, LA, LB, EP>;
+  const dim3 grid(ceil_div(N, BN), ceil_div(M, BM), n);
+  constexpr size_t kFixed = sizeof(F32Ring<LA::kContigK, BM, TM>) + sizeof(F32Ring<LB::kContigK, BN, TN>);
+  launch_k(kernel, grid, dim3((BM / TM) * (BN / TN)), spread_smem(kernel, allowed, kFixed, (long long)grid.x * grid.y * n),
+           st, g);
 }
 
 // The FP32 tiles, widest first, with the cost of an output relative to the first.
