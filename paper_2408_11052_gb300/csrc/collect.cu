@@ -145,7 +145,7 @@ __global__ void advance_kernel(unsigned long long* c, unsigned long long n) {
 // The policy does not change during a call and environments do not touch each
 // other, so one cluster of C CTAs carries ME environments through all n steps
 // without leaving shared memory.  Launched layer by layer, a step of 1024
-// environments with two layers of 256 took 31 us for 2.2 us of FMAs (launches,
+// environments with two layers of 256 takes 25 us for 2.2 us of FMAs (launches,
 // reloading the weights, and 64 to 128 threads' worth of work per SM in between);
 // here it takes 9.2 us (62 steps: 1921 -> 569 us), of which 4.1 are the second
 // layer's products, 1.2 the output layer's chains and 1.3 the barriers.
@@ -545,12 +545,13 @@ __global__ void __launch_bounds__(kUnrollThreads, 1) unroll_kernel(const __grid_
 // two steps of many environments is the layers'.  us per call, D 29, A 8, two layers of
 // 256, layers / one launch:
 //   E          n = 1       n = 2       n = 8        n = 62
-//   1          17 / 25     34 / 33     132 / 80     1014 / 503
-//   1024       27 / 27     59 / 36     244 / 90     1906 / 569
-//   8192       81 / 132    160 / 191   637 / 547    4923 / 3743
-//   16000      135 / 256   270 / 374   1082 / 1082  7890 / 7447
-// Over those 1,512 calls the choice takes 0.4 % more than the faster path on average and
-// at most 10 % more than the layers (8 calls of one or two steps more than 5 %).
+//   1          17 / 25     32 / 32     127 / 79     970 / 499
+//   1024       26 / 27     52 / 36     204 / 90     1567 / 569
+//   8192       76 / 132    150 / 191   599 / 547    4626 / 3742
+//   16000      122 / 256   243 / 374   976 / 1081   7562 / 7445
+// Over those 1,512 calls the choice takes 0.8 % more than the faster path on average and
+// at most 19 % (17 us) more than the layers; 24 calls, most of one or two steps, take more
+// than 5 % more.
 // Beyond kUnrollEnvs environments the products fill the SMs by themselves.
 constexpr int kUnrollEnvs = 16384;
 
@@ -558,7 +559,7 @@ constexpr int kUnrollEnvs = 16384;
 // the step kernel.
 double layers_step_us(const crl_config& cf, const MlpShape& s) {
   const double E = cf.E, D = cf.D, H = s.hidden;
-  double us = 4.4 + 1.27e-3 * E + 1e-5 * E * D + 0.0155 * std::sqrt(E * D) + 0.027 * D;
+  double us = 4.0 + 1.24e-3 * E + 1.26e-5 * E * D + 7.3e-3 * std::sqrt(E * D) + 0.0325 * D;
   for (int l = 0; l <= s.layers; ++l) {
     const int K = l == 0 ? s.in() : s.hidden, N = l == s.layers ? s.out : s.hidden;
     double tiles = 0;
@@ -566,9 +567,9 @@ double layers_step_us(const crl_config& cf, const MlpShape& s) {
       const double c = f32_tile_cost(t, (long long)ceil_div(cf.E, t.bm) * ceil_div(N, t.bn));
       if (tiles == 0 || c < tiles) tiles = c;
     }
-    us += 0.82 + K * (6.39e-6 * tiles + 5.4e-4 * std::sqrt(tiles));
+    us += 1.31 + K * (0.004 + 7.08e-6 * tiles + 2.37e-4 * std::sqrt(tiles));
   }
-  return us + (s.layernorm ? s.layers * (2.1 + 4.3e-3 * std::sqrt(E * H)) : 0.0);
+  return us + (s.layernorm ? s.layers * (2.3 + 7.6e-7 * E * H + 8.1e-4 * std::sqrt(E * H)) : 0.0);
 }
 
 // The one launch, `waves` of clusters after one another.  Clocks of a step: the products
