@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(32 * kColRows) col_lse_kernel(int B, const T* 
         mb = fmax(mb, x[q]);
       }
       // (the maximum's own term is 1 whatever it is: no inf - inf)
-      T t = m == mb ? s : s * dev_exp(m - mb);
+      T t = m == mb || s == T(0) ? s : s * dev_exp(m - mb);
 #pragma unroll
       for (int q = 0; q < kColBatch; ++q)
         if (i + kColRows * q < B) t += x[q] == mb ? T(1) : dev_exp(x[q] - mb);
@@ -174,7 +174,14 @@ __global__ void __launch_bounds__(32 * kColRows) col_lse_kernel(int B, const T* 
   sm_m[ry][cx] = m;
   sm_s[ry][cx] = s;
   __syncthreads();
-  if (ry == 0 && j < B) {
+  if constexpr (sizeof(T) == 8) {
+    // one warp per column (in FP64, 32 exponentials one after another take several us)
+    const int col = blockIdx.x * 32 + ry;
+    const T pm = sm_m[cx][ry], ps = sm_s[cx][ry];
+    const T mm = warp_max(pm);
+    const T ss = warp_sum(ps > T(0) ? ps * dev_exp(pm - mm) : T(0));
+    if (cx == 0 && col < B) c[col] = mm + dev_log(ss);
+  } else if (ry == 0 && j < B) {
     T mm = sm_m[0][cx];
     for (int r = 1; r < kColRows; ++r) mm = fmax(mm, sm_m[r][cx]);
     T ss = 0;

@@ -171,9 +171,13 @@ __global__ void __launch_bounds__(256) layernorm_bwd_kernel(const __grid_constan
   }
 }
 
-// Column sums over M rows: out1[n] = sum X, out2[n] = sum X*Y (Y optional).  Block = 32 columns x 32 row groups (eight groups
-// left M / 8 dependent loads per thread: 9 us at M = 256 against 4 now).
-constexpr int kSumRows = 32;
+// Column sums over M rows: out1[n] = sum X, out2[n] = sum X*Y (Y optional).  Block =
+// 32 columns x 32 row groups (eight groups left M / 8 dependent loads per thread: 9 us
+// at M = 256 against 4 now); eight groups in FP64, whose additions are slow enough
+// that merging 32 costs more than the shorter chains save (a backward of 2 x 128 with
+// LayerNorm at 64 rows: 143 us with 32, 134 with 8; from 512 rows on within 1 %).
+template <typename T>
+constexpr int kSumRows = sizeof(T) == 8 ? 8 : 32;
 template <typename T>
 struct ColSum {
   int M, N;
@@ -185,7 +189,7 @@ struct ColSums {
   ColSum<T> a[2];
 };
 template <typename T>
-__global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(const __grid_constant__ ColSums<T> args) {
+__global__ void __launch_bounds__(32 * kSumRows<T>) colsum_kernel(const __grid_constant__ ColSums<T> args) {
   pdl_enter();
   const ColSum<T>& p = args.a[blockIdx.y];
   const int M = p.M, N = p.N;
@@ -193,13 +197,13 @@ __global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(const __grid_cons
   const T* __restrict__ Y = p.Y;
   T* __restrict__ out1 = p.out1;
   T* __restrict__ out2 = p.out2;
-  __shared__ T sm[2][kSumRows][33];
+  __shared__ T sm[2][kSumRows<T>][33];
   const int cx = threadIdx.x % 32, ry = threadIdx.x / 32;
   const int n = blockIdx.x * 32 + cx;
   T a1 = 0, a2 = 0;
   if (n < N) {
 #pragma unroll 4
-    for (int m = ry; m < M; m += kSumRows) {
+    for (int m = ry; m < M; m += kSumRows<T>) {
       const size_t o = (size_t)m * N + n;
       const T x = X[o];
       a1 += x;
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(32 * kSumRows) colsum_kernel(const __grid_cons
   if (ry == 0 && n < N) {
     T s1 = 0, s2 = 0;
 #pragma unroll 8
-    for (int r = 0; r < kSumRows; ++r) {
+    for (int r = 0; r < kSumRows<T>; ++r) {
       s1 += sm[0][r][cx];
       s2 += sm[1][r][cx];
     }
@@ -233,7 +237,7 @@ void colsum(const ColSum<T>* c, int n, cudaStream_t st) {
     N = std::max(N, c[i].N);
   }
   TraceLaunch tr(CRL_TRACE_AUX, st, bytes);
-  launch_k(colsum_kernel<T>, dim3(ceil_div(N, 32), n), dim3(32 * kSumRows), 0, st, a);
+  launch_k(colsum_kernel<T>, dim3(ceil_div(N, 32), n), dim3(32 * kSumRows<T>), 0, st, a);
 }
 
 }  // namespace
