@@ -184,10 +184,10 @@ inline void launch_k_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 // whichever SMs have room first, up to their occupancy, and its CTAs stay there: the
 // FP32 products and the -L1 gradients (32 to 256 CTAs of 128 or 256 threads with 8 to
 // 40 KB) ran on a fraction of the SMs after a short kernel.  us without / with: -L1
-// loss backward, 1001 x 200, FP32 412 / 268, FP64 512 x 64 2400 / 1320; cosine loss
-// backward 2048 x 64 226 / 123; encoder forward 31 -> 256 -> 256 -> 16, 4096 rows 64 / 49;
-// 507 encoder, loss and step calls in FP32: 0.93 of the time on average, none slower
-// by more than 3 % or 2 us.  Launches without overlap lose 2 us each (8 rows: 1.5 x).
+// loss backward, 1001 x 200, FP32 416 / 289, FP64 512 x 64 2394 / 1349; cosine loss
+// backward 2048 x 64 213 / 129; encoder forward 31 -> 256 -> 256 -> 16, 4096 rows 64 / 34;
+// 507 encoder, loss and step calls in FP32: 0.94 of the time on average, none slower
+// by more than 3 % and 2 us.  Launches without overlap lose 2 us each (8 rows: 1.5 x).
 // `allowed`: the kernel's own; devices on which it may ask for that much.
 template <typename... KArgs>
 inline size_t spread_smem(void (*kernel)(KArgs...), std::atomic<uint64_t>& allowed, size_t fixed, long long ctas) {
